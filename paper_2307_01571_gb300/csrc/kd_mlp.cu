@@ -1,9 +1,9 @@
 // kd_mlp.cu -- the surrogate network: a fully connected MLP with exact-erf GELU hidden
 // layers, trained on the batched solver's outputs (seeded parameter draws -> diffraction
-// and spin-flip populations).  Hand-written kernels: tiled GEMM with fused bias / GELU
-// epilogue (FP32 on the CUDA cores, or BF16 operands on the tcgen05 tensor cores with FP32
-// accumulation in tensor memory), the GELU derivative, fixed-order column sums, MSE loss
-// and Adam.  Every reduction runs in a fixed order, so training is bitwise reproducible.
+// and spin-flip populations).  Hand-written kernels: tiled products with fused gather, bias,
+// GELU, GELU derivative and loss epilogues (FP32 on the CUDA cores, or BF16 operands on the tcgen05 tensor cores with FP32
+// accumulation in tensor memory), fixed-order column sums, the loss
+// sum and Adam.  Every reduction runs in a fixed order, so training is bitwise reproducible.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -33,9 +33,9 @@ struct kd_mlp {
     std::vector<float*> a;           // activations per layer output [cap][w[l+1]] (a[0] = input)
     float* dbuf0 = nullptr;          // gradient ping-pong buffers [cap][max width]
     float* dbuf1 = nullptr;
-    float* lossbuf = nullptr;        // [cap * w[L]] squared errors, then partials
-    float* gx = nullptr;             // gathered minibatch inputs [cap][w[0]]
-    float* gt = nullptr;             // gathered minibatch targets [cap][w[L]]
+    float* lossbuf = nullptr;        // the loss, then [cap * w[L]] squared errors
+    float* part = nullptr;           // partial gradients of layers whose batch is split
+    size_t part_cap = 0;             // its floats
     int prec = 0;                    // KD_MLP_FP32 or KD_MLP_BF16 (tensor-core GEMMs)
     int* status = nullptr;           // set when a tensor-core GEMM's bounded wait gave up
 };
@@ -55,72 +55,280 @@ __device__ __forceinline__ float gelu_grad(float x) {
     return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
 }
 
-// C[m][n] = sum_k A(m, k) B(k, n) (+ bias[n]; GELU) with A(m, k) = A[m sam + k sak] and
-// B(k, n) = B[k sbk + n sbn].  64x64 tiles, 16-deep k slabs, 256 threads, 4x4 outputs
-// per thread; the k loop runs in order (deterministic).  epi: 0 store, 1 bias, 2 bias
-// then Z = C, Y = GELU(C).
-__global__ void __launch_bounds__(256) k_gemm(const float* A, long sam, long sak, const float* B,
-                                              long sbk, long sbn, float* C, float* Y, const float* bias,
-                                              int M, int N, int K, int epi) {
-    __shared__ float As[16][64 + 1];
-    __shared__ float Bs[16][64 + 1];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-    float acc[4][4] = {{0}};
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        for (int e = threadIdx.x; e < 16 * 64; e += 256) {
-            const int kk = e / 64, mm = e % 64;
-            const int gm = m0 + mm, gk = k0 + kk;
-            As[kk][mm] = (gm < M && gk < K) ? A[gm * sam + gk * sak] : 0.0f;
-            const int gn = n0 + mm;
-            Bs[kk][mm] = (gk < K && gn < N) ? B[gk * sbk + gn * sbn] : 0.0f;
+// ------------------------------------------------------------ grouped products ----
+// Every layer's products of one pass run in ONE launch: forward, one product; backward, the
+// gradient for the layer below, the weight gradient and the bias gradient (column sums) side
+// by side, since they only share their input dZ.  The network is small (a 256 x 256 x 256
+// product is 0.9 us of the FP32 pipe), so a step is bound by the number of launches in its
+// chain and by the load latency inside each one, not by arithmetic or memory: everything
+// pointwise (gather, bias, GELU and its derivative, the loss' gradient) sits in an epilogue
+// or a loader, and a launch starts under its predecessor's tail (programmatic dependent
+// launch).  Chain of a training step: L forward launches, L backward launches, Adam.
+//
+// A step at batch 256 / FP32 went from 22 launches and 396 us to 9 launches and 51 us, at batch
+// 1024 / BF16 from 401 to 73 us (GB300, the 5-256-256-256-4 network).  What bounds it now is
+// the chain: nine dependent launches of 4-8 us, most of it launch and load latency.
+
+// One operand P(row, k) of a product C[m][n] = sum_k A(m, k) B(n, k): element p[row ld + k]
+// (kc) or p[k ld + row].  idx (may be null) selects the source row of the dimension that is
+// not contiguous (row for kc, else k); an index outside [0, nidx) reads zeros.  vec: 16-byte
+// loads along the contiguous dimension are aligned.
+struct Operand {
+    const float* p;
+    long ld;
+    const int32_t* idx;
+    long nidx;
+    int kc, vec;
+};
+enum Epi { EPI_STORE, EPI_BIAS, EPI_BIAS_GELU, EPI_BIAS_MSE, EPI_GELU_BACK };
+// A product with its epilogue: STORE C = v; BIAS C = v + b; BIAS_GELU Z = v + b, C = GELU(Z);
+// BIAS_MSE C = v + b, dY = scale (C - T), sq = (C - T)^2; GELU_BACK C = v GELU'(Z).  The k
+// range runs in `splits` parts of kper, part s stored at C + s cstride.
+struct Product {
+    Operand A, B;
+    float* C;
+    long cstride;
+    const float* bias;
+    float* Z;
+    const float* T;          // targets [nt][N], rows tidx[m] when tidx is set
+    const int32_t* tidx;
+    long nt;
+    float* dY;
+    float* sq;
+    float scale;
+    int M, N, K, epi;
+    int mt, nt_tiles, splits, kper;
+};
+// Column sums out[s][n] = sum over part s of the rows of X [M][N] (32 columns per CTA)
+struct ColSum {
+    const float* X;
+    float* out;
+    long ostride;
+    int M, N, tiles, splits, mper;
+};
+// The mean of n squared errors into out[0] (and out2[0] when set), one CTA
+struct LossSum {
+    const float* sq;
+    long n;
+    float scale;
+    float* out;
+    float* out2;
+};
+struct Group {
+    Product prod[2];
+    ColSum col;
+    LossSum loss;
+    int first[5];            // first block of product 0, product 1, column sums, loss; total
+    int* status;
+};
+
+// The epilogue of NE elements (m + i mstep, n + i nstep) of a tile, values v(i).  One loop
+// per kind: a kernel of this size runs its code once, from a cold instruction cache, so the
+// kind is decided outside the loop and the loop stays short (unrolled over every kind the
+// BF16 epilogue took 14,000 cycles a tile).
+template <int NE, int UNROLL, typename F>
+__device__ __forceinline__ void epilogue(const Product& q, int m, int mstep, int n, int nstep, int split, F v) {
+    auto each = [&](auto f) {
+#pragma unroll UNROLL
+        for (int i = 0; i < NE; ++i) {
+            const int mi = m + i * mstep, ni = n + i * nstep;
+            if (mi < q.M && ni < q.N) f(mi, ni, (long)mi * q.N + ni, v(i));
         }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            float av[4], bv[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) av[i] = As[kk][ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) bv[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-        }
+    };
+    if (q.epi == EPI_STORE) {
+        float* C = q.C + (long)split * q.cstride;
+        each([&](int, int, long o, float x) { C[o] = x; });
+    } else if (q.epi == EPI_BIAS_GELU) {
+        each([&](int, int ni, long o, float x) {
+            x += __ldg(q.bias + ni);
+            q.Z[o] = x;
+            q.C[o] = gelu(x);
+        });
+    } else if (q.epi == EPI_GELU_BACK) {
+        each([&](int, int, long o, float x) { q.C[o] = x * gelu_grad(__ldg(q.Z + o)); });
+    } else if (q.epi == EPI_BIAS) {
+        each([&](int, int ni, long o, float x) { q.C[o] = x + __ldg(q.bias + ni); });
+    } else {
+        each([&](int mi, int ni, long o, float x) {
+            const long r = q.tidx ? q.tidx[mi] : mi;
+            const float t = !q.tidx || (r >= 0 && r < q.nt) ? __ldg(q.T + r * q.N + ni) : 0.0f;
+            x += __ldg(q.bias + ni);
+            q.C[o] = x;
+            const float d = x - t;
+            q.dY[o] = q.scale * d;
+            q.sq[o] = d * d;
+        });
+    }
+}
+
+// fixed-order sum of the squared errors (256 threads)
+__device__ void loss_block(const LossSum& l) {
+    __shared__ double red[256];
+    double s = 0.0;
+    for (long i = threadIdx.x; i < l.n; i += 256) s += (double)l.sq[i];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
         __syncthreads();
     }
+    if (threadIdx.x == 0) {
+        const float v = (float)(red[0] * l.scale);
+        l.out[0] = v;
+        if (l.out2) l.out2[0] = v;
+    }
+}
+
+// 32 columns of one part of the rows: eight row groups, each in order, then their sums in
+// order (256 threads; one thread per column took 60 us for 256 rows, this disappears beside
+// the products of its launch)
+__device__ void colsum_block(const ColSum& c, int blk) {
+    __shared__ float red[8][33];
+    const int n = (blk % c.tiles) * 32 + (threadIdx.x & 31), split = blk / c.tiles, g = threadIdx.x >> 5;
+    const int m1 = min(c.M, (split + 1) * c.mper);
+    float s = 0.0f;
+    if (n < c.N)
+        for (int m = split * c.mper + g; m < m1; m += 8) s += __ldg(c.X + (long)m * c.N + n);
+    red[g][threadIdx.x & 31] = s;
+    __syncthreads();
+    if (g == 0 && n < c.N) {
+        for (int i = 1; i < 8; ++i) s += red[i][threadIdx.x];
+        c.out[(long)split * c.ostride + n] = s;
+    }
+}
+
+// FP32 products on the CUDA cores: 32 x 32 tiles (64 CTAs for a 256 x 256 output, where
+// 64 x 64 tiles gave 16), 64-deep k slabs in a ring of four shared-memory stages filled by
+// cp.async (zero-filled outside the operand), so that a K = 256 product waits for the load
+// latency once.  A slab's k range is shared by four groups of 64 threads, each with 4 x 4
+// outputs a thread (16-byte shared loads, two per 16 FMAs), whose partial sums are added in
+// a fixed order at the end.  A slab keeps its operand's own contiguous dimension: [32 rows]
+// [64 k] with 68 floats a row, a thread taking rows ty + 8 i (conflict-free 16-byte reads
+// along k), or [64 k][32 rows] with 36 floats, a thread taking rows 4 ty + i.  64 x 64 tiles
+// with one k group and 16-deep slabs of scalar loads took 44 us for 256^3 under
+// ncu; this takes 6.6.
+namespace fp32 {
+constexpr int STAGES = 4, KS = 64, KP = KS + 4, RP = 36;
+constexpr int OP = KS * RP;                        // floats of one operand's slab
+constexpr int SMEM = STAGES * 2 * OP * 4;
+static_assert(OP >= 32 * KP && STAGES * 2 * OP >= 4 * 32 * RP, "slab and reduction fit");
+
+__device__ __forceinline__ void copy16(float* dst, const float* src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                 :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void copy4(float* dst, const float* src, int bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
+                 :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+// 32 rows x 64 k of an operand into a slab, zeros outside its R rows and [.., kend): 512
+// groups of four contiguous elements, two per thread
+template <bool KC> __device__ __forceinline__ void slab_load(float* sm, const Operand& o, int r0, int R, int k0, int kend) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int c = threadIdx.x + 256 * i;
+        const int row = KC ? c >> 4 : 4 * (c & 7), k = KC ? 4 * (c & 15) : c >> 3;
+        float* dst = sm + (KC ? row * KP + k : k * RP + row);
+        const int gr = r0 + row, gk = k0 + k, at = KC ? gk : gr;
+        long line = KC ? gr : gk;
+        int n = 4;   // elements inside
+        if (gr >= R || gk >= kend) n = 0;
+        else n = min(4, (KC ? kend : R) - at);
+        if (o.idx && n > 0) {
+            line = o.idx[line];
+            if (line < 0 || line >= o.nidx) n = 0;
+        }
+        const float* src = n > 0 ? o.p + line * o.ld + at : o.p;
+        if (o.vec) {
+            copy16(dst, src, 4 * n);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) copy4(dst + e, e < n ? src + e : o.p, e < n ? 4 : 0);
+        }
+    }
+}
+// a thread's four rows (columns) u of a slab at k .. k + 3: element [i][kk]
+template <bool KC> __device__ __forceinline__ void slab_read(const float* sm, int u, int k, float (&v)[4][4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float4 q = *reinterpret_cast<const float4*>(KC ? sm + (u + 8 * i) * KP + k : sm + (k + i) * RP + 4 * u);
+        if (KC) { v[i][0] = q.x; v[i][1] = q.y; v[i][2] = q.z; v[i][3] = q.w; }
+        else { v[0][i] = q.x; v[1][i] = q.y; v[2][i] = q.z; v[3][i] = q.w; }
+    }
+}
+
+template <bool AKC, bool BKC> __device__ __forceinline__ void product(const Product& q, int blk, float* sm) {
+    const int t = threadIdx.x;
+    const int n0 = (blk % q.nt_tiles) * 32, m0 = blk / q.nt_tiles % q.mt * 32, split = blk / (q.nt_tiles * q.mt);
+    const int kbeg = split * q.kper, kend = min(q.K, kbeg + q.kper);
+    const int nslab = (kend - kbeg + KS - 1) / KS;
+    const int g = t >> 6, ty = (t & 63) >> 3, tx = t & 7;
+    auto fill = [&](int j) {
+        if (j < nslab) {
+            float* st = sm + (j % STAGES) * 2 * OP;
+            slab_load<AKC>(st, q.A, m0, q.M, kbeg + KS * j, kend);
+            slab_load<BKC>(st + OP, q.B, n0, q.N, kbeg + KS * j, kend);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int j = 0; j < STAGES - 1; ++j) fill(j);
+    float acc[4][4] = {{0.0f}};
+    for (int j = 0; j < nslab; ++j) {
+        asm volatile("cp.async.wait_group %0;" :: "n"(STAGES - 2) : "memory");
+        __syncthreads();            // slab j has landed, slab j - 1's stage is free
+        fill(j + STAGES - 1);
+        const float* as = sm + (j % STAGES) * 2 * OP;
+        const float* bs = as + OP;
+#pragma unroll
+        for (int kk = 0; kk < 16; kk += 4) {
+            float av[4][4], bv[4][4];
+            slab_read<AKC>(as, ty, 16 * g + kk, av);
+            slab_read<BKC>(bs, tx, 16 * g + kk, bv);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) acc[i][h] = fmaf(av[i][e], bv[h][e], acc[i][h]);
+        }
+    }
+    // the four groups' partial sums, through shared memory, added in order
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int m = m0 + ty * 4 + i, n = n0 + tx * 4 + j;
-            if (m >= M || n >= N) continue;
-            float v = acc[i][j];
-            if (epi >= 1) v += bias[n];
-            C[(long)m * N + n] = v;
-            if (epi == 2) Y[(long)m * N + n] = gelu(v);
-        }
+        for (int h = 0; h < 4; ++h)
+            sm[(g * 32 + (AKC ? ty + 8 * i : 4 * ty + i)) * RP + (BKC ? tx + 8 * h : 4 * tx + h)] = acc[i][h];
+    __syncthreads();
+    const float* r = sm + (t >> 3) * RP + 4 * (t & 7);
+    epilogue<4, 4>(q, m0 + (t >> 3), 0, n0 + 4 * (t & 7), 1, split,
+                   [&](int j) { return (r[j] + r[32 * RP + j]) + (r[64 * RP + j] + r[96 * RP + j]); });
 }
+}  // namespace fp32
 
-// dZ = dY * GELU'(Z), elementwise
-// ------------------------------------------------------ BF16 tensor-core GEMM -----
-// The same product and epilogues as k_gemm with BF16 operands (rounded to nearest from
-// the FP32 inputs while staging) on the 5th-generation tensor cores, FP32 accumulation in
-// tensor memory.  One CTA of 128 threads computes a 128 x 32 tile of C (narrow tiles: the
-// network's products are small, so more CTAs share them): thread r owns row m0 + r, which
-// is TMEM lane r.  The k dimension runs in 64-deep slabs through two shared-memory stages
-// in the no-swizzle K-major canonical layout (8-row x 16-byte core matrices: LBO = 128 B
-// between core matrices along k, SBO = 1024 B between 8-row groups): while thread 0's four
-// tcgen05.mma.kind::f16 (M 128, N 32, K 16; A and B both BF16) of slab j run, committed to
-// the stage's mbarrier, the threads load slab j + 1 from global memory (16-byte loads where
-// the operand is contiguous in k and aligned), wait for slab j - 1's products (bounded) and
-// store into the stage those freed.  A wait that runs out sets *status, the CTA issues no
-// further products, waits (bounded) for those in flight and skips the epilogue; the host
-// reports KD_ERR_TIMEOUT.
+// BF16 products on the 5th-generation tensor cores: the operands are rounded to BF16 (to
+// nearest, from FP32) while staging, FP32 accumulation in tensor memory.  A CTA of 256
+// threads computes a 128 x 16 tile of C (narrow tiles: the network's products are small, so
+// more CTAs share them and each has half the epilogue of a 32-wide one).  The k range runs
+// in 128-deep slabs through two shared-memory stages in the no-swizzle K-major canonical
+// layout (8-row x 16-byte core matrices) with padded strides (LBO 144 bytes between core
+// matrices along k, SBO 2320 between 8-row groups), so that neither load pattern's stores
+// serialise on the banks.  While thread 0's tcgen05.mma.kind::f16 (M 128, N 16, K 16; A and
+// B both BF16) of slab j run, committed to the stage's mbarrier, the threads load slab
+// j + 1, wait for slab j - 1's products (bounded) and store into the stage those freed.
+// Four warps read the accumulator rows back (warp w owns TMEM lanes 32 w ...) and hand them
+// to all eight through shared memory for the epilogue.  A wait that runs out sets *status,
+// the CTA issues no further products, waits (bounded) for those in flight and skips the
+// epilogue; the host reports KD_ERR_TIMEOUT.  What bounds it is the latency of the slabs'
+// loads (about 2,300 cycles each) and a cold instruction cache, not the matrix units (550
+// cycles of waiting per tile), hence the short code paths.  Under ncu 1024 x 256 x 256 takes
+// 8.8 us where 64-deep slabs loaded row by row by 128 threads took 15, and the weight
+// gradient at batch 1024, split over eight parts of the batch, 11.4 us together with the
+// gradient below, where 16 CTAs of 16 serial slabs took 43.
 namespace tcg {
-constexpr int BN = 32;                                   // columns of C per CTA
-constexpr uint32_t LBO = 128, SBO = 1024;
+constexpr int BN = 16, KS = 128;                         // columns of C per CTA, slab depth
+constexpr uint32_t LBO = 144, SBO = (KS / 8) * LBO + 16;
 constexpr uint32_t A_BYTES = 16 * SBO, B_BYTES = (BN / 8) * SBO, STAGE = A_BYTES + B_BYTES;
 constexpr uint32_t OFF_BAR = 2 * STAGE, OFF_SLOT = OFF_BAR + 16;
 constexpr uint32_t SMEM = OFF_SLOT + 16;
@@ -130,11 +338,12 @@ constexpr uint32_t TMEM_COLS = 32;
 constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                            ((uint32_t)(128 >> 4) << 24);
 constexpr long long WAIT_LIMIT = 1ll << 20;
+static_assert(STAGE % 16 == 0 && SBO % 16 == 0 && LBO % 16 == 0, "descriptor granularity");
 
 __device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((saddr & 0x3FFFF) >> 4) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);
+__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
+    return (uint64_t)((saddr & 0x3FFFF) >> 4) | ((uint64_t)((LBO >> 4) & 0x3FFF) << 16) |
+           ((uint64_t)((SBO >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);
 }
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     const uint32_t a = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(lo));
@@ -150,66 +359,83 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     }
     return false;
 }
-// eight consecutive k of one operand row (element (row, k) at p[row * sr + k * sk]), zero
-// outside [0, K) or for rows out of range
-__device__ __forceinline__ void load8(const float* p, long sr, long sk, int row, bool row_ok, int k, int K,
-                                      float* v) {
-    const float* q = p + (long)row * sr + (long)k * sk;
-    if (row_ok && sk == 1 && k + 8 <= K && ((reinterpret_cast<uintptr_t>(q) & 15) == 0)) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(q));
-        const float4 b = __ldg(reinterpret_cast<const float4*>(q) + 1);
-        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+// ROWS rows x KS k of an operand, ROWS / 8 16-byte loads per thread (256 threads).  kc: a warp
+// takes whole rows (512 contiguous bytes); !kc: a thread takes blocks of 4 rows x KB k (a warp
+// 512 bytes of a k line, or 64 for 16 rows) and transposes them in registers.
+__device__ __forceinline__ unsigned char* cell(unsigned char* dst, int row, int k) {
+    return dst + (uint32_t)(row >> 3) * SBO + (uint32_t)(k >> 3) * LBO + (uint32_t)(row & 7) * 16 + (uint32_t)(k & 7) * 2;
+}
+// 16-deep products of the slab at k0
+__device__ __forceinline__ int steps_of(int k0, int kend) { return min(KS, kend - k0 + 15) / 16; }
+template <int ROWS> struct Tile {
+    float4 v[ROWS / 8];
+    bool whole;      // v holds the tile; else it is read element by element at the store
+};
+template <int ROWS, bool KC> __device__ __forceinline__ void tile_load(const Operand& o, int r0, int R, int k0, int kend, Tile<ROWS>& s) {
+    const int t = threadIdx.x;
+    s.whole = o.vec && !o.idx && r0 + ROWS <= R && k0 + KS <= kend;
+    if (!s.whole) return;
+    constexpr int KB = ROWS == 128 ? 8 : 2;
+    const float* p = o.p + (KC ? (long)(r0 + (t >> 5)) * o.ld + k0 + 4 * (t & 31)
+                               : (long)(k0 + KB * (t / (ROWS / 4))) * o.ld + r0 + 4 * (t % (ROWS / 4)));
+#pragma unroll
+    for (int i = 0; i < ROWS / 8; ++i) {
+        const long line = KC ? 8 * i : 64 * (i / KB) + i % KB;
+        s.v[i] = __ldg(reinterpret_cast<const float4*>(p + line * o.ld));
+    }
+}
+__device__ __forceinline__ float elem(const float4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
+template <int ROWS, bool KC>
+__device__ __forceinline__ void tile_store(unsigned char* dst, const Operand& o, int r0, int R, int k0, int kend, const Tile<ROWS>& s) {
+    const int t = threadIdx.x;
+    if (!s.whole) {
+        // edges, gathered rows, odd strides: element by element, zeros outside, up to the
+        // last 16-deep step that holds any k
+#pragma unroll 1
+        for (int c = t; c < ROWS * 2 * steps_of(k0, kend); c += 256) {
+            const int row = r0 + c % ROWS, k = k0 + 8 * (c / ROWS);
+            float v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                bool in = row < R && k + e < kend;
+                long line = KC ? row : k + e;
+                if (in && o.idx) {
+                    line = o.idx[line];
+                    in = line >= 0 && line < o.nidx;
+                }
+                v[e] = in ? __ldg(o.p + line * o.ld + (KC ? k + e : row)) : 0.0f;
+            }
+            *reinterpret_cast<uint4*>(cell(dst, row - r0, k - k0)) =
+                make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+        }
+    } else if constexpr (KC) {
+#pragma unroll
+        for (int i = 0; i < ROWS / 8; ++i)
+            *reinterpret_cast<uint2*>(cell(dst, (t >> 5) + 8 * i, 4 * (t & 31))) =
+                make_uint2(pack_bf16(s.v[i].x, s.v[i].y), pack_bf16(s.v[i].z, s.v[i].w));
+    } else if constexpr (ROWS == 128) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                *reinterpret_cast<uint4*>(cell(dst, 4 * (t & 31) + e, 8 * (t >> 5) + 64 * i)) =
+                    make_uint4(pack_bf16(elem(s.v[8 * i + 0], e), elem(s.v[8 * i + 1], e)),
+                               pack_bf16(elem(s.v[8 * i + 2], e), elem(s.v[8 * i + 3], e)),
+                               pack_bf16(elem(s.v[8 * i + 4], e), elem(s.v[8 * i + 5], e)),
+                               pack_bf16(elem(s.v[8 * i + 6], e), elem(s.v[8 * i + 7], e)));
     } else {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = (row_ok && k + e < K) ? __ldg(q + (long)e * sk) : 0.0f;
+        for (int e = 0; e < 4; ++e)
+            *reinterpret_cast<uint32_t*>(cell(dst, 4 * (t & 3) + e, 2 * (t >> 2))) = pack_bf16(elem(s.v[0], e), elem(s.v[1], e));
     }
 }
 }  // namespace tcg
 
-// one 64-deep slab of A (128 rows: 8 chunks of 8 k per thread) and B (32 rows n: thread t
-// holds row t & 31, chunks 2 (t >> 5) and 2 (t >> 5) + 1) in registers
-struct Slab {
-    float a[8][8];
-    float b[2][8];
-};
-
-__device__ __forceinline__ void slab_load(const float* A, long sam, long sak, const float* B, long sbk, long sbn,
-                                          int m, int M, int n0, int N, int K, int k0, Slab& s) {
-    const int t = threadIdx.x;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) tcg::load8(A, sam, sak, m, m < M, k0 + 8 * c, K, s.a[c]);
-    const int nn = t & 31, n = n0 + nn;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) tcg::load8(B, sbn, sbk, n, n < N, k0 + 8 * (2 * (t >> 5) + h), K, s.b[h]);
-}
-
-__device__ __forceinline__ void slab_store(unsigned char* stage, const Slab& s) {
-    const int t = threadIdx.x;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        const uint32_t o = (uint32_t)(t >> 3) * tcg::SBO + (uint32_t)c * tcg::LBO + (uint32_t)(t & 7) * 16;
-        *reinterpret_cast<uint4*>(stage + o) =
-            make_uint4(tcg::pack_bf16(s.a[c][0], s.a[c][1]), tcg::pack_bf16(s.a[c][2], s.a[c][3]),
-                       tcg::pack_bf16(s.a[c][4], s.a[c][5]), tcg::pack_bf16(s.a[c][6], s.a[c][7]));
-    }
-    const int nn = t & 31;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int c = 2 * (t >> 5) + h;
-        const uint32_t o = (uint32_t)(nn >> 3) * tcg::SBO + (uint32_t)c * tcg::LBO + (uint32_t)(nn & 7) * 16;
-        *reinterpret_cast<uint4*>(stage + tcg::A_BYTES + o) =
-            make_uint4(tcg::pack_bf16(s.b[h][0], s.b[h][1]), tcg::pack_bf16(s.b[h][2], s.b[h][3]),
-                       tcg::pack_bf16(s.b[h][4], s.b[h][5]), tcg::pack_bf16(s.b[h][6], s.b[h][7]));
-    }
-}
-
-__global__ void __launch_bounds__(128) k_gemm_bf16(const float* A, long sam, long sak, const float* B,
-                                                   long sbk, long sbn, float* C, float* Y, const float* bias,
-                                                   int M, int N, int K, int epi, int* status) {
-    extern __shared__ __align__(1024) unsigned char sm[];
+template <bool AKC, bool BKC>
+__device__ __forceinline__ void product_bf16(const Product& q, int blk, int* status, unsigned char* sm) {
     const int t = threadIdx.x, w = t >> 5;
-    const int m0 = blockIdx.y * 128, n0 = blockIdx.x * tcg::BN;
+    const int n0 = (blk % q.nt_tiles) * tcg::BN, m0 = blk / q.nt_tiles % q.mt * 128, split = blk / (q.nt_tiles * q.mt);
+    const int kbeg = split * q.kper, kend = min(q.K, kbeg + q.kper);
     const uint32_t s0 = tcg::su32(sm);
     const uint32_t bar[2] = {s0 + tcg::OFF_BAR, s0 + tcg::OFF_BAR + 8};
     if (w == 0) {
@@ -222,33 +448,33 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(const float* A, long sam, lon
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bar[1]));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *reinterpret_cast<const uint32_t*>(sm + tcg::OFF_SLOT);
-    const int m = m0 + t;
-    const int nslab = (K + 63) / 64;
+    const int nslab = (kend - kbeg + tcg::KS - 1) / tcg::KS;
     uint32_t phase[2] = {0u, 0u};
     bool ok = true;
     int issued = 0;          // slabs whose products were issued (and committed)
     int waited = 0;          // slabs whose products were waited for
-    Slab sl;
+    tcg::Tile<128> ta;
+    tcg::Tile<tcg::BN> tb;
     if (nslab > 0) {
-        slab_load(A, sam, sak, B, sbk, sbn, m, M, n0, N, K, 0, sl);
-        slab_store(sm, sl);
+        tcg::tile_load<128, AKC>(q.A, m0, q.M, kbeg, kend, ta);
+        tcg::tile_load<tcg::BN, BKC>(q.B, n0, q.N, kbeg, kend, tb);
+        tcg::tile_store<128, AKC>(sm, q.A, m0, q.M, kbeg, kend, ta);
+        tcg::tile_store<tcg::BN, BKC>(sm + tcg::A_BYTES, q.B, n0, q.N, kbeg, kend, tb);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *reinterpret_cast<const uint32_t*>(sm + tcg::OFF_SLOT);
     for (int j = 0; j < nslab && ok; ++j) {
         const int b = j & 1;
         if (t == 0) {
             const uint32_t sa = s0 + (uint32_t)b * tcg::STAGE;
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-                const uint64_t da = tcg::sdesc(sa + (uint32_t)ks * 2 * tcg::LBO, tcg::LBO, tcg::SBO);
-                const uint64_t db = tcg::sdesc(sa + tcg::A_BYTES + (uint32_t)ks * 2 * tcg::LBO, tcg::LBO, tcg::SBO);
+            for (int ks = 0; ks < tcg::KS / 16; ++ks) {
+                if (ks >= tcg::steps_of(kbeg + tcg::KS * j, kend)) break;
+                const uint64_t da = tcg::sdesc(sa + (uint32_t)ks * 2 * tcg::LBO);
+                const uint64_t db = tcg::sdesc(sa + tcg::A_BYTES + (uint32_t)ks * 2 * tcg::LBO);
                 const uint32_t acc = (j > 0 || ks > 0) ? 1u : 0u;
                 asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
@@ -259,7 +485,10 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(const float* A, long sam, lon
         }
         issued = j + 1;
         // the next slab's global loads run while these products do
-        if (j + 1 < nslab) slab_load(A, sam, sak, B, sbk, sbn, m, M, n0, N, K, 64 * (j + 1), sl);
+        if (j + 1 < nslab) {
+            tcg::tile_load<128, AKC>(q.A, m0, q.M, kbeg + tcg::KS * (j + 1), kend, ta);
+            tcg::tile_load<tcg::BN, BKC>(q.B, n0, q.N, kbeg + tcg::KS * (j + 1), kend, tb);
+        }
         bool got = true;
         if (j >= 1) {   // slab j - 1's products read the stage slab j + 1 goes to
             got = tcg::mbar_wait(bar[b ^ 1], phase[b ^ 1]);
@@ -269,7 +498,9 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(const float* A, long sam, lon
             }
         }
         if (got && j + 1 < nslab) {
-            slab_store(sm + (uint32_t)(b ^ 1) * tcg::STAGE, sl);
+            unsigned char* st = sm + (uint32_t)(b ^ 1) * tcg::STAGE;
+            tcg::tile_store<128, AKC>(st, q.A, m0, q.M, kbeg + tcg::KS * (j + 1), kend, ta);
+            tcg::tile_store<tcg::BN, BKC>(st + tcg::A_BYTES, q.B, n0, q.N, kbeg + tcg::KS * (j + 1), kend, tb);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -289,92 +520,98 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(const float* A, long sam, lon
     }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     ok = __syncthreads_and(ok) != 0;
-    if (ok && nslab > 0) {
-        // row m's 32 columns from TMEM lane t: two 16-column loads
-        const uint32_t trow = tmem + ((uint32_t)((w & 3) * 32) << 16);
-        uint32_t r[32];
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                         "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                         : "=r"(r[16 * j + 0]), "=r"(r[16 * j + 1]), "=r"(r[16 * j + 2]), "=r"(r[16 * j + 3]),
-                           "=r"(r[16 * j + 4]), "=r"(r[16 * j + 5]), "=r"(r[16 * j + 6]), "=r"(r[16 * j + 7]),
-                           "=r"(r[16 * j + 8]), "=r"(r[16 * j + 9]), "=r"(r[16 * j + 10]), "=r"(r[16 * j + 11]),
-                           "=r"(r[16 * j + 12]), "=r"(r[16 * j + 13]), "=r"(r[16 * j + 14]), "=r"(r[16 * j + 15])
-                         : "r"(trow + 16 * j));
+    if (ok && nslab > 0 && w < 4) {
+        // row m0 + t's 16 columns from TMEM lane t
+        const uint32_t trow = tmem + ((uint32_t)(w * 32) << 16);
+        uint32_t r[16];
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+                     "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+                       "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+                       "=r"(r[14]), "=r"(r[15])
+                     : "r"(trow));
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (m < M) {
+        // transposed through shared memory (the stages' products are done), so that the
+        // epilogue's global accesses run along the rows
+        float* tr = reinterpret_cast<float*>(sm);
 #pragma unroll
-            for (int j = 0; j < tcg::BN; ++j) {
-                const int n = n0 + j;
-                if (n >= N) break;
-                float c = __uint_as_float(r[j]);
-                if (epi >= 1) c += bias[n];
-                C[(long)m * N + n] = c;
-                if (epi == 2) Y[(long)m * N + n] = gelu(c);
-            }
-        }
+        for (int j = 0; j < tcg::BN; ++j) tr[t * 17 + j] = __uint_as_float(r[j]);
     }
-    if (!ok && t == 0) atomicOr(status, 1);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (ok && nslab > 0) {
+        const float* tr = reinterpret_cast<const float*>(sm) + (t >> 4) * 17 + (t & 15);
+        epilogue<8, 2>(q, m0 + (t >> 4), 16, n0 + (t & 15), 0, split, [&](int i) { return tr[16 * i * 17]; });
+    }
+    if (!ok && t == 0) atomicOr(status, 1);
     if (w == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(tcg::TMEM_COLS));
 }
 
-__global__ void k_gelu_back(const float* dY, const float* Z, float* dZ, long n) {
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-        dZ[i] = dY[i] * gelu_grad(Z[i]);
-}
-
-// db[n] = sum_m dZ[m][n], rows in order (one thread per column)
-__global__ void k_colsum(const float* dZ, int M, int N, float* db) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    float s = 0.0f;
-    for (int m = 0; m < M; ++m) s += dZ[(long)m * N + n];
-    db[n] = s;
-}
-
-// MSE over B x D outputs: dY = 2 (Y - T) / (B D), sq[i] = (Y - T)^2
-__global__ void k_mse(const float* Y, const float* T, float* dY, float* sq, long n, float scale) {
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const float d = Y[i] - T[i];
-        dY[i] = scale * d;
-        sq[i] = d * d;
+// One launch of a pass: the block index selects the product (and its tile and part), the
+// column sums or the loss.
+template <int BF16> __global__ void __launch_bounds__(256) k_group(const __grid_constant__ Group g) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    const int blk = blockIdx.x;
+    if (blk >= g.first[3]) {
+        loss_block(g.loss);
+    } else if (blk >= g.first[2]) {
+        colsum_block(g.col, blk - g.first[2]);
+    } else {
+        // the orientations that occur: forward (rows x rows), the gradient below (rows x
+        // columns), the weight gradient (columns x columns)
+        // by value: read once into registers (a reference into the parameter block is read
+        // again after every store, 7 us per tile)
+        Product q = g.prod[0];
+        int b = blk;
+        if (blk >= g.first[1]) {
+            q = g.prod[1];
+            b -= g.first[1];
+        }
+        extern __shared__ __align__(1024) unsigned char sm[];
+        if constexpr (BF16) {
+            if (!q.A.kc) product_bf16<false, false>(q, b, g.status, sm);
+            else if (q.B.kc) product_bf16<true, true>(q, b, g.status, sm);
+            else product_bf16<true, false>(q, b, g.status, sm);
+        } else {
+            float* f = reinterpret_cast<float*>(sm);
+            if (!q.A.kc) fp32::product<false, false>(q, b, f);
+            else if (q.B.kc) fp32::product<true, true>(q, b, f);
+            else fp32::product<true, false>(q, b, f);
+        }
     }
 }
 
-// fixed-order sum of n floats times scale into out[0] (one block)
-__global__ void k_sum(const float* x, long n, float scale, float* out) {
-    __shared__ double red[256];
-    double s = 0.0;
-    for (long i = threadIdx.x; i < n; i += blockDim.x) s += (double)x[i];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[0] = (float)(red[0] * scale);
+// Where the gradient of each layer lies: `parts` partial sums (over parts of the batch) at
+// src + s stride, each [W_l | b_l]; off[l] is the layer's first parameter, off[L] the count.
+struct GradParts {
+    int L;
+    long off[17];
+    const float* src[16];
+    long stride[16];
+    int parts[16];
+};
+__device__ __forceinline__ float grad_of(const GradParts& q, long i) {
+    int l = 0;
+    while (l + 1 < q.L && i >= q.off[l + 1]) ++l;
+    const float* p = q.src[l] + (i - q.off[l]);
+    float g = p[0];
+    for (int s = 1; s < q.parts[l]; ++s) g += p[s * q.stride[l]];
+    return g;
+}
+__global__ void k_sum_parts(const __grid_constant__ GradParts q, float* out) {
+    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < q.off[q.L]; i += (long)gridDim.x * blockDim.x)
+        out[i] = grad_of(q, i);
 }
 
-// dst[i][:] = src[idx[i]][:] for i < n (rows of `width` floats); an index outside
-// [0, nsrc) gives a row of zeros
-__global__ void k_gather_rows(const float* src, int width, long nsrc, const int32_t* idx, int n, float* dst) {
-    const long total = (long)n * width;
-    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x) {
-        const int i = (int)(e / width), j = (int)(e % width);
-        const long r = idx[i];
-        dst[e] = (r >= 0 && r < nsrc) ? src[r * width + j] : 0.0f;
-    }
-}
-
-__global__ void k_adam(float* p, const float* g, float* m1, float* m2, long n, float lr, float b1,
+__global__ void k_adam(float* p, const __grid_constant__ GradParts q, float* m1, float* m2, float lr, float b1,
                        float b2, float eps, float c1, float c2) {
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const float gi = g[i];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < q.off[q.L]; i += (long)gridDim.x * blockDim.x) {
+        const float gi = grad_of(q, i);
         const float a = b1 * m1[i] + (1.0f - b1) * gi;
         const float b = b2 * m2[i] + (1.0f - b2) * gi * gi;
         m1[i] = a;
@@ -383,25 +620,59 @@ __global__ void k_adam(float* p, const float* g, float* m1, float* m2, long n, f
     }
 }
 
-cudaError_t gemm(const kd_mlp* net, const float* A, long sam, long sak, const float* B, long sbk, long sbn,
-                 float* C, float* Y, const float* bias, int M, int N, int K, int epi, cudaStream_t s) {
-    if (net->prec == KD_MLP_BF16) {
-        // two 20 KB stages: at most 5 CTAs per SM, whose tensor memory (32 columns each)
-        // fits the SM's 512 columns, so no allocation waits
-        static bool attr = false;
-        constexpr int smem = (int)tcg::SMEM;
-        if (!attr) {
-            cudaError_t e = cudaFuncSetAttribute(k_gemm_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            if (e != cudaSuccess) return e;
-            attr = true;
-        }
-        dim3 grid((N + tcg::BN - 1) / tcg::BN, (M + 127) / 128);
-        k_gemm_bf16<<<grid, 128, smem, s>>>(A, sam, sak, B, sbk, sbn, C, Y, bias, M, N, K, epi, net->status);
-        return cudaGetLastError();
+// ---------------------------------------------------------------- host side -------
+Operand operand(const float* p, long ld, bool kc, const int32_t* idx = nullptr, long nidx = 0) {
+    const bool vec = ld % 4 == 0 && (reinterpret_cast<uintptr_t>(p) & 15) == 0;
+    return Operand{p, ld, idx, nidx, kc ? 1 : 0, vec ? 1 : 0};
+}
+
+// tiles of the product at the network's precision, its k range in `splits` parts
+void tile(const kd_mlp* n, Product* q, int splits) {
+    const int bm = n->prec == KD_MLP_BF16 ? 128 : 32, bn = n->prec == KD_MLP_BF16 ? tcg::BN : 32;
+    q->mt = (q->M + bm - 1) / bm;
+    q->nt_tiles = (q->N + bn - 1) / bn;
+    q->splits = splits;
+    q->kper = (q->K + splits - 1) / splits;
+}
+long blocks(const Product& q) { return (long)q.mt * q.nt_tiles * q.splits; }
+
+template <typename... KP, typename... KA>
+cudaError_t launch_pdl(void (*k)(KP...), long grid, int threads, int smem, cudaStream_t s, KA... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
+cudaError_t launch_group(const kd_mlp* n, Group& g, int nprod, cudaStream_t s) {
+    long b = 0;
+    for (int i = 0; i < 2; ++i) {
+        g.first[i] = (int)b;
+        if (i < nprod) b += blocks(g.prod[i]);
     }
-    dim3 grid((N + 63) / 64, (M + 63) / 64);
-    k_gemm<<<grid, 256, 0, s>>>(A, sam, sak, B, sbk, sbn, C, Y, bias, M, N, K, epi);
-    return cudaGetLastError();
+    g.first[2] = (int)b;
+    b += (long)g.col.tiles * g.col.splits;
+    g.first[3] = (int)b;
+    b += g.loss.n > 0 ? 1 : 0;
+    g.first[4] = (int)b;
+    if (b > 0x7fffffffL) return cudaErrorInvalidValue;
+    g.status = n->status;
+    const bool bf = n->prec == KD_MLP_BF16;
+    // BF16: two 41 KB stages and 32 columns of tensor memory per CTA: two CTAs per SM, whose
+    // columns fit the SM's 512, so no allocation waits
+    const int smem = bf ? (int)tcg::SMEM : fp32::SMEM;
+    static const cudaError_t attr[2] = {
+        cudaFuncSetAttribute(k_group<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, fp32::SMEM),
+        cudaFuncSetAttribute(k_group<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tcg::SMEM)};
+    if (attr[bf] != cudaSuccess) return attr[bf];
+    return bf ? launch_pdl(k_group<1>, b, 256, smem, s, g) : launch_pdl(k_group<0>, b, 256, smem, s, g);
 }
 
 // KD_ERR_TIMEOUT (and the flag cleared) when a tensor-core GEMM's bounded wait gave up
@@ -427,9 +698,6 @@ int ensure_cap(kd_mlp* n, int batch) {
     cudaFree(n->dbuf0);
     cudaFree(n->dbuf1);
     cudaFree(n->lossbuf);
-    cudaFree(n->gx);
-    cudaFree(n->gt);
-    n->gx = n->gt = nullptr;   // gathered-batch buffers, re-made at the new capacity
     n->z.assign(n->L, nullptr);
     n->a.assign(n->L + 1, nullptr);
     for (int l = 0; l < n->L; ++l) {
@@ -443,48 +711,126 @@ int ensure_cap(kd_mlp* n, int batch) {
     return KD_OK;
 }
 
-// forward pass from device input x (batch rows): a[l+1] = act(a[l] W_l^T + b_l); the
-// last layer is linear (its output is a[L])
-int forward(kd_mlp* n, const float* x, int batch, cudaStream_t s) {
-    n->a[0] = const_cast<float*>(x);
+// A minibatch on the device: rows of x and t (targets, may be null), or rows idx[.] of nsrc
+struct Batch {
+    const float* x;
+    const float* t;
+    const int32_t* idx;
+    long nsrc;
+    int rows;
+};
+
+// forward pass: a[l+1] = act(a[l] W_l^T + b_l); the last layer is linear (its output is
+// a[L]) and, with targets, also writes the loss' gradient to dbuf0 and the squared errors
+int forward(kd_mlp* n, const Batch& in, cudaStream_t s) {
+    const long nout = (long)in.rows * n->w[n->L];
     for (int l = 0; l < n->L; ++l) {
         const int fi = n->w[l], fo = n->w[l + 1];
         const bool last = l == n->L - 1;
-        float* out = last ? n->a[l + 1] : n->z[l];
-        MLP_CUDA(gemm(n, n->a[l], fi, 1, n->param + n->woff[l], 1, fi, out, last ? nullptr : n->a[l + 1],
-                      n->param + n->boff[l], batch, fo, fi, last ? 1 : 2, s));
+        Group g{};
+        Product& q = g.prod[0];
+        q.A = l == 0 ? operand(in.x, fi, true, in.idx, in.nsrc) : operand(n->a[l], fi, true);
+        q.B = operand(n->param + n->woff[l], fi, true);
+        q.C = n->a[l + 1];
+        q.bias = n->param + n->boff[l];
+        q.Z = last ? nullptr : n->z[l];
+        q.M = in.rows;
+        q.N = fo;
+        q.K = fi;
+        q.epi = !last ? EPI_BIAS_GELU : in.t ? EPI_BIAS_MSE : EPI_BIAS;
+        if (last && in.t) {
+            q.T = in.t;
+            q.tidx = in.idx;
+            q.nt = in.nsrc;
+            q.dY = n->dbuf0;
+            q.sq = n->lossbuf + 1;
+            q.scale = 2.0f / (float)nout;
+        }
+        tile(n, &q, 1);
+        MLP_CUDA(launch_group(n, g, 1, s));
     }
     return KD_OK;
 }
 
-// loss and gradients for targets t (device): returns via lossbuf[0] the mean squared error
-int backward(kd_mlp* n, const float* t, int batch, cudaStream_t s) {
-    const int D = n->w[n->L];
-    const long nout = (long)batch * D;
-    float* sq = n->lossbuf + 1;
-    k_mse<<<(int)((nout + 255) / 256), 256, 0, s>>>(n->a[n->L], t, n->dbuf0, sq, nout, 2.0f / (float)nout);
-    MLP_CUDA(cudaGetLastError());
-    k_sum<<<1, 256, 0, s>>>(sq, nout, 1.0f / (float)nout, n->lossbuf);   // mean squared error
-    MLP_CUDA(cudaGetLastError());
-    float* dcur = n->dbuf0;   // gradient w.r.t. the output of layer l (pre-activation for the last)
+// Parts of the batch the weight gradient of an fo x fi layer is summed in: enough for about
+// two CTAs on every SM when its tiles alone leave most of them idle, at least 128 (BF16: one
+// slab) or 256 rows each, at most eight.
+int grad_parts(const kd_mlp* n, int fo, int fi, int rows) {
+    const bool bf = n->prec == KD_MLP_BF16;
+    const int bm = bf ? 128 : 32, least = bf ? 128 : 256;
+    const int bn = bf ? tcg::BN : 32;
+    const long tiles = (long)((fo + bm - 1) / bm) * ((fi + bn - 1) / bn);
+    const long fill = (304 + tiles - 1) / tiles, depth = rows / least;
+    const long p = fill < depth ? fill : depth;
+    return (int)(p < 1 ? 1 : p > 8 ? 8 : p);
+}
+
+// Gradients after forward() with targets: layer l's partial sums where `gp` says, the mean
+// squared error in lossbuf[0] (and *loss2).
+int backward(kd_mlp* n, const Batch& in, GradParts* gp, float* loss2, cudaStream_t s) {
+    const int L = n->L;
+    size_t need = 0;
+    gp->L = L;
+    for (int l = 0; l < L; ++l) {
+        const size_t cnt = (size_t)n->w[l + 1] * n->w[l] + n->w[l + 1];
+        gp->off[l] = (long)n->woff[l];
+        gp->parts[l] = grad_parts(n, n->w[l + 1], n->w[l], in.rows);
+        gp->stride[l] = (long)cnt;
+        if (gp->parts[l] > 1) need += cnt * gp->parts[l];
+    }
+    gp->off[L] = (long)n->nparam;
+    if (need > n->part_cap) {
+        cudaFree(n->part);
+        n->part = nullptr;
+        n->part_cap = 0;
+        MLP_CUDA(cudaMalloc(&n->part, need * sizeof(float)));
+        n->part_cap = need;
+    }
+    float* at = n->part;
+    float* dcur = n->dbuf0;   // dZ_l
     float* dnext = n->dbuf1;
-    for (int l = n->L - 1; l >= 0; --l) {
-        const int fi = n->w[l], fo = n->w[l + 1];
-        if (l != n->L - 1) {   // through the GELU: dZ = dA * GELU'(Z)
-            const long cnt = (long)batch * fo;
-            k_gelu_back<<<(int)((cnt + 255) / 256), 256, 0, s>>>(dcur, n->z[l], dcur, cnt);
-            MLP_CUDA(cudaGetLastError());
+    for (int l = L - 1; l >= 0; --l) {
+        const int fi = n->w[l], fo = n->w[l + 1], parts = gp->parts[l];
+        float* dst = n->grad + n->woff[l];
+        if (parts > 1) {
+            dst = at;
+            at += gp->stride[l] * parts;
+        }
+        gp->src[l] = dst;
+        Group g{};
+        int np = 0;
+        if (l > 0) {  // dZ_{l-1}[b][i] = (sum_o dZ[b][o] W_l[o][i]) GELU'(Z_{l-1}[b][i])
+            Product& q = g.prod[np++];
+            q.A = operand(dcur, fo, true);
+            q.B = operand(n->param + n->woff[l], fi, false);
+            q.C = dnext;
+            q.Z = n->z[l - 1];
+            q.M = in.rows;
+            q.N = fi;
+            q.K = fo;
+            q.epi = EPI_GELU_BACK;
+            tile(n, &q, 1);
         }
         // dW_l[o][i] = sum_b dZ[b][o] a_l[b][i];  db_l[o] = sum_b dZ[b][o]
-        MLP_CUDA(gemm(n, dcur, 1, fo, n->a[l], fi, 1, n->grad + n->woff[l], nullptr, nullptr, fo, fi, batch, 0, s));
-        k_colsum<<<(fo + 127) / 128, 128, 0, s>>>(dcur, batch, fo, n->grad + n->boff[l]);
-        MLP_CUDA(cudaGetLastError());
-        if (l > 0) {  // dA_{l}[b][i] = sum_o dZ[b][o] W_l[o][i]
-            MLP_CUDA(gemm(n, dcur, fo, 1, n->param + n->woff[l], fi, 1, dnext, nullptr, nullptr, batch, fi, fo, 0, s));
-            float* tmp = dcur;
-            dcur = dnext;
-            dnext = tmp;
+        Product& q = g.prod[np++];
+        q.A = operand(dcur, fo, false);
+        q.B = l == 0 ? operand(in.x, fi, false, in.idx, in.nsrc) : operand(n->a[l], fi, false);
+        q.C = dst;
+        q.cstride = gp->stride[l];
+        q.M = fo;
+        q.N = fi;
+        q.K = in.rows;
+        q.epi = EPI_STORE;
+        tile(n, &q, parts);
+        g.col = ColSum{dcur, dst + (size_t)fo * fi, gp->stride[l], in.rows, fo, (fo + 31) / 32, parts, q.kper};
+        if (l == L - 1) {
+            const long nout = (long)in.rows * fo;
+            g.loss = LossSum{n->lossbuf + 1, nout, 1.0f / (float)nout, n->lossbuf, loss2};
         }
+        MLP_CUDA(launch_group(n, g, np, s));
+        float* tmp = dcur;
+        dcur = dnext;
+        dnext = tmp;
     }
     return KD_OK;
 }
@@ -493,6 +839,32 @@ int copy_io(void* dst, const void* src, size_t bytes, int32_t where_dst, int32_t
     cudaMemcpyKind k = where_src == KD_HOST ? (where_dst == KD_HOST ? cudaMemcpyHostToHost : cudaMemcpyHostToDevice)
                                             : (where_dst == KD_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice);
     MLP_CUDA(cudaMemcpyAsync(dst, src, bytes, k, s));
+    return KD_OK;
+}
+
+// the gradients in one buffer (grad): layers summed in parts are added up into it
+int gather_grads(kd_mlp* n, GradParts& gp, cudaStream_t s) {
+    bool split = false;
+    for (int l = 0; l < gp.L; ++l) split = split || gp.parts[l] > 1;
+    if (!split) return KD_OK;
+    k_sum_parts<<<(int)((n->nparam + 255) / 256), 256, 0, s>>>(gp, n->grad);
+    MLP_CUDA(cudaGetLastError());
+    return KD_OK;
+}
+
+int train_step(kd_mlp* n, const Batch& in, float lr, float* loss_dev, cudaStream_t s) {
+    MLP_CUDA(cudaSetDevice(n->device));
+    int rc = ensure_cap(n, in.rows);
+    if (rc) return rc;
+    GradParts gp;
+    rc = forward(n, in, s);
+    if (!rc) rc = backward(n, in, &gp, loss_dev, s);
+    if (rc) return rc;
+    ++n->adam_t;
+    const float b1 = 0.9f, b2 = 0.999f;
+    const float c1 = 1.0f - powf(b1, (float)n->adam_t), c2 = 1.0f - powf(b2, (float)n->adam_t);
+    MLP_CUDA(launch_pdl(k_adam, (long)((n->nparam + 255) / 256), 256, 0, s, n->param, gp, n->m1, n->m2, lr, b1, b2,
+                        1e-8f, c1, c2));
     return KD_OK;
 }
 
@@ -541,8 +913,7 @@ void kd_mlp_destroy(kd_mlp* n) {
     cudaFree(n->dbuf0);
     cudaFree(n->dbuf1);
     cudaFree(n->lossbuf);
-    cudaFree(n->gx);
-    cudaFree(n->gt);
+    cudaFree(n->part);
     cudaFree(n->status);
     cudaFree(n->param);
     cudaFree(n->grad);
@@ -597,7 +968,7 @@ int kd_mlp_forward(kd_mlp* n, const float* x, int32_t batch, float* y, int32_t w
         if (rc) return rc;
         xd = n->dbuf1;
     }
-    rc = forward(n, xd, batch, s);
+    rc = forward(n, Batch{xd, nullptr, nullptr, 0, batch}, s);
     if (rc) return rc;
     rc = copy_io(y, n->a[n->L], sizeof(float) * (size_t)batch * n->w[n->L], where, KD_DEVICE, s);
     if (rc) return rc;
@@ -628,8 +999,11 @@ int kd_mlp_gradients(kd_mlp* n, const float* x, const float* t, int32_t batch, f
         xd = tmp_x;
         td = tmp_t;
     }
-    rc = forward(n, xd, batch, s);
-    if (!rc) rc = backward(n, td, batch, s);
+    const Batch in{xd, td, nullptr, 0, batch};
+    GradParts gp;
+    rc = forward(n, in, s);
+    if (!rc) rc = backward(n, in, &gp, nullptr, s);
+    if (!rc && grads) rc = gather_grads(n, gp, s);
     if (!rc && loss) rc = copy_io(loss, n->lossbuf, sizeof(float), where, KD_DEVICE, s);
     if (!rc && grads) rc = copy_io(grads, n->grad, n->nparam * sizeof(float), where, KD_DEVICE, s);
     if (where == KD_HOST) {
@@ -645,39 +1019,13 @@ int kd_mlp_train_step_gather(kd_mlp* n, const float* x_all, const float* t_all, 
                              const int32_t* idx, int32_t batch, float lr, float* loss_dev, void* cuda_stream) {
     if (!n || !x_all || !t_all || !idx || n_all <= 0 || batch <= 0 || !(lr > 0))
         return err(KD_ERR_ARG, "kd_mlp_train_step_gather: bad argument");
-    MLP_CUDA(cudaSetDevice(n->device));
-    cudaStream_t s = (cudaStream_t)cuda_stream;
-    int rc = ensure_cap(n, batch);
-    if (rc) return rc;
-    if (!n->gx) {
-        MLP_CUDA(cudaMalloc(&n->gx, (size_t)n->cap * n->w[0] * sizeof(float)));
-        MLP_CUDA(cudaMalloc(&n->gt, (size_t)n->cap * n->w[n->L] * sizeof(float)));
-    }
-    const int win = n->w[0], wout = n->w[n->L];
-    k_gather_rows<<<(batch * win + 255) / 256, 256, 0, s>>>(x_all, win, (long)n_all, idx, batch, n->gx);
-    k_gather_rows<<<(batch * wout + 255) / 256, 256, 0, s>>>(t_all, wout, (long)n_all, idx, batch, n->gt);
-    MLP_CUDA(cudaGetLastError());
-    return kd_mlp_train_step(n, n->gx, n->gt, batch, lr, loss_dev, cuda_stream);
+    return train_step(n, Batch{x_all, t_all, idx, (long)n_all, batch}, lr, loss_dev, (cudaStream_t)cuda_stream);
 }
 
 int kd_mlp_train_step(kd_mlp* n, const float* x, const float* t, int32_t batch, float lr,
                       float* loss_dev, void* cuda_stream) {
     if (!n || !x || !t || batch <= 0 || !(lr > 0)) return err(KD_ERR_ARG, "kd_mlp_train_step: bad argument");
-    MLP_CUDA(cudaSetDevice(n->device));
-    cudaStream_t s = (cudaStream_t)cuda_stream;
-    int rc = ensure_cap(n, batch);
-    if (rc) return rc;
-    rc = forward(n, x, batch, s);
-    if (!rc) rc = backward(n, t, batch, s);
-    if (rc) return rc;
-    ++n->adam_t;
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = 1.0f - powf(b1, (float)n->adam_t), c2 = 1.0f - powf(b2, (float)n->adam_t);
-    k_adam<<<(int)((n->nparam + 255) / 256), 256, 0, s>>>(n->param, n->grad, n->m1, n->m2, (long)n->nparam,
-                                                          lr, b1, b2, 1e-8f, c1, c2);
-    MLP_CUDA(cudaGetLastError());
-    if (loss_dev) MLP_CUDA(cudaMemcpyAsync(loss_dev, n->lossbuf, sizeof(float), cudaMemcpyDeviceToDevice, s));
-    return KD_OK;
+    return train_step(n, Batch{x, t, nullptr, 0, batch}, lr, loss_dev, (cudaStream_t)cuda_stream);
 }
 
 }  // extern "C"
