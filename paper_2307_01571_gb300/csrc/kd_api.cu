@@ -883,7 +883,7 @@ SweepArgs make_args(const kd_sim* s, int axis, int op, const void* in, void* out
     const int logn = axis == AXIS_X ? s->lx : s->ly;
     const int var = s->prec == KD_FP64 ? 0 : s->var[axis];
     const bool dwk = s->dw && !view;   // the double-word kernels
-    a.tw = dwk ? s->tw_dw[axis] : s->tw[axis][sweep_loge(s->prec == KD_FP64, axis, logn, var) - 2];
+    a.tw = dwk ? s->tw_dw[axis] : s->tw[axis][(s->prec == KD_FP64 ? sweep_loge_f64(logn) : sweep_loge(axis, logn, var)) - 2];
     a.dwconst = s->dwconst;
     a.clock = s->clock;
     a.steps = s->steps;

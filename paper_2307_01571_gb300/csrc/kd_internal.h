@@ -106,16 +106,16 @@ __host__ __device__ constexpr SweepVariant sweep_variant(int axis, int v) {
          : v == 3 ? SweepVariant{3, 256, 4, 2, 28, 0}
                   : SweepVariant{3, 256, 4, 4, 16, 0});
 }
-// spinor components per CTA: FP64 CTAs own both pairs (the costly FP64 field is evaluated
-// once) except at N = 4096, where registers allow one pair
-__host__ __device__ constexpr int sweep_nc(bool f64, int axis, int logn, int v) {
-    return f64 ? (logn >= 12 ? 2 : 4) : sweep_variant(axis, v).nc;
-}
-// log2 of the elements per thread (the radix of the Stockham stages)
-__host__ __device__ constexpr int sweep_loge(bool f64, int axis, int logn, int v) {
-    const int lmax = f64 ? (sweep_nc(f64, axis, logn, v) == 2 ? 3 : 2) : sweep_variant(axis, v).loge;
+// spinor components per thread of the FP32 sweeps
+__host__ __device__ constexpr int sweep_nc(int axis, int v) { return sweep_variant(axis, v).nc; }
+// log2 of the elements per thread (the radix of the Stockham stages): FP32, FP64
+__host__ __device__ constexpr int sweep_loge(int axis, int logn, int v) {
+    const int lmax = sweep_variant(axis, v).loge;
     return logn < lmax ? logn : lmax;
 }
+// radix-4 stages up to 1024 points, radix-8 above, so that a line's threads stay within 256
+// (512 at 4096) and two lines fit on an SM
+__host__ __device__ constexpr int sweep_loge_f64(int logn) { return logn < 2 ? logn : (logn <= 10 ? 2 : 3); }
 
 // log2 of the elements per thread of the double-word form: radix-4 stages (four
 // double-word complex values per component keep the register use within two CTAs per SM)

@@ -20,6 +20,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <type_traits>
 
@@ -172,23 +173,38 @@ template <typename T, int LOGN, int AXIS, int V> struct Cfg {
     static constexpr bool DWT = std::is_same<T, DW>::value;      // double-word form
     static constexpr SweepVariant VS = sweep_variant(AXIS, F64 ? 0 : V);
     static constexpr int N = 1 << LOGN;
-    // components per thread: the double-word form keeps one pair per thread (its
-    // arithmetic needs many registers) and shares the field between the pairs of a CTA
-    static constexpr int NC = DWT ? 2 : sweep_nc(F64, AXIS, LOGN, V);
-    static constexpr int LOGE = DWT ? sweep_loge_dw(LOGN) : sweep_loge(F64, AXIS, LOGN, V);
+    // components per thread: the 64-bit forms keep one pair per thread
+    static constexpr int NC = F64 ? 2 : sweep_nc(AXIS, V);
+    static constexpr int LOGE = F64 ? (DWT ? sweep_loge_dw(LOGN) : sweep_loge_f64(LOGN)) : sweep_loge(AXIS, LOGN, V);
     static constexpr int E = 1 << LOGE;                          // elements per thread
     static constexpr int TF = N / E;                             // threads per line
-    // lines per CTA: rows are batched up to the variant's thread count; column tiles take
-    // that many threads and at least MINB columns (FP64: 2), i.e. >= 64-128 contiguous
-    // bytes per tile row, within 512 threads
-    static constexpr int MINB = F64 ? 2 : VS.minb;
+    // lines per CTA (FP32): rows are batched up to the variant's thread count; column tiles
+    // take that many threads and at least MINB columns, i.e. >= 64 contiguous bytes per tile
+    // row, within 512 threads
+    static constexpr int MINB = DWT ? 2 : VS.minb;
     // field sharing between the two pairs of a line (x axis, one pair per thread)
-    static constexpr bool SHARE = AXIS == AXIS_X && NC == 2 && TF <= 256 &&
-                                  (DWT || (!F64 && VS.share != 0));
+    static constexpr bool SHARE = AXIS == AXIS_X && NC == 2 && (DWT ? TF <= 128 : !F64 && TF <= 256 && VS.share != 0);
+    // The same between the two CTAs of a cluster (FP64; double-word from 1024 points): the CTAs
+    // of a row's two pairs evaluate half of the row's factors each and store them into both
+    // CTAs' shared memory.  The field is 100 (FP64) to 450 operations a point, so both pairs
+    // must not evaluate it; with the pairs in one CTA (double-word) or one thread (FP64) a
+    // 1024-point row takes a whole SM, and 512 rows on 152 SMs leave every sixth SM idle (4
+    // rounds of 3.4).  Half rows fit twice on an SM and go out in 6.7 of 7.  x sweep of
+    // 1024x512: FP64 422 -> 368 us, double-word 84.5 -> 74.0 (at 512 points and below two
+    // whole rows fit an SM and one CTA per row is as fast: 21.3 against 21.7 at 512x256).
+    // The FP64 pipe is then busy 98 % of the time: fewer FP64 operations are what is left.
+    static constexpr bool CSHARE = AXIS == AXIS_X && F64 && !SHARE;
     static constexpr int PCTA = SHARE ? 2 : 1;                  // pairs per CTA (NC = 2)
-    static constexpr int BATCH = AXIS == AXIS_X ? cmax(1, (DWT ? 256 : F64 ? 128 : VS.threads) / PCTA / TF)
-                                                : (TF * MINB > 512 ? cmax(1, 512 / TF)
-                                                                   : cmax(MINB, (F64 ? 256 : VS.threads) / TF));
+    // The 64-bit forms are bound by arithmetic, so what counts is that every SM has lines: one
+    // warp of lines per CTA (not for double-word columns, whose tiles of 256 threads measured
+    // faster: 17.0 against 19.4 us at 512x256).  128 lines of 128 points in CTAs of 4 rows and
+    // 8 columns used 32 and 16 of the 152 SMs.  FP64 columns are then read in 32-byte sectors,
+    // which costs less than a tenth of the arithmetic.  128x128 FP64: x 43.9 -> 21.4 us, y
+    // 74.5 -> 18.9; 1024x512 y 363 -> 313.
+    static constexpr int BATCH =
+        F64 && (!DWT || AXIS == AXIS_X) ? cmax(1, 32 / TF)
+        : AXIS == AXIS_X                ? cmax(1, VS.threads / PCTA / TF)
+                                        : (TF * MINB > 512 ? cmax(1, 512 / TF) : cmax(MINB, (DWT ? 256 : VS.threads) / TF));
     static constexpr int THREADS = TF * BATCH * PCTA;
     static constexpr int CPP = F64 ? 1 : 2;                      // complex per 16-byte unit
     static constexpr int NPL = NC / CPP;                         // units per point in the CTA
@@ -197,14 +213,16 @@ template <typename T, int LOGN, int AXIS, int V> struct Cfg {
     static constexpr int NST = plan_nst(LOGN, LOGE);
     static constexpr int BUF_UNITS = PCTA * BATCH * NPL * N;     // one exchange buffer
     // resident CTAs per SM the FP32 sweeps are built for (the variant's resident warps;
-    // the default puts the 1024x512 grid's lines in one wave); FP64 sweeps keep their full
-    // register budget
-    static constexpr int MINBLK = DWT ? cmax(1, 16 * 32 / THREADS)
-                                      : (F64 ? 1 : cmax(1, VS.resident_warps * 32 / THREADS));
+    // the default puts the 1024x512 grid's lines in one wave); 16 warps (128 registers a
+    // thread) for the 64-bit forms
+    static constexpr int MINBLK = cmax(1, (F64 ? 16 : VS.resident_warps) * 32 / THREADS);
     // two exchange buffers (one barrier per exchange) only when they keep that occupancy
     static constexpr bool DB = 2 * BUF_UNITS * 16 * MINBLK <= 200 * 1024;
-    static constexpr int SMEM_BYTES = cmax(NST > 1 ? (DB ? 2 : 1) * BUF_UNITS * 16 : 16,
-                                           SHARE ? BATCH * N * (DWT ? 32 : 16) : 16);
+    static constexpr int BUF_BYTES = cmax(NST > 1 ? (DB ? 2 : 1) * BUF_UNITS * 16 : 16,
+                                          SHARE && !F64 ? BATCH * N * 16 : 16);
+    // the 64-bit forms' factors [3][BATCH][N] of 8 bytes have their own region (a cluster's peer
+    // writes into it while this CTA still exchanges)
+    static constexpr int SMEM_BYTES = BUF_BYTES + (F64 && AXIS == AXIS_X ? 24 * BATCH * N : 0);
     // lanes of one 8-lane (128-byte) shared-memory wavefront cover 2^LOGG consecutive
     // butterflies
     static constexpr int LOGG =
@@ -549,65 +567,77 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
     }
 
     KD_DI static void op_potential(const SweepArgs& a, const Ctx& c, C* v, const RowField rf) {
-        if constexpr (DWF) op_potential_dw(a, c, v, rf);
+        if constexpr (Cf::F64) op_potential_shared(a, c, v, rf);
         else op_potential_std(a, c, v, rf);
     }
 
-    // the double-word potential step: the field of the standing wave as in op_potential_std
-    // with every quantity a double-word and exp, sin, cos of kd_dw.cuh (relative error
-    // ~1e-14 of the field, so that the factor is exact to the double-word rounding unit
-    // over thousands of steps); table a.xtab holds per column x two double-word 4-vectors
-    // (Theta0, x/(x_R w^2), w0/w, 1/w^2) and (1/w, cos zeta, sin zeta, cos k x) as four
-    // float4 [2][nx][2]
-    KD_DI static void op_potential_dw(const SweepArgs& a, const Ctx& c, C* v, const RowField rf) {
-        if constexpr (DWF) {
+    // whether this sweep trades potential factors through its cluster (uniform in the grid)
+    KD_DI static bool trades(const SweepArgs& a) { return Cf::CSHARE && a.op == OP_POTENTIAL && a.kind != 0; }
+    KD_DI static void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+    KD_DI static void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+    // The potential step of the 64-bit forms.  The two halves of a CTA, or the two CTAs of a
+    // cluster, hold the two pairs of the same rows, thread for thread the same points: each
+    // evaluates the factors (cos theta - 1, s a_y, s a_x) of its half of every thread's points
+    // (e of parity c.pair) and stores them into the shared memory of both.  In a cluster, the
+    // peer's first barrier phase (arrived at the kernel's start) says that it runs; the second
+    // that all factors are in place.  Nothing is stored into the peer after that, so either
+    // CTA may exit.
+    KD_DI static void op_potential_shared(const SweepArgs& a, const Ctx& c, C* v, const RowField rf) {
+        if constexpr (Cf::F64) {
             if (a.kind == 0) return;
-            constexpr int R = 1 << LR_OP;
-            const DW y = rf.y, st = rf.st;
-            const DW y2 = dw_mul(y, y);
-            const DW kap = dw_from_double(a.kappa), e4 = dw_from_double(a.eps4);
-            if constexpr (!Cf::SHARE) {
-                // pairs in separate CTAs (lines of more than 256 threads): every thread
-                // evaluates the factors of all its points
-#pragma unroll
-                for (int m = 0; m < E / R; ++m)
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const int x = c.jt + m * TF + r * (N / R);
-                        const DWFactor f = dw_potential_factor(a.xtab, a.dwconst, a.nx, x, a.kind,
-                                                               a.longitudinal, y, y2, st, kap, e4);
-                        apply_potential_dw(c, v + (m * R + r) * NC, f.c1, f.say, f.sax);
-                    }
-                return;
+            constexpr int R = 1 << LR_OP, PL = BATCH * N;
+            using F = typename std::conditional<DWF, float2, double>::type;
+            F* fac = reinterpret_cast<F*>(reinterpret_cast<unsigned char*>(c.sm) + Cf::BUF_BYTES) + c.bb % BATCH * N;
+            uint32_t peer = 0;
+            if constexpr (Cf::CSHARE) {
+                asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer)
+                    : "r"((uint32_t)__cvta_generic_to_shared(fac)), "r"(c.pair ^ 1));
+                cluster_wait();
             }
-            // the two pairs' threads own the same points: each evaluates the factors of the
-            // points of parity c.pair into shared memory, and both read all of them back
-            constexpr int SLOT = Cf::DB ? ((NST - 1) & 1) * Cf::BUF_UNITS : 0;
-            float4* fsh = reinterpret_cast<float4*>(c.sm + SLOT) + 2 * (c.bb % BATCH) * N;
+            const T y = rf.y, st = rf.st, y2 = y * y;
 #pragma unroll
-            for (int m = 0; m < E / R; ++m)
+            for (int h = 0; h < E / 2; ++h) {
+                const int e = 2 * h + c.pair;
+                const int x = c.jt + (e / R) * TF + (e % R) * (N / R);
+                F f[3];
+                if constexpr (DWF) {
+                    const DWFactor q = dw_potential_factor(a.xtab, a.dwconst, a.nx, x, a.kind, a.longitudinal, y, y2,
+                                                           st, dw_from_double(a.kappa), dw_from_double(a.eps4));
+                    f[0] = make_float2(q.c1.h, q.c1.l);
+                    f[1] = make_float2(q.say.h, q.say.l);
+                    f[2] = make_float2(q.sax.h, q.sax.l);
+                } else {
+                    potential_factor(a, x, y, y2, st, a.kappa, a.eps4, f);
+                }
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    if (((m * R + r) & 1) != c.pair) continue;
-                    const int x = c.jt + m * TF + r * (N / R);
-                    const DWFactor f = dw_potential_factor(a.xtab, a.dwconst, a.nx, x, a.kind, a.longitudinal,
-                                                           y, y2, st, kap, e4);
-                    if (c.valid) {
-                        fsh[2 * x] = make_float4(f.c1.h, f.c1.l, f.say.h, f.say.l);
-                        fsh[2 * x + 1] = make_float4(f.sax.h, f.sax.l, 0.0f, 0.0f);
+                for (int k = 0; k < 3; ++k) {
+                    fac[k * PL + x] = f[k];
+                    if constexpr (Cf::CSHARE) {
+                        long long bits;
+                        memcpy(&bits, &f[k], 8);
+                        asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(peer + 8u * (uint32_t)(k * PL + x)), "l"(bits)
+                                     : "memory");
                     }
                 }
-            block_sync(c);
+            }
+            if constexpr (Cf::CSHARE) {
+                cluster_arrive();
+                cluster_wait();
+            } else {
+                block_sync(c);
+            }
 #pragma unroll
             for (int m = 0; m < E / R; ++m)
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     const int x = c.jt + m * TF + r * (N / R);
-                    const float4 f0 = c.valid ? fsh[2 * x] : make_float4(0.f, 0.f, 0.f, 0.f);
-                    const float4 f1 = c.valid ? fsh[2 * x + 1] : make_float4(0.f, 0.f, 0.f, 0.f);
-                    apply_potential_dw(c, v + (m * R + r) * NC, DW{f0.x, f0.y}, DW{f0.z, f0.w}, DW{f1.x, f1.y});
+                    const F f0 = fac[x], f1 = fac[PL + x], f2 = fac[2 * PL + x];
+                    if constexpr (DWF)
+                        apply_potential_dw(c, v + (m * R + r) * NC, DW{f0.x, f0.y}, DW{f1.x, f1.y}, DW{f2.x, f2.y});
+                    else
+                        apply_potential(c, v + (m * R + r) * NC, f0, f1, f2);
                 }
-            if constexpr (!Cf::DB) block_sync(c);
         }
     }
 
@@ -625,10 +655,47 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
         }
     }
 
+    // the factor (cos theta - 1, s a_y, s a_x), s = sin(theta)/|a|, of one point
+    KD_DI static void potential_factor(const SweepArgs& a, int x, T y, T y2, T st, T kap, T e4, T* f) {
+        using T4 = typename std::conditional<sizeof(T) == 4, float4, double4>::type;
+        const T4* xt = reinterpret_cast<const T4*>(a.xtab);   // [2][nx] vectors
+        const T4 t1 = xt[a.nx + x];      // (1/w, cos zeta, sin zeta, cos k x)
+        T ax = T(0), ay;
+        if (a.kind == 1) {
+            ay = T(-2) * st * t1.w;
+        } else {
+            const T4 t0 = xt[x];         // (Theta0, x/(x_R w^2), w0/w, 1/w^2)
+            const T G = t0.z * fexp(-y2 * t0.w);
+            T th = t0.x - t0.y * y2;
+            if constexpr (sizeof(T) == 4) th -= 6.283185307f * rintf(th * 0.159154943f);
+            T sn, cs;
+            fsincos(th, &sn, &cs);
+            const T sg = st * G;
+            ay = T(-2) * sg * cs;
+            if (a.longitudinal) ax = e4 * sg * (y * t1.x) * (sn * t1.y + cs * t1.z);
+        }
+        const T a2 = ax * ax + ay * ay;
+        const T th2 = kap * kap * a2;
+        T c1, s;   // cos(theta) - 1 and sin(theta)/|a|, theta = kappa |a|
+        if (th2 < T(0.0625)) {
+            T sinc;
+            small_rotation(th2, &c1, &sinc);
+            s = kap * sinc;
+        } else {
+            const T amag = sqrt(a2);
+            T sh, ch;
+            sincos_(T(0.5) * kap * amag, &sh, &ch);
+            c1 = T(-2) * sh * sh;
+            s = T(2) * sh * ch / amag;
+        }
+        f[0] = c1;
+        f[1] = s * ay;
+        f[2] = s * ax;
+    }
+
     KD_DI static void op_potential_std(const SweepArgs& a, const Ctx& c, C* v, const RowField rf) {
         if (a.kind == 0) return;
         constexpr int R = 1 << LR_OP;
-        using T4 = typename std::conditional<sizeof(T) == 4, float4, double4>::type;
         const T y = rf.y, st = rf.st;
         T kap, e4;
         if constexpr (sizeof(T) == 4) {
@@ -639,9 +706,6 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
             e4 = a.eps4;
         }
         const T y2 = y * y;
-        const T kap2 = kap * kap;
-        const T4* xt = reinterpret_cast<const T4*>(a.xtab);   // [2][nx] vectors
-        const int nx = a.nx;
         // field sharing: this thread evaluates the points e = m R + r of parity c.pair, and
         // both pairs' threads read all factors (cos theta - 1, s a_y, s a_x) back from
         // shared memory
@@ -658,39 +722,12 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
                 if constexpr (Cf::SHARE) {
                     if (((m * R + r) & 1) != c.pair) continue;
                 }
-                const T4 t1 = xt[nx + x];        // (1/w, cos zeta, sin zeta, cos k x)
-                T ax = T(0), ay;
-                if (a.kind == 1) {
-                    ay = T(-2) * st * t1.w;
-                } else {
-                    const T4 t0 = xt[x];         // (Theta0, x/(x_R w^2), w0/w, 1/w^2)
-                    const T G = t0.z * fexp(-y2 * t0.w);
-                    T th = t0.x - t0.y * y2;
-                    if constexpr (sizeof(T) == 4) th -= 6.283185307f * rintf(th * 0.159154943f);
-                    T sn, cs;
-                    fsincos(th, &sn, &cs);
-                    const T sg = st * G;
-                    ay = T(-2) * sg * cs;
-                    if (a.longitudinal) ax = e4 * sg * (y * t1.x) * (sn * t1.y + cs * t1.z);
-                }
-                const T a2 = ax * ax + ay * ay;
-                const T th2 = kap2 * a2;
-                T c1, s;   // cos(theta) - 1 and sin(theta)/|a|, theta = kappa |a|
-                if (th2 < T(0.0625)) {
-                    T sinc;
-                    small_rotation(th2, &c1, &sinc);
-                    s = kap * sinc;
-                } else {
-                    const T amag = sqrt(a2);
-                    T sh, ch;
-                    sincos_(T(0.5) * kap * amag, &sh, &ch);
-                    c1 = T(-2) * sh * sh;
-                    s = T(2) * sh * ch / amag;
-                }
+                T f[3];
+                potential_factor(a, x, y, y2, st, kap, e4, f);
                 if constexpr (Cf::SHARE) {
-                    if (c.valid) fsh[x] = make_float4(c1, s * ay, s * ax, 0.0f);
+                    if (c.valid) fsh[x] = make_float4(f[0], f[1], f[2], 0.0f);
                 } else {
-                    apply_potential(c, v + (m * R + r) * NC, c1, s * ay, s * ax);
+                    apply_potential(c, v + (m * R + r) * NC, f[0], f[1], f[2]);
                 }
             }
         if constexpr (Cf::SHARE) {
@@ -863,6 +900,7 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
         c.valid = c.line < (AXIS == AXIS_X ? a.ny : a.nx);
         c.sm = reinterpret_cast<U*>(smem);
         C v[E * NC];
+        if (trades(a)) cluster_arrive();   // this CTA runs: its shared memory may be written
         // programmatic dependent launch: everything above ran while the previous kernel
         // in the stream was still finishing; its results are visible after this wait
         // (a hardware-managed wait for the prerequisite grid, not a spin loop)
@@ -880,8 +918,8 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
             if constexpr (HAS1) fft<DIR1, false, 0, 0>(a, c, v);
             if (a.op == OP_POTENTIAL) op_potential(a, c, v, rf);
         }
-        // with field sharing the factor trade takes exchange slot NST - 1, so FFT2 starts at NST
-        if constexpr (HAS2) fft<DIR2, true, Cf::SHARE ? NST : (HAS1 ? NST - 1 : 0), 0>(a, c, v);
+        // with field sharing (FP32) the factor trade takes exchange slot NST - 1, so FFT2 starts at NST
+        if constexpr (HAS2) fft<DIR2, true, Cf::SHARE && !Cf::F64 ? NST : (HAS1 ? NST - 1 : 0), 0>(a, c, v);
         store<LR_STORE>(a, c, v);
     }
 };
@@ -909,11 +947,13 @@ cudaError_t launch_one(const SweepArgs& a, cudaStream_t s) {
     cfg.blockDim = dim3(Cf::THREADS);
     cfg.dynamicSmemBytes = Cf::SMEM_BYTES;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim = {2, 1, 1};
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = Cf::CSHARE ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, k, a);
 }
 
