@@ -113,7 +113,7 @@ struct kd_sim {
     size_t P;
     void* psi = nullptr;
     void* work = nullptr;
-    void* tw[2][2] = {};   // twiddle tables [axis][loge - 2] (radix-4 and radix-8 schedules)
+    void* tw[2][3] = {};   // twiddle tables [axis][loge - 2] (radix-4, radix-8, FP32: radix-16)
     int var[2] = {0, 0};   // sweep launch variant per axis (kd_autotune)
     void* xtab = nullptr;
     void* kxtab = nullptr;
@@ -664,9 +664,9 @@ template <typename T> int upload_dw_tables(kd_sim* s, const std::vector<T>& xt, 
 template <typename T> int upload_tables_t(kd_sim* s) {
     const int nx = s->g.nx;
     // stage-major twiddle tables, built on the device in FP64 (<= 2N entries of 16 B)
-    // for both radix schedules a launch variant may use
+    // for every radix schedule a launch shape may use
     for (int ax = 0; ax < 2; ++ax)
-        for (int le = 2; le <= 3; ++le) {
+        for (int le = 2; le <= (sizeof(T) == 4 ? 4 : 3); ++le) {
             int entries = 0;
             const int logn = ax == 0 ? s->lx : s->ly;
             void* dst = s->tw[ax][le - 2];
@@ -870,6 +870,12 @@ int build_dt_tables(kd_sim* s, double dt) {
     return s->prec == KD_FP64 ? build_dt_tables_t<double>(s, dt) : build_dt_tables_t<float>(s, dt);
 }
 
+// The compiled form of the FP32 sweeps that the simulation's launch variant runs on its grid
+int form(const kd_sim* s, int axis) {
+    return axis == AXIS_X ? sweep_form_of(axis, s->var[axis], s->lx, s->g.ny)
+                          : sweep_form_of(axis, s->var[axis], s->ly, s->g.nx);
+}
+
 // One fused sweep of the state (the simulation's own form), or, with view = true, an FP64
 // transform of the FP64 view of the state (read-outs of the double-word form).
 SweepArgs make_args(const kd_sim* s, int axis, int op, const void* in, void* out, int n_local,
@@ -881,9 +887,8 @@ SweepArgs make_args(const kd_sim* s, int axis, int op, const void* in, void* out
     a.ny = s->g.ny;
     a.op = op;
     const int logn = axis == AXIS_X ? s->lx : s->ly;
-    const int var = s->prec == KD_FP64 ? 0 : s->var[axis];
     const bool dwk = s->dw && !view;   // the double-word kernels
-    a.tw = dwk ? s->tw_dw[axis] : s->tw[axis][(s->prec == KD_FP64 ? sweep_loge_f64(logn) : sweep_loge(axis, logn, var)) - 2];
+    a.tw = dwk ? s->tw_dw[axis] : s->tw[axis][(s->prec == KD_FP64 ? sweep_loge_f64(logn) : sweep_loge(axis, logn, form(s, axis))) - 2];
     a.dwconst = s->dwconst;
     a.clock = s->clock;
     a.steps = s->steps;
@@ -917,13 +922,12 @@ cudaError_t sweep(kd_sim* s, int axis, int shape, int op, const void* in, void* 
                   double tau, bool view = false) {
     const SweepArgs a = make_args(s, axis, op, in, out, n_local, tau, view);
     const int logn = axis == AXIS_X ? s->lx : s->ly;
-    const int var = s->prec == KD_FP64 ? 0 : s->var[axis];
     const bool dwk = s->dw && !view;
     ++s->launches;
     if (s->tc && shape == SHAPE_F1F2 && tc_supported(logn)) return launch_tc_sweep(axis, a, s->stream);
     if (dwk) return launch_sweep_dw(axis, shape, logn, a, s->stream);
     return s->prec == KD_FP64 ? launch_sweep_f64(axis, shape, logn, a, s->stream)
-                              : launch_sweep_f32(var, axis, shape, logn, a, s->stream);
+                              : launch_sweep_f32(form(s, axis), axis, shape, logn, a, s->stream);
 }
 
 // ------------------------------------------------------------------ autotuner ------
@@ -1354,7 +1358,7 @@ int kd_create(const kd_units* units, const kd_grid* grid, const kd_field* field,
             return bail(fail(KD_ERR_CUDA, "event create failed"));
     KD_ALLOC(s->psi, spinor_bytes(s));
     KD_ALLOC(s->work, spinor_bytes(s));
-    for (int le = 0; le < 2; ++le) {
+    for (int le = 0; le < 3; ++le) {
         KD_ALLOC(s->tw[AXIS_X][le], 2 * (size_t)grid->nx * 16);
         KD_ALLOC(s->tw[AXIS_Y][le], 2 * (size_t)grid->ny * 16);
     }
@@ -1400,7 +1404,7 @@ void kd_destroy(kd_sim* s) {
     cudaSetDevice(s->device);
     cudaStreamSynchronize(s->stream);
     clear_graphs(s);
-    void* bufs[] = {s->psi, s->work, s->tw[0][0], s->tw[0][1], s->tw[1][0], s->tw[1][1], s->xtab,
+    void* bufs[] = {s->psi, s->work, s->tw[0][0], s->tw[0][1], s->tw[0][2], s->tw[1][0], s->tw[1][1], s->tw[1][2], s->xtab,
                     s->kxtab, s->kytab, s->ktab, s->clock, s->steps, s->rowsum, s->md, s->scalar,
                     s->obs_dev, s->status, s->tc_b, s->tc_tw, s->tc_scale, s->tw_dw[0], s->tw_dw[1],
                     s->dwconst, s->view};
@@ -1807,7 +1811,7 @@ int persist_upload(kd_batch* b, const std::vector<StepPlan>& plans, bool* hold) 
         // the member's own launch variants where the kernel holds them, else its defaults;
         // the same number of CTA-fulls per work item for every member (uneven groups let
         // the large members' items set the pace of every sweep)
-        m.vx_alt = persist_variant_alt(AXIS_X, s->var[AXIS_X], s->lx);
+        m.vx_alt = persist_variant_alt(AXIS_X, form(s, AXIS_X), s->lx);
         m.vy_alt = persist_variant_alt(AXIS_Y, s->var[AXIS_Y], s->ly);
         m.cy = persist_ctas(AXIS_Y, m.vy_alt, s->ly, s->g.nx);
         m.cx = persist_ctas(AXIS_X, m.vx_alt, s->lx, s->g.ny);

@@ -107,10 +107,56 @@ __host__ __device__ constexpr SweepVariant sweep_variant(int axis, int v) {
                   : SweepVariant{3, 256, 4, 4, 16, 0});
 }
 // spinor components per thread of the FP32 sweeps
-__host__ __device__ constexpr int sweep_nc(int axis, int v) { return sweep_variant(axis, v).nc; }
+__host__ __device__ constexpr int sweep_nc(int axis, int v);
+
+// The compiled forms of the FP32 sweeps: 0 ... 3 the variants as in the table, and two that
+// the default (variants 0 and 1) becomes by the grid's size, sweep_form_of below.
+//   small: radix-4 stages, one or two rows / two columns per CTA.  A small grid is bound by
+//     the latency of one CTA and by idle SMs: 128 columns of 128 points in tiles of eight
+//     columns and both pairs were 16 CTAs on 152 SMs.
+//   large: radix-16 stages (sixteen elements a thread).  A grid of many rounds is bound by the
+//     shared-memory exchanges and twiddle loads together with the FP32 pipe; radix-16 stages
+//     take two thirds of the former, and many rounds make up for the fewer warps.
+constexpr int kFormSmall = 4, kFormLarge = 5, kNumSweepForms = 6;
+__host__ __device__ constexpr SweepVariant sweep_form(int axis, int form) {
+    if (form < kNumSweepVariants) return sweep_variant(axis, form);
+    if (axis == AXIS_X) return form == kFormSmall ? SweepVariant{2, 64, 1, 2, 32, 0} : SweepVariant{4, 64, 1, 2, 16, 0};
+    return form == kFormSmall ? SweepVariant{2, 64, 2, 2, 32, 0} : SweepVariant{4, 256, 2, 2, 16, 0};
+}
+// axis lengths a form is compiled for
+__host__ __device__ constexpr bool sweep_form_holds(int form, int logn) {
+    return form == kFormSmall ? logn <= 11 : (form == kFormLarge ? logn >= 10 : true);
+}
+// The form that variant v runs on `lines` lines of 2^logn points.  The lines lie where the
+// measured times cross (GB300, us per sweep, default form against the chosen one):
+//   x, up to 2^17 points: 64x64 4.9 : 3.2, 256x256 5.6 : 4.2, 1024x128 7.4 : 6.5, 2048x64
+//     7.7 : 7.3; at 2^18 the radix-8 default is ahead (512x512 8.6 : 9.2);
+//   x, 2048 and 4096 points: both pairs per thread (variant 3, the field evaluated once) up to
+//     2^20 points (2048x128 12.9 : 10.9, 2048x256 18.7 : 15.5, 4096x256 40.0 : 33.1), then
+//     large (2048x512 29.7 : 27.8, 4096x2048 288 : 234); 4096x64 is too few rows for
+//     variant 3 (11.1 : 16.7);
+//   y up to 512 points: small up to 2^16 points (64x64 5.4 : 2.2, 128x128 6.5 : 2.5, 256x256
+//     7.1 : 4.1), radix-4 tiles of both pairs at 2^17 (512x256 7.2 : 5.0);
+//   y from 1024 points (few columns): small up to 2^17 points (128x1024 15.6 : 7.0, 64x2048
+//     18.7 : 10.1), one pair per CTA at 2^18 (256x1024 15.8 : 9.8, 128x2048 18.8 : 11.2),
+//     then large (1024x1024 30.7 : 29.5, 2048x1024 61.6 : 54.6, 4096x2048 292 : 263).
+inline int sweep_form_of(int axis, int v, int logn, int lines) {
+    if (v > 1) return v;
+    const long long points = (long long)lines << logn;
+    if (axis == AXIS_X) {
+        if (logn <= 11 && points <= 1 << 17) return kFormSmall;
+        if (logn <= 10 || points <= 1 << (logn == 11 ? 17 : 18)) return v;
+        return points < 1 << 20 ? 3 : kFormLarge;
+    }
+    if (logn <= 9) return points <= 1 << 16 ? kFormSmall : (points <= 1 << 17 ? 2 : v);
+    if (logn <= 11 && points <= 1 << 17) return kFormSmall;
+    return points <= 1 << 18 ? 3 : kFormLarge;
+}
+
+__host__ __device__ constexpr int sweep_nc(int axis, int v) { return sweep_form(axis, v).nc; }
 // log2 of the elements per thread (the radix of the Stockham stages): FP32, FP64
 __host__ __device__ constexpr int sweep_loge(int axis, int logn, int v) {
-    const int lmax = sweep_variant(axis, v).loge;
+    const int lmax = sweep_form(axis, v).loge;
     return logn < lmax ? logn : lmax;
 }
 // radix-4 stages up to 1024 points, radix-8 above, so that a line's threads stay within 256
@@ -122,11 +168,11 @@ __host__ __device__ constexpr int sweep_loge_f64(int logn) { return logn < 2 ? l
 // up to 1024-point lines, radix-8 above (a line's threads stay within 256)
 __host__ __device__ constexpr int sweep_loge_dw(int logn) { return logn < 2 ? logn : (logn <= 10 ? 2 : 3); }
 
-// Launches one sweep; returns cudaSuccess or the launch error.  logn in [2, 12],
-// variant in [0, kNumSweepVariants).
+// Launches one sweep; returns cudaSuccess or the launch error.  logn in [2, 12], form in
+// [0, kNumSweepForms) and compiled for logn.
 template <int V>
 cudaError_t launch_sweep_f32_v(int axis, int shape, int logn, const SweepArgs& a, cudaStream_t s);
-cudaError_t launch_sweep_f32(int variant, int axis, int shape, int logn, const SweepArgs& a,
+cudaError_t launch_sweep_f32(int form, int axis, int shape, int logn, const SweepArgs& a,
                              cudaStream_t s);
 cudaError_t launch_sweep_f64(int axis, int shape, int logn, const SweepArgs& a, cudaStream_t s);
 // Double-word form (KD_DW): the FP64 form's launch shapes with every real a float pair.

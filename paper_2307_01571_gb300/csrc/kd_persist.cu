@@ -244,7 +244,8 @@ int persist_ctas(int axis, int alt, int logn, int lines) {
 }
 
 int persist_variant_alt(int axis, int variant, int logn) {
-    if (axis == AXIS_X) return variant == kVX1 ? 1 : 0;
+    // the small form's rows take the radix-4 variant's arithmetic (they differ in threads per CTA)
+    if (axis == AXIS_X) return variant == kVX1 || variant == kFormSmall ? 1 : 0;
     return variant == kVY1 && logn <= kMaxLogVY1 ? 1 : 0;
 }
 

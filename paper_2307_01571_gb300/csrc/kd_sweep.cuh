@@ -110,20 +110,64 @@ template <int DIR, int S, typename C> KD_DI void dft8(C* a) {
     }
 }
 
+// a times c + DIR i s, the constants as hi + lo pairs (as the stage twiddles; FP32)
+template <int DIR> KD_DI float2 mul_const(float2 a, double c, double s) {
+    const float ch = (float)c, cl = (float)(c - (double)ch), sn = (float)s;
+    const float sh = DIR > 0 ? sn : -sn, sl = (float)(DIR > 0 ? s - (double)sn : (double)sn - s);
+    return make_float2(fmaf(a.x, ch, fmaf(-a.y, sh, fmaf(a.x, cl, -a.y * sl))),
+                       fmaf(a.x, sh, fmaf(a.y, ch, fmaf(a.x, sl, a.y * cl))));
+}
+
+// sixteen points as four by four (FP32): two thirds of the exchanges and twiddle loads of
+// radix-8 stages, for lines long enough to fill the SMs with a quarter fewer warps
+template <int DIR, int S> KD_DI void dft16(float2* a) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) dft4<DIR, 4 * S>(a + j * S);
+    constexpr double c = 0.92387953251128675613, s = 0.38268343236508977173;   // cos, sin of pi/8
+    auto w2 = [](float2 v) { return make_float2(mul_rsqrt2(v.x - DIR * v.y), mul_rsqrt2(v.y + DIR * v.x)); };
+    auto w6 = [](float2 v) { return make_float2(mul_rsqrt2(-v.x - DIR * v.y), mul_rsqrt2(-v.y + DIR * v.x)); };
+    a[5 * S] = mul_const<DIR>(a[5 * S], c, s);        // w16^(j k), j k = 1 1
+    a[6 * S] = w2(a[6 * S]);                          // 2 1
+    a[7 * S] = mul_const<DIR>(a[7 * S], s, c);        // 3 1
+    a[9 * S] = w2(a[9 * S]);                          // 1 2
+    a[10 * S] = mul_i<DIR>(a[10 * S]);                // 2 2
+    a[11 * S] = w6(a[11 * S]);                        // 3 2
+    a[13 * S] = mul_const<DIR>(a[13 * S], s, c);      // 1 3
+    a[14 * S] = w6(a[14 * S]);                        // 2 3
+    a[15 * S] = mul_const<DIR>(a[15 * S], -c, -s);    // 3 3
+    float2 b[16];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        dft4<DIR, S>(a + 4 * k * S);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) b[k + 4 * q] = a[(4 * k + q) * S];
+    }
+#pragma unroll
+    for (int k = 0; k < 16; ++k) a[k * S] = b[k];
+}
+
 template <int R, int DIR, int S, typename C> KD_DI void dftR(C* a) {
     if constexpr (R == 2) dft2<DIR, S>(a);
     else if constexpr (R == 4) dft4<DIR, S>(a);
-    else dft8<DIR, S>(a);
+    else if constexpr (R == 8) dft8<DIR, S>(a);
+    else dft16<DIR, S>(a);
 }
 
 // ------------------------------------------------------------- plan ---------------
 // Radix plan of an N = 2^logn point FFT with maximum radix 2^loge: as many radix-2^loge
 // stages as fit, the remainder as radix-4 or radix-2 stages.
 __host__ __device__ constexpr int plan_nst(int logn, int loge) {
+    if (loge == 4) return logn % 4 == 0 ? logn / 4 : logn / 4 + 1;
     return loge == 3 ? (logn % 3 == 0 ? logn / 3 : logn / 3 + 1)
                      : (loge == 2 ? logn / 2 + logn % 2 : logn);
 }
 __host__ __device__ constexpr int plan_logr(int logn, int loge, int s) {
+    if (loge == 4) {
+        int q = logn / 4, r = logn % 4;
+        if (r == 0) return 4;
+        if (r == 1) return s < q - 1 ? 4 : (s == q - 1 ? 3 : 2);
+        return s < q ? 4 : r;
+    }
     if (loge == 3) {
         int q = logn / 3, r = logn % 3;
         if (r == 0) return 3;
@@ -171,7 +215,7 @@ __host__ __device__ constexpr int clog2(int v) { return v <= 1 ? 0 : 1 + clog2(v
 template <typename T, int LOGN, int AXIS, int V> struct Cfg {
     static constexpr bool F64 = sizeof(T) == 8;                  // FP64 or double-word
     static constexpr bool DWT = std::is_same<T, DW>::value;      // double-word form
-    static constexpr SweepVariant VS = sweep_variant(AXIS, F64 ? 0 : V);
+    static constexpr SweepVariant VS = sweep_form(AXIS, F64 ? 0 : V);
     static constexpr int N = 1 << LOGN;
     // components per thread: the 64-bit forms keep one pair per thread
     static constexpr int NC = F64 ? 2 : sweep_nc(AXIS, V);
@@ -911,8 +955,10 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
         if constexpr (PDL) asm volatile("griddepcontrol.launch_dependents;");
         if constexpr (AXIS == AXIS_Y) {
             C kab[E];
-            if (a.op == OP_KINETIC) load_ktab(a, c, kab);
+            // (after the FFT where sixteen elements a thread leave no registers for it)
+            if (E < 16 && a.op == OP_KINETIC) load_ktab(a, c, kab);
             if constexpr (HAS1) fft<DIR1, false, 0, 0>(a, c, v);
+            if (E >= 16 && a.op == OP_KINETIC) load_ktab(a, c, kab);
             if (a.op == OP_KINETIC) op_kinetic(a, c, v, kab);
         } else {
             if constexpr (HAS1) fft<DIR1, false, 0, 0>(a, c, v);
@@ -1030,6 +1076,8 @@ template <typename T, int LOGN, int LOGE> cudaError_t build_tw(void* out, int* e
 template <typename T, int LOGN> cudaError_t build_tw_e(int loge, void* out, int* entries, cudaStream_t s) {
     if (loge == 2) return build_tw<T, LOGN, 2>(out, entries, s);
     if (loge == 3) return build_tw<T, LOGN, 3>(out, entries, s);
+    if constexpr (std::is_same<T, float>::value)
+        if (loge == 4) return build_tw<T, LOGN, 4>(out, entries, s);
     return cudaErrorInvalidValue;
 }
 
@@ -1050,20 +1098,26 @@ template <typename T> cudaError_t build_twiddles(int logn, int loge, void* out, 
     }
 }
 
+template <typename T, int LOGN, int AXIS, int SHAPE, int V>
+cudaError_t launch_held(const SweepArgs& a, cudaStream_t s) {
+    if constexpr (sizeof(T) == 4 && !sweep_form_holds(V, LOGN)) return cudaErrorInvalidValue;
+    else return launch_one<T, LOGN, AXIS, SHAPE, V>(a, s);
+}
+
 template <typename T, int AXIS, int SHAPE, int V>
 cudaError_t launch_logn(int logn, const SweepArgs& a, cudaStream_t s) {
     switch (logn) {
-        case 2: return launch_one<T, 2, AXIS, SHAPE, V>(a, s);
-        case 3: return launch_one<T, 3, AXIS, SHAPE, V>(a, s);
-        case 4: return launch_one<T, 4, AXIS, SHAPE, V>(a, s);
-        case 5: return launch_one<T, 5, AXIS, SHAPE, V>(a, s);
-        case 6: return launch_one<T, 6, AXIS, SHAPE, V>(a, s);
-        case 7: return launch_one<T, 7, AXIS, SHAPE, V>(a, s);
-        case 8: return launch_one<T, 8, AXIS, SHAPE, V>(a, s);
-        case 9: return launch_one<T, 9, AXIS, SHAPE, V>(a, s);
-        case 10: return launch_one<T, 10, AXIS, SHAPE, V>(a, s);
-        case 11: return launch_one<T, 11, AXIS, SHAPE, V>(a, s);
-        case 12: return launch_one<T, 12, AXIS, SHAPE, V>(a, s);
+        case 2: return launch_held<T, 2, AXIS, SHAPE, V>(a, s);
+        case 3: return launch_held<T, 3, AXIS, SHAPE, V>(a, s);
+        case 4: return launch_held<T, 4, AXIS, SHAPE, V>(a, s);
+        case 5: return launch_held<T, 5, AXIS, SHAPE, V>(a, s);
+        case 6: return launch_held<T, 6, AXIS, SHAPE, V>(a, s);
+        case 7: return launch_held<T, 7, AXIS, SHAPE, V>(a, s);
+        case 8: return launch_held<T, 8, AXIS, SHAPE, V>(a, s);
+        case 9: return launch_held<T, 9, AXIS, SHAPE, V>(a, s);
+        case 10: return launch_held<T, 10, AXIS, SHAPE, V>(a, s);
+        case 11: return launch_held<T, 11, AXIS, SHAPE, V>(a, s);
+        case 12: return launch_held<T, 12, AXIS, SHAPE, V>(a, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -1,6 +1,6 @@
 // Instantiates the fused sweep kernels for float spinors, one launch variant per object
 // file: the build compiles this file once per KD_SWEEP_VARIANT so that the variants
-// compile in parallel.
+// compile in parallel (kd_sweep_f32_forms.cu does the same for the forms beyond them).
 #include "kd_sweep.cuh"
 
 #ifndef KD_SWEEP_VARIANT
@@ -15,14 +15,23 @@ cudaError_t launch_sweep_f32_v(int axis, int shape, int logn, const SweepArgs& a
 template cudaError_t launch_sweep_f32_v<KD_SWEEP_VARIANT>(int, int, int, const SweepArgs&, cudaStream_t);
 
 #if KD_SWEEP_VARIANT == 0
-cudaError_t launch_sweep_f32(int variant, int axis, int shape, int logn, const SweepArgs& a,
+// the others are instantiated in their own objects
+extern template cudaError_t launch_sweep_f32_v<1>(int, int, int, const SweepArgs&, cudaStream_t);
+extern template cudaError_t launch_sweep_f32_v<2>(int, int, int, const SweepArgs&, cudaStream_t);
+extern template cudaError_t launch_sweep_f32_v<3>(int, int, int, const SweepArgs&, cudaStream_t);
+extern template cudaError_t launch_sweep_f32_v<kFormSmall>(int, int, int, const SweepArgs&, cudaStream_t);
+extern template cudaError_t launch_sweep_f32_v<kFormLarge>(int, int, int, const SweepArgs&, cudaStream_t);
+
+cudaError_t launch_sweep_f32(int form, int axis, int shape, int logn, const SweepArgs& a,
                              cudaStream_t s) {
-    static_assert(kNumSweepVariants == 4, "one case per compiled variant");
-    switch (variant) {
+    static_assert(kNumSweepVariants == 4 && kNumSweepForms == 6, "one case per compiled form");
+    switch (form) {
         case 0: return launch_sweep_f32_v<0>(axis, shape, logn, a, s);
         case 1: return launch_sweep_f32_v<1>(axis, shape, logn, a, s);
         case 2: return launch_sweep_f32_v<2>(axis, shape, logn, a, s);
         case 3: return launch_sweep_f32_v<3>(axis, shape, logn, a, s);
+        case kFormSmall: return launch_sweep_f32_v<kFormSmall>(axis, shape, logn, a, s);
+        case kFormLarge: return launch_sweep_f32_v<kFormLarge>(axis, shape, logn, a, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -1,0 +1,69 @@
+"""The FP32 sweeps' compiled forms by grid size (small, both pairs per thread, large): the
+default variant on either side of every line of the rule, each against the oracle and, bit for
+bit, against variant 1 and a repeated run."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2307_01571_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def kd():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2307_01571_gb300 import _build
+    _build.build()
+    from paper_2307_01571_gb300 import kd as mod
+    return mod
+
+
+# two steps of FP32 rounding (2^-24 a rounding, ~20 of them a stage and point, growing as their
+# square root): 5e-6 of max |psi| is ten times the FP32 form's measured 5.7e-7 after four steps
+TOL = 5e-6
+
+
+@pytest.mark.parametrize("nx,ny", [
+    (4, 4096), (4096, 4), (4096, 16), (16, 4096),            # longest axes, fewest lines
+    (128, 128), (512, 128), (512, 256), (512, 512),          # y lines at 2^16 and 2^17 points
+    (2048, 64), (2048, 128), (4096, 64), (4096, 128),        # x: small / both pairs
+    (64, 1024), (128, 1024), (256, 1024), (512, 1024),       # y: small / one pair / large
+    (128, 2048), (256, 2048)])
+def test_default_form_matches_oracle(kd, nx, ny):
+    wl = W.small(nx, ny, W.GAUSS, units=W.ATOMIC, nsteps=2, a0=0.4)
+    u, g, f = wl.units, wl.grid, wl.field
+    psi = W.random_spinor(nx, ny, nx + 3 * ny).astype(np.complex64)
+    ref = oracle.step(u, g, f, psi.astype(np.complex128), 0.0, wl.dt, 2)
+    out = []
+    for v in ((0, 0), (1, 1), (0, 0)):
+        with kd.Sim(u, g, f, kd.KD_FP32) as sim:
+            sim.sweep_variants = v
+            sim.set_spinor(psi)
+            sim.step(wl.dt, 2)
+            out.append(sim.get_spinor())
+    assert np.max(np.abs(out[0] - ref)) <= TOL * np.max(np.abs(ref))
+    assert np.array_equal(out[0], out[1]) and np.array_equal(out[0], out[2])
+
+
+def test_large_forms_keep_a_plane_wave(kd):
+    """2048 x 2048 points (the large form on both axes, beyond the oracle): a positive-energy
+    plane wave is an eigenstate of every free step, psi(n) = psi(0) exp(-i (E - v p_y) n dt)."""
+    wl = W.small(2048, 2048, W.NONE, units=W.ATOMIC, nsteps=20)
+    u, g, f = wl.units, wl.grid, wl.field
+    kx, ky = 37, -21
+    px = 2 * np.pi * kx / (g.x_max - g.x_min)
+    py = 2 * np.pi * ky / (g.y_max - g.y_min)
+    pix, piy = px + f.p_shift_x, py + f.p_shift_y
+    spin = oracle.spinor_u(u, pix, piy, 1)
+    ph = np.exp(2j * np.pi * (kx * np.arange(2048)[None, :] / 2048 + ky * np.arange(2048)[:, None] / 2048))
+    psi = (ph[:, :, None] * spin).astype(np.complex64)
+    with kd.Sim(u, g, f, kd.KD_FP32) as sim:
+        sim.set_spinor(psi)
+        sim.step(wl.dt, 20)
+        got = sim.get_spinor()
+    E = np.sqrt(u.mc2 ** 2 + u.c ** 2 * (pix ** 2 + piy ** 2))
+    ref = psi * np.exp(-1j * (E - f.box_vy * py) * 20 * wl.dt)
+    assert np.max(np.abs(got - ref)) <= 2e-5 * np.max(np.abs(ref))
