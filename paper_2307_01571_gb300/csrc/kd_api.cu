@@ -212,19 +212,46 @@ __global__ void k_ktab(T* out, int nx, int ny, double dpx, double dpy, double sh
     const double G = sqrt(gm * gm + gx * gx + gy * gy);
     const float a0 = (float)a, b0 = (float)b;
     const double ang0 = atan2(P * b * E / c, 1.0 + P * a);
+    float av[7], bv[7];
+    double xv[7], yv[7];
+    av[3] = a0;
+    bv[3] = b0;
+#pragma unroll
+    for (int k = 2; k >= 0; --k) {
+        av[k] = nextafterf(av[k + 1], -INFINITY);
+        bv[k] = nextafterf(bv[k + 1], -INFINITY);
+        av[6 - k] = nextafterf(av[5 - k], INFINITY);
+        bv[6 - k] = nextafterf(bv[5 - k], INFINITY);
+    }
+#pragma unroll
+    for (int k = 0; k < 7; ++k) {
+        xv[k] = 1.0 + P * (double)av[k];
+        yv[k] = P * (double)bv[k] * G;
+    }
+    // The angle term needs an FP64 atan2 (49 of them made this kernel 2.5 ms at 1024x512 and
+    // 40 at 4096x2048, several times the steps of a short first call; now 0.9 and 15).  It is not negative, so
+    // a pair whose modulus term alone exceeds the whole measure of any one pair cannot win:
+    // with the pair of smallest modulus term as that bound a handful of the 49 remain.
+    double um = 1e300, xm = 1.0, ym = 0.0;
+#pragma unroll
+    for (int p = 0; p < 7; ++p)
+#pragma unroll
+        for (int q = 0; q < 7; ++q) {
+            const double u = fabs(fma(xv[p], xv[p], yv[q] * yv[q]) - 1.0);
+            if (u < um) { um = u; xm = xv[p]; ym = yv[q]; }
+        }
+    const double bound = um + 1e-3 * fabs(atan2(ym, xm) - ang0);
     float ba = a0, bb = b0;
     double best = 1e300;
-    float ai = a0;
-    for (int k = 0; k < 3; ++k) ai = nextafterf(ai, -INFINITY);
-    for (int da = -3; da <= 3; ++da, ai = nextafterf(ai, INFINITY)) {
-        float bi = b0;
-        for (int k = 0; k < 3; ++k) bi = nextafterf(bi, -INFINITY);
-        for (int db = -3; db <= 3; ++db, bi = nextafterf(bi, INFINITY)) {
-            const double x = 1.0 + P * (double)ai, y = P * (double)bi * G;
-            const double g = fabs(x * x + y * y - 1.0) + 1e-3 * fabs(atan2(y, x) - ang0);
-            if (g < best) { best = g; ba = ai; bb = bi; }
+#pragma unroll
+    for (int p = 0; p < 7; ++p)
+#pragma unroll 1
+        for (int q = 0; q < 7; ++q) {
+            const double u = fabs(fma(xv[p], xv[p], yv[q] * yv[q]) - 1.0);
+            if (u > bound) continue;
+            const double g = u + 1e-3 * fabs(atan2(yv[q], xv[p]) - ang0);
+            if (g < best) { best = g; ba = av[p]; bb = bv[q]; }
         }
-    }
     out[2 * i] = (T)ba;
     out[2 * i + 1] = (T)bb;
 }
@@ -809,18 +836,32 @@ template <typename T> void unit_phase(double ph, T* fx, T* fy) {
     *fx = (T)x;
     *fy = (T)y;
     if (sizeof(T) != 4) return;
-    double best = 1e300;
-    float xi = (float)x;
-    for (int k = 0; k < 3; ++k) xi = nextafterf(xi, -INFINITY);
-    for (int dx = -3; dx <= 3; ++dx, xi = nextafterf(xi, INFINITY)) {
-        float yi = (float)y;
-        for (int k = 0; k < 3; ++k) yi = nextafterf(yi, -INFINITY);
-        for (int dy = -3; dy <= 3; ++dy, yi = nextafterf(yi, INFINITY)) {
-            const double g = fabs(2.0 * xi + (double)xi * xi + (double)yi * yi) +
-                             1e-3 * fabs(atan2((double)yi, 1.0 + xi) - ph);
-            if (g < best) { best = g; *fx = (T)xi; *fy = (T)yi; }
-        }
+    // as in k_ktab: the angle of those pairs only whose modulus term does not exceed the
+    // whole measure of the pair with the smallest one
+    float xv[7], yv[7];
+    xv[3] = (float)x;
+    yv[3] = (float)y;
+    for (int k = 2; k >= 0; --k) {
+        xv[k] = nextafterf(xv[k + 1], -INFINITY);
+        yv[k] = nextafterf(yv[k + 1], -INFINITY);
+        xv[6 - k] = nextafterf(xv[5 - k], INFINITY);
+        yv[6 - k] = nextafterf(yv[5 - k], INFINITY);
     }
+    auto modulus = [](double xi, double yi) { return fabs(2.0 * xi + xi * xi + yi * yi); };
+    auto angle = [&](float xi, float yi) { return 1e-3 * fabs(atan2((double)yi, 1.0 + xi) - ph); };
+    int pm = 3, qm = 3;
+    for (int p = 0; p < 7; ++p)
+        for (int q = 0; q < 7; ++q)
+            if (modulus(xv[p], yv[q]) < modulus(xv[pm], yv[qm])) { pm = p; qm = q; }
+    const double bound = modulus(xv[pm], yv[qm]) + angle(xv[pm], yv[qm]);
+    double best = 1e300;
+    for (int p = 0; p < 7; ++p)
+        for (int q = 0; q < 7; ++q) {
+            const double u = modulus(xv[p], yv[q]);
+            if (u > bound) continue;
+            const double g = u + angle(xv[p], yv[q]);
+            if (g < best) { best = g; *fx = (T)xv[p]; *fy = (T)yv[q]; }
+        }
 }
 
 // Tables that depend on dt: the per-row (pi_y, cos(phi) - 1, sin(phi)) of the frame phase
