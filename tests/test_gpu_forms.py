@@ -67,3 +67,34 @@ def test_large_forms_keep_a_plane_wave(kd):
     E = np.sqrt(u.mc2 ** 2 + u.c ** 2 * (pix ** 2 + piy ** 2))
     ref = psi * np.exp(-1j * (E - f.box_vy * py) * 20 * wl.dt)
     assert np.max(np.abs(got - ref)) <= 2e-5 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64", "dw"])
+def test_runs_from_new_states_and_times_replay_the_same_steps(kd, prec):
+    """The step graphs outlive a new time or packet (nothing captured depends on them): every
+    run on a used handle equals the same run on a fresh one, with read-outs whose windows and
+    basis change in between."""
+    wl = W.small(64, 128, W.GAUSS, units=W.ATOMIC, a0=0.3)
+    u, g, f = wl.units, wl.grid, wl.field
+    p2 = W.Packet(1.5 * wl.packet.p0x, wl.packet.p0y, 0.1 * g.x_max, 0.2 * g.y_max, wl.packet.sigma_p, -1, 1)
+    prec = {"fp32": kd.KD_FP32, "fp64": kd.KD_FP64, "dw": kd.KD_DW}[prec]
+
+    def run(sim, k):
+        if k == 2:
+            sim.set_spinor(W.random_spinor(64, 128, 3))
+            sim.set_time(1.7 * wl.dt)
+        else:
+            sim.init_packet(wl.packet if k == 0 else p2)
+        obs = sim.step(wl.dt, 12, obs_every=4)
+        obs += sim.step(wl.dt, 6)
+        return sim.get_spinor(), obs, sim.get_time()
+
+    with kd.Sim(u, g, f, prec) as used:
+        for k in (0, 1, 0, 2, 1, 2):
+            psi, obs, t = run(used, k)
+            with kd.Sim(u, g, f, prec) as fresh:
+                if k == 2:
+                    fresh.init_packet(p2 if np.isclose(spec_basis, 1) else wl.packet)   # the read-out spec
+                ref, ref_obs, ref_t = run(fresh, k)
+            spec_basis = 1 if k == 1 else (0 if k == 0 else spec_basis)
+            assert np.array_equal(psi, ref) and obs == ref_obs and t == ref_t
