@@ -115,6 +115,7 @@ struct kd_sim {
     void* work = nullptr;
     void* tw[2][3] = {};   // twiddle tables [axis][loge - 2] (radix-4, radix-8, FP32: radix-16)
     int var[2] = {0, 0};   // sweep launch variant per axis (kd_autotune)
+    bool crowded = false;  // while a batch that fills the SMs enqueues this simulation's work
     void* xtab = nullptr;
     void* kxtab = nullptr;
     void* kytab = nullptr;
@@ -917,8 +918,8 @@ int build_dt_tables(kd_sim* s, double dt) {
 
 // The compiled form of the FP32 sweeps that the simulation's launch variant runs on its grid
 int form(const kd_sim* s, int axis) {
-    return axis == AXIS_X ? sweep_form_of(axis, s->var[axis], s->lx, s->g.ny)
-                          : sweep_form_of(axis, s->var[axis], s->ly, s->g.nx);
+    return axis == AXIS_X ? sweep_form_of(axis, s->var[axis], s->lx, s->g.ny, s->crowded)
+                          : sweep_form_of(axis, s->var[axis], s->ly, s->g.nx, s->crowded);
 }
 
 // One fused sweep of the state (the simulation's own form), or, with view = true, an FP64
@@ -1801,6 +1802,7 @@ struct kd_batch {
     cudaEvent_t fork = nullptr;
     std::vector<cudaEvent_t> join;
     int device = 0;
+    bool crowded = false;            // the members together fill the SMs (sweep_form_of)
     // one graph per chunk shape: all simulations' chunks as concurrent branches
     std::map<GraphKey, std::pair<cudaGraphExec_t, std::vector<int64_t>>> graphs;
     std::vector<uint64_t> gens;      // simulations' graph generations the graphs were built on
@@ -1930,7 +1932,9 @@ template <typename F> int fork_join(kd_batch* b, cudaStream_t origin, F fn) {
         KD_CUDA(cudaStreamWaitEvent(s->cap_stream, b->fork, 0));
         cudaStream_t saved = s->stream;
         s->stream = s->cap_stream;
+        s->crowded = b->crowded;
         int rc = fn(s, i);
+        s->crowded = false;
         s->stream = saved;
         if (rc) return rc;
         KD_CUDA(cudaEventRecord(b->join[i], s->cap_stream));
@@ -1961,6 +1965,9 @@ int kd_batch_create(kd_sim* const* sims, int32_t n, void* cuda_stream, kd_batch*
     b->stream = (cudaStream_t)cuda_stream;
     b->device = dev;
     b->join.assign(n, nullptr);
+    size_t points = 0;
+    for (const kd_sim* s : b->sims) points += s->P;
+    b->crowded = n > 1 && points > ((size_t)1 << 18);
     bool ok = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) == cudaSuccess &&
               cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess;
     for (int32_t i = 0; ok && i < n; ++i)
@@ -1970,6 +1977,22 @@ int kd_batch_create(kd_sim* const* sims, int32_t n, void* cuda_stream, kd_batch*
         return fail(KD_ERR_CUDA, "stream/event creation failed");
     }
     b->gens.assign(n, ~0ull);
+    if (b->crowded) {   // first launches of the forms that only a crowded batch runs, once per shape
+        std::map<std::pair<int, int>, int> seen;
+        for (kd_sim* s : b->sims) {
+            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+            if (s->prec == KD_FP64 || seen[{s->lx, s->ly}]++ || cudaStreamIsCapturing(s->stream, &cs) != cudaSuccess ||
+                cs != cudaStreamCaptureStatusNone)
+                continue;
+            s->crowded = true;
+            int rc = warm_variants(s);
+            s->crowded = false;
+            if (rc) {
+                kd_batch_destroy(b);
+                return rc;
+            }
+        }
+    }
     *out = b;
     return KD_OK;
 }

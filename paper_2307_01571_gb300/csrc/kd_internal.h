@@ -140,8 +140,14 @@ __host__ __device__ constexpr bool sweep_form_holds(int form, int logn) {
 //   y from 1024 points (few columns): small up to 2^17 points (128x1024 15.6 : 7.0, 64x2048
 //     18.7 : 10.1), one pair per CTA at 2^18 (256x1024 15.8 : 9.8, 128x2048 18.8 : 11.2),
 //     then large (1024x1024 30.7 : 29.5, 2048x1024 61.6 : 54.6, 4096x2048 292 : 263).
-inline int sweep_form_of(int axis, int v, int logn, int lines) {
+// crowded: other simulations run beside this one and fill the SMs (a batch).  The small
+// form's narrow column tiles, which spread one small grid over the SMs, then only cost memory
+// transactions: the wide radix-4 tiles of variant 2 take their place.  They differ from the
+// small form in threads and components per CTA alone, so a member still equals itself run
+// alone, bit for bit.  16 members of 128x128 ... 512x256: 20.5 against 22.6 G point-steps/s.
+inline int sweep_form_of(int axis, int v, int logn, int lines, bool crowded) {
     if (v > 1) return v;
+    if (crowded && axis == AXIS_Y && logn <= 9 && ((long long)lines << logn) <= 1 << 16) return 2;
     const long long points = (long long)lines << logn;
     if (axis == AXIS_X) {
         if (logn <= 11 && points <= 1 << 17) return kFormSmall;

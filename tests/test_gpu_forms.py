@@ -69,6 +69,29 @@ def test_large_forms_keep_a_plane_wave(kd):
     assert np.max(np.abs(got - ref)) <= 2e-5 * np.max(np.abs(ref))
 
 
+def test_members_of_a_crowded_batch_equal_members_alone(kd):
+    """Together the members fill the SMs (2^18 points and more), so their small column sweeps
+    run wide tiles; each still equals itself run alone, bit for bit."""
+    shapes = [(128, 128), (256, 128), (256, 256), (64, 512), (512, 64), (32, 32), (256, 256), (128, 256)]
+    wls = [W.small(nx, ny, W.GAUSS, units=W.ATOMIC, a0=0.05 * (i + 1)).with_(precision=1)
+           for i, (nx, ny) in enumerate(shapes * 2)]
+    assert sum(w.points for w in wls) > 1 << 18
+    alone = []
+    for wl in wls:
+        with kd.Sim.from_workload(wl) as sim:
+            sim.init_packet(wl.packet)
+            obs = sim.step(wl.dt, 30, obs_every=10)
+            alone.append((sim.get_spinor(), obs))
+    sims = [kd.Sim.from_workload(wl) for wl in wls]
+    for s, wl in zip(sims, wls):
+        s.init_packet(wl.packet)
+    with kd.Batch(sims) as b:
+        obs = b.step([wl.dt for wl in wls], 30, obs_every=10)
+    for s, o, (ref, ref_obs) in zip(sims, obs, alone):
+        assert np.array_equal(s.get_spinor(), ref) and o == ref_obs
+        s.close()
+
+
 @pytest.mark.parametrize("prec", ["fp32", "fp64", "dw"])
 def test_runs_from_new_states_and_times_replay_the_same_steps(kd, prec):
     """The step graphs outlive a new time or packet (nothing captured depends on them): every
