@@ -21,11 +21,43 @@
 
 namespace kd {
 
-struct DW {
-    float h, l;
-};
-
 #define KD_DWI __host__ __device__ __forceinline__
+
+// Two floats in one 64-bit register pair, operated on by the packed FP32 instructions
+// (add / mul / fma .rn.f32x2): one issue slot for two operations at the pipe's full rate
+// (79 TFLOP/s either way, measured on FMA chains; with an integer operation beside every
+// FMA 45 against 31), each lane rounded exactly as the scalar instruction.  The double-word
+// sweeps hold a pair's two spinor components in the lanes: their long chains of dependent
+// operations then take half the issue slots and half the code (the scalar form stalled on
+// instruction fetch).  x sweep, us: 2048x1024 370 -> 297, 2048x128 51.5 -> 44.8, 1024x512
+// 74.0 -> 71.4; y 62.1 -> 59.7.  What bounds them now is the FP32 pipe (44 of 71 us at
+// 1024x512).  The FP32 form gains nothing from it: its twiddles have to be duplicated into
+// both lanes for only eight packed operations each (1024x512 13.2 -> 13.5 us).
+struct F2 {
+    float2 v;
+};
+#ifdef __CUDACC__
+__device__ __forceinline__ F2 dup2(float a) { return F2{make_float2(a, a)}; }
+__device__ __forceinline__ F2 pair2(float a, float b) { return F2{make_float2(a, b)}; }
+__device__ __forceinline__ F2 swap2(F2 a) { return F2{make_float2(a.v.y, a.v.x)}; }
+__device__ __forceinline__ F2 operator-(F2 a) { return F2{make_float2(-a.v.x, -a.v.y)}; }
+__device__ __forceinline__ F2 f_add(F2 a, F2 b) { return F2{__fadd2_rn(a.v, b.v)}; }
+__device__ __forceinline__ F2 f_sub(F2 a, F2 b) { return F2{__fadd2_rn(a.v, (-b).v)}; }
+__device__ __forceinline__ F2 f_mul(F2 a, F2 b) { return F2{__fmul2_rn(a.v, b.v)}; }
+__device__ __forceinline__ F2 f_fma(F2 a, F2 b, F2 c) { return F2{__ffma2_rn(a.v, b.v, c.v)}; }
+__device__ __forceinline__ F2 operator+(F2 a, F2 b) { return f_add(a, b); }
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) { return f_sub(a, b); }
+__device__ __forceinline__ F2 operator*(F2 a, F2 b) { return f_mul(a, b); }
+// sign factor +-1 (the FFT direction) times x: exact
+__device__ __forceinline__ F2 operator*(int sgn, F2 x) { return sgn > 0 ? x : -x; }
+#endif
+
+// A double-word real, or (L = F2) two of them, one per lane
+template <typename L> struct DWT {
+    L h, l;
+};
+using DW = DWT<float>;
+using DW2 = DWT<F2>;
 
 #ifdef __CUDA_ARCH__
 KD_DWI float f_add(float a, float b) { return __fadd_rn(a, b); }
@@ -39,19 +71,19 @@ KD_DWI float f_mul(float a, float b) { volatile float s = a * b; return s; }
 KD_DWI float f_fma(float a, float b, float c) { return fmaf(a, b, c); }
 #endif
 
-KD_DWI DW two_sum(float a, float b) {
-    const float s = f_add(a, b);
-    const float bb = f_sub(s, a);
-    const float e = f_add(f_sub(a, f_sub(s, bb)), f_sub(b, bb));
-    return DW{s, e};
+template <typename L> KD_DWI DWT<L> two_sum(L a, L b) {
+    const L s = f_add(a, b);
+    const L bb = f_sub(s, a);
+    const L e = f_add(f_sub(a, f_sub(s, bb)), f_sub(b, bb));
+    return DWT<L>{s, e};
 }
-KD_DWI DW fast_two_sum(float a, float b) {   // |a| >= |b| or a == 0
-    const float s = f_add(a, b);
-    return DW{s, f_sub(b, f_sub(s, a))};
+template <typename L> KD_DWI DWT<L> fast_two_sum(L a, L b) {   // |a| >= |b| or a == 0
+    const L s = f_add(a, b);
+    return DWT<L>{s, f_sub(b, f_sub(s, a))};
 }
-KD_DWI DW two_prod(float a, float b) {
-    const float p = f_mul(a, b);
-    return DW{p, f_fma(a, b, -p)};
+template <typename L> KD_DWI DWT<L> two_prod(L a, L b) {
+    const L p = f_mul(a, b);
+    return DWT<L>{p, f_fma(a, b, -p)};
 }
 
 KD_DWI DW dw(float a) { return DW{a, 0.0f}; }
@@ -63,29 +95,29 @@ KD_DWI float pow2_neg(int m) {
     return ldexpf(1.0f, -m);
 #endif
 }
-KD_DWI DW dw_neg(DW x) { return DW{-x.h, -x.l}; }
+template <typename L> KD_DWI DWT<L> dw_neg(DWT<L> x) { return DWT<L>{-x.h, -x.l}; }
 // x * 2^k for a power-of-two float p (exact)
-KD_DWI DW dw_scale(DW x, float p) { return DW{x.h * p, x.l * p}; }
+template <typename L> KD_DWI DWT<L> dw_scale(DWT<L> x, L p) { return DWT<L>{x.h * p, x.l * p}; }
 
 // x + y (sloppy double-word sum): absolute error <= ~2^-47 (|x| + |y|)
-KD_DWI DW dw_add(DW x, DW y) {
-    const DW s = two_sum(x.h, y.h);
-    const float v = f_add(x.l, y.l);
-    const float w = f_add(s.l, v);
+template <typename L> KD_DWI DWT<L> dw_add(DWT<L> x, DWT<L> y) {
+    const DWT<L> s = two_sum(x.h, y.h);
+    const L v = f_add(x.l, y.l);
+    const L w = f_add(s.l, v);
     return fast_two_sum(s.h, w);
 }
-KD_DWI DW dw_sub(DW x, DW y) { return dw_add(x, dw_neg(y)); }
+template <typename L> KD_DWI DWT<L> dw_sub(DWT<L> x, DWT<L> y) { return dw_add(x, dw_neg(y)); }
 // Lazy sums for a butterfly's first level: x + y as (h, l) with h = fl(x.h + y.h) exact to
 // its TwoSum error and l = that error plus both low parts, not renormalised (|l| may exceed
 // half an ulp of h).  dw_add_lazy then adds two such pairs and renormalises once: the
 // result has the sloppy double-word sum's absolute error bound (a few 2^-48 of the summed
 // magnitudes) with one Fast2Sum instead of three.
-KD_DWI DW dw_add_part(DW x, DW y) {
-    const DW s = two_sum(x.h, y.h);
-    return DW{s.h, f_add(s.l, f_add(x.l, y.l))};
+template <typename L> KD_DWI DWT<L> dw_add_part(DWT<L> x, DWT<L> y) {
+    const DWT<L> s = two_sum(x.h, y.h);
+    return DWT<L>{s.h, f_add(s.l, f_add(x.l, y.l))};
 }
-KD_DWI DW dw_add_lazy(DW x, DW y) {
-    const DW s = two_sum(x.h, y.h);
+template <typename L> KD_DWI DWT<L> dw_add_lazy(DWT<L> x, DWT<L> y) {
+    const DWT<L> s = two_sum(x.h, y.h);
     return fast_two_sum(s.h, f_add(s.l, f_add(x.l, y.l)));
 }
 // x + y with y a float
@@ -94,9 +126,9 @@ KD_DWI DW dw_add_f(DW x, float y) {
     return fast_two_sum(s.h, f_add(s.l, x.l));
 }
 // x * y, both double-words (FMA form): relative error <= ~5 2^-48
-KD_DWI DW dw_mul(DW x, DW y) {
-    const DW c = two_prod(x.h, y.h);
-    const float t = f_fma(x.l, y.h, f_mul(x.h, y.l));
+template <typename L> KD_DWI DWT<L> dw_mul(DWT<L> x, DWT<L> y) {
+    const DWT<L> c = two_prod(x.h, y.h);
+    const L t = f_fma(x.l, y.h, f_mul(x.h, y.l));
     return fast_two_sum(c.h, f_add(c.l, t));
 }
 // x * y with y a float: relative error <= ~2 2^-48
@@ -106,11 +138,11 @@ KD_DWI DW dw_mul_f(DW x, float y) {
 }
 // a x + b y as one double-word (the real part of a complex product): the two leading
 // products exactly, their sum by TwoSum, every small term gathered in one float
-KD_DWI DW dw_dot2(DW a, DW x, DW b, DW y) {
-    const DW p = two_prod(a.h, x.h);
-    const DW q = two_prod(b.h, y.h);
-    const DW s = two_sum(p.h, q.h);
-    float t = f_add(p.l, q.l);
+template <typename L> KD_DWI DWT<L> dw_dot2(DWT<L> a, DWT<L> x, DWT<L> b, DWT<L> y) {
+    const DWT<L> p = two_prod(a.h, x.h);
+    const DWT<L> q = two_prod(b.h, y.h);
+    const DWT<L> s = two_sum(p.h, q.h);
+    L t = f_add(p.l, q.l);
     t = f_add(t, s.l);
     t = f_fma(a.h, x.l, t);
     t = f_fma(a.l, x.h, t);
@@ -122,17 +154,17 @@ KD_DWI DW dw_dot2(DW a, DW x, DW b, DW y) {
 // The same dot product without the final renormalisation (|l| may exceed half an ulp of
 // h): for values that go straight into a butterfly's first level (dw_add_part / dw_add),
 // whose TwoSum of the high parts is exact whatever the low parts are
-KD_DWI DW dw_dot2_part(DW a, DW x, DW b, DW y) {
-    const DW p = two_prod(a.h, x.h);
-    const DW q = two_prod(b.h, y.h);
-    const DW s = two_sum(p.h, q.h);
-    float t = f_add(p.l, q.l);
+template <typename L> KD_DWI DWT<L> dw_dot2_part(DWT<L> a, DWT<L> x, DWT<L> b, DWT<L> y) {
+    const DWT<L> p = two_prod(a.h, x.h);
+    const DWT<L> q = two_prod(b.h, y.h);
+    const DWT<L> s = two_sum(p.h, q.h);
+    L t = f_add(p.l, q.l);
     t = f_add(t, s.l);
     t = f_fma(a.h, x.l, t);
     t = f_fma(a.l, x.h, t);
     t = f_fma(b.h, y.l, t);
     t = f_fma(b.l, y.h, t);
-    return DW{s.h, t};
+    return DWT<L>{s.h, t};
 }
 
 // Splits a double into the nearest double-word (exact for the 48 leading bits); host or
@@ -144,12 +176,12 @@ KD_DWI DW dw_from_double(double d) {
 }
 KD_DWI double dw_to_double(DW x) { return (double)x.h + (double)x.l; }
 
-KD_DWI DW operator+(DW x, DW y) { return dw_add(x, y); }
-KD_DWI DW operator-(DW x, DW y) { return dw_sub(x, y); }
-KD_DWI DW operator-(DW x) { return dw_neg(x); }
-KD_DWI DW operator*(DW x, DW y) { return dw_mul(x, y); }
+template <typename L> KD_DWI DWT<L> operator+(DWT<L> x, DWT<L> y) { return dw_add(x, y); }
+template <typename L> KD_DWI DWT<L> operator-(DWT<L> x, DWT<L> y) { return dw_sub(x, y); }
+template <typename L> KD_DWI DWT<L> operator-(DWT<L> x) { return dw_neg(x); }
+template <typename L> KD_DWI DWT<L> operator*(DWT<L> x, DWT<L> y) { return dw_mul(x, y); }
 // sign factor +-1 (the FFT direction) times x: exact
-KD_DWI DW operator*(int sgn, DW x) { return sgn > 0 ? x : dw_neg(x); }
+template <typename L> KD_DWI DWT<L> operator*(int sgn, DWT<L> x) { return sgn > 0 ? x : dw_neg(x); }
 
 // sqrt(x) for x >= 0: float seed and one correction, relative error ~2^-47
 KD_DWI DW dw_sqrt(DW x) {
@@ -230,22 +262,28 @@ KD_DWI void dw_sincos(DW th, const DWConst* K, DW* sn, DW* cs) {
 
 // ------------------------------------------------------------ complex double-word -
 // members named x, y like float2/double2, so the FFT engine's generic complex code applies
-struct DWC {
-    DW x, y;
+template <typename L> struct DWCT {
+    DWT<L> x, y;
 };
-KD_DWI DWC dwc(DW re, DW im) { return DWC{re, im}; }
-KD_DWI DWC dwc_add(DWC a, DWC b) { return DWC{dw_add(a.x, b.x), dw_add(a.y, b.y)}; }
-KD_DWI DWC dwc_sub(DWC a, DWC b) { return DWC{dw_sub(a.x, b.x), dw_sub(a.y, b.y)}; }
+using DW2C = DWCT<F2>;   // a pair's two components, one per lane
+template <typename L> KD_DWI DWCT<L> dwc_add(DWCT<L> a, DWCT<L> b) { return DWCT<L>{dw_add(a.x, b.x), dw_add(a.y, b.y)}; }
 // a * w, w = (c, s): (a.x c - a.y s, a.x s + a.y c)
-KD_DWI DWC dwc_mul(DWC a, DWC w) {
-    return DWC{dw_dot2(a.x, w.x, dw_neg(a.y), w.y), dw_dot2(a.x, w.y, a.y, w.x)};
+template <typename L> KD_DWI DWCT<L> dwc_mul(DWCT<L> a, DWCT<L> w) {
+    return DWCT<L>{dw_dot2(a.x, w.x, dw_neg(a.y), w.y), dw_dot2(a.x, w.y, a.y, w.x)};
 }
 // a * w unnormalised (dw_dot2_part): the FFT's twiddle products, which feed the next
 // butterfly directly
-KD_DWI DWC dwc_mul_part(DWC a, DWC w) {
-    return DWC{dw_dot2_part(a.x, w.x, dw_neg(a.y), w.y), dw_dot2_part(a.x, w.y, a.y, w.x)};
+template <typename L> KD_DWI DWCT<L> dwc_mul_part(DWCT<L> a, DWCT<L> w) {
+    return DWCT<L>{dw_dot2_part(a.x, w.x, dw_neg(a.y), w.y), dw_dot2_part(a.x, w.y, a.y, w.x)};
 }
 // a * r for a real double-word r
-KD_DWI DWC dwc_mul_r(DWC a, DW r) { return DWC{dw_mul(a.x, r), dw_mul(a.y, r)}; }
+template <typename L> KD_DWI DWCT<L> dwc_mul_r(DWCT<L> a, DWT<L> r) { return DWCT<L>{dw_mul(a.x, r), dw_mul(a.y, r)}; }
+
+#ifdef __CUDACC__
+// both lanes the same double-word; the lanes exchanged; (x, -x)
+__device__ __forceinline__ DW2 dup2(DW x) { return DW2{dup2(x.h), dup2(x.l)}; }
+__device__ __forceinline__ DW2 swap2(DW2 x) { return DW2{swap2(x.h), swap2(x.l)}; }
+__device__ __forceinline__ DW2 alt2(DW x) { return DW2{pair2(x.h, -x.h), pair2(x.l, -x.l)}; }
+#endif
 
 }  // namespace kd

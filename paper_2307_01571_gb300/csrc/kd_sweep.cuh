@@ -31,10 +31,12 @@ namespace kd {
 
 #define KD_DI __device__ __forceinline__
 
+// What a thread holds of a point: complex components, or (double-word) a pair's two
+// components in the lanes of packed reals.  tab: the kinetic table's (a, b) entry.
 template <typename T> struct Cx;
-template <> struct Cx<float> { using t = float2; };
-template <> struct Cx<double> { using t = double2; };
-template <> struct Cx<DW> { using t = DWC; };
+template <> struct Cx<float> { using t = float2; using tab = float2; };
+template <> struct Cx<double> { using t = double2; using tab = double2; };
+template <> struct Cx<DW> { using t = DW2C; using tab = float4; };
 
 template <typename C> KD_DI C mk(decltype(C::x) a, decltype(C::x) b) { C r; r.x = a; r.y = b; return r; }
 template <typename C> KD_DI C cadd(C a, C b) { return mk<C>(a.x + b.x, a.y + b.y); }
@@ -68,25 +70,25 @@ template <int DIR, int S, typename C> KD_DI void dft4(C* a) {
 
 // The same four-point DFT on double-word values: the first level's sums and differences
 // stay unnormalised (dw_add_part) and each output renormalises once (dw_add_lazy)
-template <int DIR, int S> KD_DI void dft4(DWC* a) {
-    const DW s02x = dw_add_part(a[0].x, a[2 * S].x), s02y = dw_add_part(a[0].y, a[2 * S].y);
-    const DW d02x = dw_add_part(a[0].x, dw_neg(a[2 * S].x)), d02y = dw_add_part(a[0].y, dw_neg(a[2 * S].y));
-    const DW s13x = dw_add_part(a[S].x, a[3 * S].x), s13y = dw_add_part(a[S].y, a[3 * S].y);
-    const DW d13x = dw_add_part(a[S].x, dw_neg(a[3 * S].x)), d13y = dw_add_part(a[S].y, dw_neg(a[3 * S].y));
+template <int DIR, int S> KD_DI void dft4(DW2C* a) {
+    const DW2 s02x = dw_add_part(a[0].x, a[2 * S].x), s02y = dw_add_part(a[0].y, a[2 * S].y);
+    const DW2 d02x = dw_add_part(a[0].x, dw_neg(a[2 * S].x)), d02y = dw_add_part(a[0].y, dw_neg(a[2 * S].y));
+    const DW2 s13x = dw_add_part(a[S].x, a[3 * S].x), s13y = dw_add_part(a[S].y, a[3 * S].y);
+    const DW2 d13x = dw_add_part(a[S].x, dw_neg(a[3 * S].x)), d13y = dw_add_part(a[S].y, dw_neg(a[3 * S].y));
     // r = (DIR i) d13
-    const DW rx = DIR > 0 ? dw_neg(d13y) : d13y, ry = DIR > 0 ? d13x : dw_neg(d13x);
-    a[0] = DWC{dw_add_lazy(s02x, s13x), dw_add_lazy(s02y, s13y)};
-    a[2 * S] = DWC{dw_add_lazy(s02x, dw_neg(s13x)), dw_add_lazy(s02y, dw_neg(s13y))};
-    a[S] = DWC{dw_add_lazy(d02x, rx), dw_add_lazy(d02y, ry)};
-    a[3 * S] = DWC{dw_add_lazy(d02x, dw_neg(rx)), dw_add_lazy(d02y, dw_neg(ry))};
+    const DW2 rx = DIR > 0 ? dw_neg(d13y) : d13y, ry = DIR > 0 ? d13x : dw_neg(d13x);
+    a[0] = DW2C{dw_add_lazy(s02x, s13x), dw_add_lazy(s02y, s13y)};
+    a[2 * S] = DW2C{dw_add_lazy(s02x, dw_neg(s13x)), dw_add_lazy(s02y, dw_neg(s13y))};
+    a[S] = DW2C{dw_add_lazy(d02x, rx), dw_add_lazy(d02y, ry)};
+    a[3 * S] = DW2C{dw_add_lazy(d02x, dw_neg(rx)), dw_add_lazy(d02y, dw_neg(ry))};
 }
 
 // multiply by 1/sqrt(2) as a hi + lo pair: a single rounded constant would make every
 // radix-8 butterfly shrink the norm of two of its eight inputs by 2 h^2 - 1 (about 4e-8
 // in FP32), a bias that accumulates over thousands of steps
 template <typename T> KD_DI T mul_rsqrt2(T x) {
-    if constexpr (std::is_same<T, DW>::value) {
-        return dw_mul(x, DW{0.707106769f, 1.21016175e-08f});
+    if constexpr (std::is_same<T, DW2>::value) {
+        return dw_mul(x, dup2(DW{0.707106769f, 1.21016175e-08f}));
     } else if constexpr (sizeof(T) == 4) {
         return fmaf(x, 0.707106769084930419921875f, x * 1.2101617e-08f);
     } else {
@@ -253,6 +255,7 @@ template <typename T, int LOGN, int AXIS, int V> struct Cfg {
     static constexpr int CPP = F64 ? 1 : 2;                      // complex per 16-byte unit
     static constexpr int NPL = NC / CPP;                         // units per point in the CTA
     static constexpr int PPP = 2 / CPP;                          // units per point per pair
+    static constexpr int NR = DWT ? NC / 2 : NC;                 // register elements per point
     static constexpr int NPAIRS = SHARE ? 1 : 4 / NC;            // CTAs per line group
     static constexpr int NST = plan_nst(LOGN, LOGE);
     static constexpr int BUF_UNITS = PCTA * BATCH * NPL * N;     // one exchange buffer
@@ -294,22 +297,46 @@ template <int LA, int LB> __host__ __device__ constexpr int expand(int j) {
 }
 
 // ------------------------------------------------------- register <-> 16 B --------
+// Unit p of a point's register elements e: pack / unpack in the global layout (complex
+// components one after the other), spack / sunpack in shared memory, where the packed form
+// keeps its lanes together (no register moves).
 template <typename T> struct Unit;
 template <> struct Unit<float> {
     using U = float4;
-    KD_DI static U pack(const float2* c) { return make_float4(c[0].x, c[0].y, c[1].x, c[1].y); }
-    KD_DI static void unpack(U u, float2* c) { c[0] = make_float2(u.x, u.y); c[1] = make_float2(u.z, u.w); }
+    KD_DI static U pack(const float2* e, int p) { return make_float4(e[2 * p].x, e[2 * p].y, e[2 * p + 1].x, e[2 * p + 1].y); }
+    KD_DI static void unpack(U u, float2* e, int p) { e[2 * p] = make_float2(u.x, u.y); e[2 * p + 1] = make_float2(u.z, u.w); }
+    KD_DI static U spack(const float2* e, int p) { return pack(e, p); }
+    KD_DI static void sunpack(U u, float2* e, int p) { unpack(u, e, p); }
 };
 template <> struct Unit<double> {
     using U = double2;
-    KD_DI static U pack(const double2* c) { return c[0]; }
-    KD_DI static void unpack(U u, double2* c) { c[0] = u; }
+    KD_DI static U pack(const double2* e, int p) { return e[p]; }
+    KD_DI static void unpack(U u, double2* e, int p) { e[p] = u; }
+    KD_DI static U spack(const double2* e, int p) { return e[p]; }
+    KD_DI static void sunpack(U u, double2* e, int p) { e[p] = u; }
 };
-// double-word complex: (re.h, re.l, im.h, im.l), each real in the 8 bytes a double would take
+// double-word: in global memory each complex is (re.h, re.l, im.h, im.l), each real in the
+// 8 bytes a double would take
 template <> struct Unit<DW> {
     using U = float4;
-    KD_DI static U pack(const DWC* c) { return make_float4(c[0].x.h, c[0].x.l, c[0].y.h, c[0].y.l); }
-    KD_DI static void unpack(U u, DWC* c) { c[0] = DWC{DW{u.x, u.y}, DW{u.z, u.w}}; }
+    KD_DI static U pack(const DW2C* e, int p) {
+        const DW2C& c = e[p >> 1];
+        return p & 1 ? make_float4(c.x.h.v.y, c.x.l.v.y, c.y.h.v.y, c.y.l.v.y)
+                     : make_float4(c.x.h.v.x, c.x.l.v.x, c.y.h.v.x, c.y.l.v.x);
+    }
+    KD_DI static void unpack(U u, DW2C* e, int p) {
+        DW2C& c = e[p >> 1];
+        if (p & 1) { c.x.h.v.y = u.x; c.x.l.v.y = u.y; c.y.h.v.y = u.z; c.y.l.v.y = u.w; }
+        else { c.x.h.v.x = u.x; c.x.l.v.x = u.y; c.y.h.v.x = u.z; c.y.l.v.x = u.w; }
+    }
+    KD_DI static U spack(const DW2C* e, int p) {
+        const DW2& r = p & 1 ? e[p >> 1].y : e[p >> 1].x;
+        return make_float4(r.h.v.x, r.h.v.y, r.l.v.x, r.l.v.y);
+    }
+    KD_DI static void sunpack(U u, DW2C* e, int p) {
+        DW2& r = p & 1 ? e[p >> 1].y : e[p >> 1].x;
+        r = DW2{pair2(u.x, u.y), pair2(u.z, u.w)};
+    }
 };
 
 // ------------------------------------------------- double-word potential factor ---
@@ -373,10 +400,11 @@ static __device__ __noinline__ DWFactor dw_potential_factor(const void* xtab_, c
 template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
     using Cf = Cfg<T, LOGN, AXIS, V>;
     using C = typename Cx<T>::t;
+    using TabC = typename Cx<T>::tab;
     using U = typename Unit<T>::U;
     static constexpr int N = Cf::N, E = Cf::E, TF = Cf::TF, NC = Cf::NC, NST = Cf::NST;
     static constexpr bool DWF = std::is_same<T, DW>::value;   // double-word form
-    static constexpr int NPL = Cf::NPL, CPP = Cf::CPP, BATCH = Cf::BATCH;
+    static constexpr int NPL = Cf::NPL, NR = Cf::NR, BATCH = Cf::BATCH;
     // direction of the first and second FFT (forward = -1)
     static constexpr int DIR1 = AXIS == AXIS_X ? +1 : -1;
     static constexpr int DIR2 = -DIR1;
@@ -432,7 +460,7 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
                     // reused twiddle and field tables stay resident in L1
                     if (c.valid) u = __ldcg(g + unit_of(a, c, pt, p));
                     else u = U{};
-                    Unit<T>::unpack(u, v + (m * R + r) * NC + p * CPP);
+                    Unit<T>::unpack(u, v + (m * R + r) * NR, p);
                 }
             }
     }
@@ -447,7 +475,7 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
                 int idx = c.jt + m * TF + r * (N / R);
                 const long long pt = point_of(a, c.line, idx);
 #pragma unroll
-                for (int p = 0; p < NPL; ++p) __stcg(g + unit_of(a, c, pt, p), Unit<T>::pack(v + (m * R + r) * NC + p * CPP));
+                for (int p = 0; p < NPL; ++p) __stcg(g + unit_of(a, c, pt, p), Unit<T>::pack(v + (m * R + r) * NR, p));
             }
     }
 
@@ -459,7 +487,7 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
         constexpr int NS = 1 << LNS;
 #pragma unroll
         for (int m = 0; m < E / R; ++m) {
-            C* b = v + m * R * NC;
+            C* b = v + m * R * NR;
             if constexpr (LNS > 0) {
                 const int k = (c.jt + m * TF) & (NS - 1);
 #pragma unroll
@@ -472,11 +500,11 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
                         const float4 w4 = __ldg(reinterpret_cast<const float4*>(a.tw) + idx);
                         const float sh = DIR > 0 ? -w4.y : w4.y, sl = DIR > 0 ? -w4.w : w4.w;
 #pragma unroll
-                        for (int q = 0; q < NC; ++q) {
-                            const C x = b[r * NC + q];
+                        for (int q = 0; q < NR; ++q) {
+                            const C x = b[r * NR + q];
                             const float re = fmaf(x.x, w4.x, fmaf(-x.y, sh, fmaf(x.x, w4.z, -x.y * sl)));
                             const float im = fmaf(x.x, sh, fmaf(x.y, w4.x, fmaf(x.x, sl, x.y * w4.z)));
-                            b[r * NC + q] = mk<C>(re, im);
+                            b[r * NR + q] = mk<C>(re, im);
                         }
                     } else if constexpr (DWF) {
                         // double-word twiddle (c_hi, s_hi, c_lo, s_lo), unit modulus far
@@ -484,19 +512,19 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
                         // unnormalised into this stage's butterfly, whose first level adds
                         // their high parts exactly and renormalises
                         const float4 w4 = __ldg(reinterpret_cast<const float4*>(a.tw) + idx);
-                        const DWC w = DWC{DW{w4.x, w4.z}, DIR > 0 ? DW{-w4.y, -w4.w} : DW{w4.y, w4.w}};
+                        const C w = C{dup2(DW{w4.x, w4.z}), dup2(DIR > 0 ? DW{-w4.y, -w4.w} : DW{w4.y, w4.w})};
 #pragma unroll
-                        for (int q = 0; q < NC; ++q) b[r * NC + q] = dwc_mul_part(b[r * NC + q], w);
+                        for (int q = 0; q < NR; ++q) b[r * NR + q] = dwc_mul_part(b[r * NR + q], w);
                     } else {
                         C w = __ldg(reinterpret_cast<const C*>(a.tw) + idx);
                         if (DIR > 0) w.y = -w.y;
 #pragma unroll
-                        for (int q = 0; q < NC; ++q) b[r * NC + q] = cmul(b[r * NC + q], w);
+                        for (int q = 0; q < NR; ++q) b[r * NR + q] = cmul(b[r * NR + q], w);
                     }
                 }
             }
 #pragma unroll
-            for (int q = 0; q < NC; ++q) dftR<R, DIR, NC>(b + q);
+            for (int q = 0; q < NR; ++q) dftR<R, DIR, NR>(b + q);
         }
     }
 
@@ -526,7 +554,7 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
             for (int r = 0; r < R; ++r) {
                 const int k = lin(swz<LA, LB, G>(expand<LA, LB>(m * TF)) ^ (r << LA));
 #pragma unroll
-                for (int p = 0; p < NPL; ++p) sm[(wb ^ k) + p * PSTRIDE] = Unit<T>::pack(v + (m * R + r) * NC + p * CPP);
+                for (int p = 0; p < NPL; ++p) sm[(wb ^ k) + p * PSTRIDE] = Unit<T>::spack(v + (m * R + r) * NR, p);
             }
         block_sync(c);
 #pragma unroll
@@ -535,7 +563,7 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
             for (int r = 0; r < RN; ++r) {
                 const int k = lin(swz<LA, LB, G>((m * TF) | (r << (LOGN - LRN))));
 #pragma unroll
-                for (int p = 0; p < NPL; ++p) Unit<T>::unpack(sm[(rb ^ k) + p * PSTRIDE], v + (m * RN + r) * NC + p * CPP);
+                for (int p = 0; p < NPL; ++p) Unit<T>::sunpack(sm[(rb ^ k) + p * PSTRIDE], v + (m * RN + r) * NR, p);
             }
         if constexpr (!Cf::DB) block_sync(c);
     }
@@ -678,24 +706,21 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
                     const int x = c.jt + m * TF + r * (N / R);
                     const F f0 = fac[x], f1 = fac[PL + x], f2 = fac[2 * PL + x];
                     if constexpr (DWF)
-                        apply_potential_dw(c, v + (m * R + r) * NC, DW{f0.x, f0.y}, DW{f1.x, f1.y}, DW{f2.x, f2.y});
+                        apply_potential_dw(c, v + (m * R + r) * NR, DW{f0.x, f0.y}, DW{f1.x, f1.y}, DW{f2.x, f2.y});
                     else
-                        apply_potential(c, v + (m * R + r) * NC, f0, f1, f2);
+                        apply_potential(c, v + (m * R + r) * NR, f0, f1, f2);
                 }
         }
     }
 
     // (1 + c1) + i (s a).alpha on this thread's pair at one point, double-word: say = s a_y
-    // (negated for pair 1), sax = s a_x
+    // (negated for pair 1), sax = s a_x; both components at once, each lane's product with
+    // the other component
     KD_DI static void apply_potential_dw(const Ctx& c, C* e, DW c1, DW say0, DW sax) {
         if constexpr (DWF) {
-            const DW say = c.pair == 0 ? say0 : dw_neg(say0);
-            const C u = e[0], l = e[1];
-            const C q1 = C{say, sax}, q2 = C{dw_neg(say), sax};
-            const C du = dwc_add(dwc_mul_r(u, c1), dwc_mul(l, q1));
-            const C dl = dwc_add(dwc_mul_r(l, c1), dwc_mul(u, q2));
-            e[0] = dwc_add(u, du);
-            e[1] = dwc_add(l, dl);
+            const C own = e[0], oth = C{swap2(own.x), swap2(own.y)};
+            const C q = C{alt2(c.pair == 0 ? say0 : dw_neg(say0)), dup2(sax)};
+            e[0] = dwc_add(own, dwc_add(dwc_mul_r(own, dup2(c1)), dwc_mul(oth, q)));
         }
     }
 
@@ -771,7 +796,7 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
                 if constexpr (Cf::SHARE) {
                     if (c.valid) fsh[x] = make_float4(f[0], f[1], f[2], 0.0f);
                 } else {
-                    apply_potential(c, v + (m * R + r) * NC, f[0], f[1], f[2]);
+                    apply_potential(c, v + (m * R + r) * NR, f[0], f[1], f[2]);
                 }
             }
         if constexpr (Cf::SHARE) {
@@ -782,7 +807,7 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
                 for (int r = 0; r < R; ++r) {
                     const int x = c.jt + m * TF + r * (N / R);
                     const float4 f = c.valid ? fsh[x] : make_float4(0.f, 0.f, 0.f, 0.f);
-                    apply_potential(c, v + (m * R + r) * NC, f.x, f.y, f.z);
+                    apply_potential(c, v + (m * R + r) * NR, f.x, f.y, f.z);
                 }
             // single buffer: the next exchange writes over the factors
             if constexpr (!Cf::DB) block_sync(c);
@@ -814,25 +839,19 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
     // times 1 + f; each result is a rounding around psi itself, which carries no bias.
     // per-point kinetic table entries of this thread (op layout), loaded at kernel start
     // so that their L2 latency overlaps the first FFT
-    KD_DI static void load_ktab(const SweepArgs& a, const Ctx& c, C* kab) {
+    KD_DI static void load_ktab(const SweepArgs& a, const Ctx& c, TabC* kab) {
         constexpr int R = 1 << LR_OP;
-        const C* kt = reinterpret_cast<const C*>(a.ktab);
+        const TabC* kt = reinterpret_cast<const TabC*>(a.ktab);
 #pragma unroll
         for (int m = 0; m < E / R; ++m)
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 const int ky = c.jt + m * TF + r * (N / R);
-                if constexpr (DWF) {
-                    const float4 q = c.valid ? __ldcg(reinterpret_cast<const float4*>(a.ktab) + (long long)ky * a.nx + c.line)
-                                             : make_float4(0.f, 0.f, 0.f, 0.f);
-                    kab[m * R + r] = DWC{DW{q.x, q.y}, DW{q.z, q.w}};
-                } else {
-                    kab[m * R + r] = c.valid ? __ldcg(kt + (long long)ky * a.nx + c.line) : mk<C>(T(0), T(0));
-                }
+                kab[m * R + r] = c.valid ? __ldcg(kt + (long long)ky * a.nx + c.line) : TabC{};
             }
     }
 
-    KD_DI static void op_kinetic(const SweepArgs& a, const Ctx& c, C* v, const C* kab) {
+    KD_DI static void op_kinetic(const SweepArgs& a, const Ctx& c, C* v, const TabC* kab) {
         if constexpr (DWF) op_kinetic_dw(a, c, v, kab);
         else op_kinetic_std(a, c, v, kab);
     }
@@ -840,49 +859,40 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
     // the double-word kinetic step, the same factor as op_kinetic_std: tables a.kxtab
     // [nx] double-word pi_x (float2), a.kytab [ny][2] float4 (pi_y, cos phi - 1 | sin phi),
     // a.ktab [ny][nx] float4 ((C - 1)/P, c S/P)
-    KD_DI static void op_kinetic_dw(const SweepArgs& a, const Ctx& c, C* v, const C* kab) {
+    KD_DI static void op_kinetic_dw(const SweepArgs& a, const Ctx& c, C* v, const TabC* kab) {
         if constexpr (DWF) {
             constexpr int R = 1 << LR_OP;
             const float2 px = __ldg(reinterpret_cast<const float2*>(a.kxtab) + c.line);
-            const DW pix = DW{px.x, px.y};
-            const DW mc = dw_from_double(a.mc);
-            const float invP = (float)a.invP;   // a power of two: exact
+            const DW2 pix = dup2(DW{px.x, px.y});
+            const DW2 mc = alt2(dw_from_double(a.mc));
+            const F2 invP = dup2((float)a.invP);   // a power of two: exact
             const float4* kyt = reinterpret_cast<const float4*>(a.kytab);
 #pragma unroll
             for (int m = 0; m < E / R; ++m)
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     const int ky = c.jt + m * TF + r * (N / R);
-                    const C ab = kab[m * R + r];
+                    const float4 ab = kab[m * R + r];
                     const float4 y0 = __ldg(kyt + 2 * ky), y1 = __ldg(kyt + 2 * ky + 1);
-                    const DW fx = DW{y0.z, y0.w}, fy = DW{y1.x, y1.y};
-                    C* e = v + (m * R + r) * NC;
-#pragma unroll
-                    for (int q = 0; q < NC / 2; ++q) {
-                        const int pr = NC == 4 ? q : c.pair;
-                        const DW piy = pr == 0 ? DW{y0.x, y0.y} : DW{-y0.x, -y0.y};
-                        const C u = e[2 * q], l = e[2 * q + 1];
-                        // G = H0/c on the pair: (mc u + (pix - i piy) l, (pix + i piy) u - mc l)
-                        const C hu = C{dw_add(dw_dot2(mc, u.x, pix, l.x), dw_mul(piy, l.y)),
-                                       dw_sub(dw_dot2(mc, u.y, pix, l.y), dw_mul(piy, l.x))};
-                        const C hl = C{dw_sub(dw_dot2(pix, u.x, piy, dw_neg(u.y)), dw_mul(mc, l.x)),
-                                       dw_sub(dw_dot2(pix, u.y, piy, u.x), dw_mul(mc, l.y))};
-                        // u/P + a u - i b hu
-                        const C u1 = C{dw_add(dw_scale(u.x, invP), dw_dot2(ab.x, u.x, ab.y, hu.y)),
-                                       dw_add(dw_scale(u.y, invP), dw_dot2(ab.x, u.y, dw_neg(ab.y), hu.x))};
-                        const C l1 = C{dw_add(dw_scale(l.x, invP), dw_dot2(ab.x, l.x, ab.y, hl.y)),
-                                       dw_add(dw_scale(l.y, invP), dw_dot2(ab.x, l.y, dw_neg(ab.y), hl.x))};
-                        // times 1 + f (frame translation phase)
-                        e[2 * q] = C{dw_add(u1.x, dw_dot2(fx, u1.x, dw_neg(fy), u1.y)),
+                    const DW2 ka = dup2(DW{ab.x, ab.y}), kb = dup2(DW{ab.z, ab.w});
+                    const DW2 fx = dup2(DW{y0.z, y0.w}), fy = dup2(DW{y1.x, y1.y});
+                    const DW2 piy = alt2(c.pair == 0 ? DW{y0.x, y0.y} : DW{-y0.x, -y0.y});
+                    const C own = v[m * R + r], oth = C{swap2(own.x), swap2(own.y)};
+                    // G = H0/c on the pair, both components at once:
+                    // (mc u + pix l + piy l', -mc l + pix u - piy u'), l' = -i l
+                    const C h = C{dw_add(dw_dot2(mc, own.x, pix, oth.x), dw_mul(piy, oth.y)),
+                                  dw_sub(dw_dot2(mc, own.y, pix, oth.y), dw_mul(piy, oth.x))};
+                    // psi/P + a psi - i b G psi
+                    const C u1 = C{dw_add(dw_scale(own.x, invP), dw_dot2(ka, own.x, kb, h.y)),
+                                   dw_add(dw_scale(own.y, invP), dw_dot2(ka, own.y, dw_neg(kb), h.x))};
+                    // times 1 + f (frame translation phase)
+                    v[m * R + r] = C{dw_add(u1.x, dw_dot2(fx, u1.x, dw_neg(fy), u1.y)),
                                      dw_add(u1.y, dw_dot2(fx, u1.y, fy, u1.x))};
-                        e[2 * q + 1] = C{dw_add(l1.x, dw_dot2(fx, l1.x, dw_neg(fy), l1.y)),
-                                         dw_add(l1.y, dw_dot2(fx, l1.y, fy, l1.x))};
-                    }
                 }
         }
     }
 
-    KD_DI static void op_kinetic_std(const SweepArgs& a, const Ctx& c, C* v, const C* kab) {
+    KD_DI static void op_kinetic_std(const SweepArgs& a, const Ctx& c, C* v, const TabC* kab) {
         constexpr int R = 1 << LR_OP;
         const T pix = __ldg(reinterpret_cast<const T*>(a.kxtab) + c.line);
         T mc, invP;   // invP = 1/P is exact (power of two)
@@ -895,9 +905,9 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 const int ky = c.jt + m * TF + r * (N / R);
-                const C ab = kab[m * R + r];
+                const TabC ab = kab[m * R + r];
                 const T4 yv = kyt[ky];                   // (pi_y, cos phi - 1, sin phi, 0)
-                C* e = v + (m * R + r) * NC;
+                C* e = v + (m * R + r) * NR;
 #pragma unroll
                 for (int q = 0; q < NC / 2; ++q) {
                     const int pr = NC == 4 ? q : c.pair;
@@ -954,7 +964,7 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
         c.line = (blk / Cf::NPAIRS) * BATCH + c.bb % BATCH;
         c.valid = c.line < (AXIS == AXIS_X ? a.ny : a.nx);
         c.sm = reinterpret_cast<U*>(smem);
-        C v[E * NC];
+        C v[E * NR];
         if (trades(a)) cluster_arrive();   // this CTA runs: its shared memory may be written
         // programmatic dependent launch: everything above ran while the previous kernel
         // in the stream was still finishing; its results are visible after this wait
@@ -965,7 +975,7 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
         // the next kernel may start its own prologue as our CTAs retire
         if constexpr (PDL) asm volatile("griddepcontrol.launch_dependents;");
         if constexpr (AXIS == AXIS_Y) {
-            C kab[E];
+            TabC kab[E];
             // (after the FFT where sixteen elements a thread leave no registers for it)
             if (E < 16 && a.op == OP_KINETIC) load_ktab(a, c, kab);
             if constexpr (HAS1) fft<DIR1, false, 0, 0>(a, c, v);
