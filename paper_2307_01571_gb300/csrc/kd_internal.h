@@ -109,7 +109,7 @@ __host__ __device__ constexpr SweepVariant sweep_variant(int axis, int v) {
 // spinor components per thread of the FP32 sweeps
 __host__ __device__ constexpr int sweep_nc(int axis, int v);
 
-// The compiled forms of the FP32 sweeps: 0 ... 3 the variants as in the table, and two that
+// The compiled forms of the FP32 sweeps: 0 ... 3 the variants as in the table, and three that
 // the default (variants 0 and 1) becomes by the grid's size, sweep_form_of below.
 //   small: radix-4 stages, one or two rows / two columns per CTA.  A small grid is bound by
 //     the latency of one CTA and by idle SMs: 128 columns of 128 points in tiles of eight
@@ -117,15 +117,23 @@ __host__ __device__ constexpr int sweep_nc(int axis, int v);
 //   large: radix-16 stages (sixteen elements a thread).  A grid of many rounds is bound by the
 //     shared-memory exchanges and twiddle loads together with the FP32 pipe; radix-16 stages
 //     take two thirds of the former, and many rounds make up for the fewer warps.
-constexpr int kFormSmall = 4, kFormLarge = 5, kNumSweepForms = 6;
+//   wide: the small form with column tiles of 256 threads, for small grids in a batch that
+//     fills the SMs anyway.  It differs in threads per CTA alone, so a member still equals
+//     itself run alone, bit for bit.
+constexpr int kFormSmall = 4, kFormLarge = 5, kFormWide = 6, kNumSweepForms = 7;
 __host__ __device__ constexpr SweepVariant sweep_form(int axis, int form) {
     if (form < kNumSweepVariants) return sweep_variant(axis, form);
-    if (axis == AXIS_X) return form == kFormSmall ? SweepVariant{2, 64, 1, 2, 32, 0} : SweepVariant{4, 64, 1, 2, 16, 0};
-    return form == kFormSmall ? SweepVariant{2, 64, 2, 2, 32, 0} : SweepVariant{4, 256, 2, 2, 16, 0};
+    if (axis == AXIS_X) return form == kFormLarge ? SweepVariant{4, 64, 1, 2, 16, 0} : SweepVariant{2, 64, 1, 2, 32, 0};
+    return form == kFormSmall  ? SweepVariant{2, 64, 2, 2, 32, 0}
+           : form == kFormWide ? SweepVariant{2, 256, 4, 2, 32, 0}
+                               : SweepVariant{4, 256, 2, 2, 16, 0};
 }
-// axis lengths a form is compiled for
-__host__ __device__ constexpr bool sweep_form_holds(int form, int logn) {
-    return form == kFormSmall ? logn <= 11 : (form == kFormLarge ? logn >= 10 : true);
+// axes and lengths a form is compiled for
+__host__ __device__ constexpr bool sweep_form_holds(int axis, int form, int logn) {
+    return form == kFormSmall   ? logn <= 11
+           : form == kFormLarge ? logn >= 10
+           : form == kFormWide  ? axis == AXIS_Y && logn <= 9
+                                : true;
 }
 // The form that variant v runs on `lines` lines of 2^logn points.  The lines lie where the
 // measured times cross (GB300, us per sweep, default form against the chosen one):
@@ -142,12 +150,11 @@ __host__ __device__ constexpr bool sweep_form_holds(int form, int logn) {
 //     then large (1024x1024 30.7 : 29.5, 2048x1024 61.6 : 54.6, 4096x2048 292 : 263).
 // crowded: other simulations run beside this one and fill the SMs (a batch).  The small
 // form's narrow column tiles, which spread one small grid over the SMs, then only cost memory
-// transactions: the wide radix-4 tiles of variant 2 take their place.  They differ from the
-// small form in threads and components per CTA alone, so a member still equals itself run
-// alone, bit for bit.  16 members of 128x128 ... 512x256: 20.5 against 22.6 G point-steps/s.
+// transactions: the wide form takes their place.  16 members of 128x128 ... 512x256: 20.5
+// against 21.7 G point-steps/s.
 inline int sweep_form_of(int axis, int v, int logn, int lines, bool crowded) {
     if (v > 1) return v;
-    if (crowded && axis == AXIS_Y && logn <= 9 && ((long long)lines << logn) <= 1 << 16) return 2;
+    if (crowded && axis == AXIS_Y && logn <= 9 && ((long long)lines << logn) <= 1 << 16) return kFormWide;
     const long long points = (long long)lines << logn;
     if (axis == AXIS_X) {
         if (logn <= 11 && points <= 1 << 17) return kFormSmall;
