@@ -19,6 +19,7 @@
 #include <mutex>
 #include <string>
 #include <tuple>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/kd.h"
@@ -126,7 +127,7 @@ struct kd_sim {
     int64_t steps_cap = 0;
     double* rowsum = nullptr;
     double* md = nullptr;
-    double* scalar = nullptr;   // [0] norm of a reduction, [1] reference norm
+    double* scalar = nullptr;   // [1] the watchdog's reference norm
     kd_obs* obs_dev = nullptr;
     int64_t obs_dev_cap = 0;
     int* status = nullptr;
@@ -292,63 +293,85 @@ __host__ __device__ inline size_t slot_off(size_t P, size_t point, int s) {
     return ((size_t)(s >> 1) * P + point) * 4 + 2 * (s & 1);
 }
 
-// Per-row sum of |psi|^2 over both pair planes (fixed-order tree: bitwise reproducible).
+// Sum of v over the block's threads in a fixed order (bitwise reproducible), the same value
+// in every thread: shuffles within the warps, then the warps' sums in order.  sh: one double
+// per warp.  (A shared-memory tree with a barrier per level cost 1-2 us per reduction.)
+__device__ __forceinline__ double block_sum(double v, double* sh) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = sh[0];
+    for (int w = 1; w < (int)blockDim.x / 32; ++w) v += sh[w];
+    return v;
+}
+
+// Per-row sum of |psi|^2 over both pair planes, one block per row (fixed order).
 template <typename T>
 __global__ void k_rowsum(const T* psi, int nx, int ny, double* rowsum) {
-    __shared__ double red[256];
+    using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+    constexpr int PER = 16 / sizeof(T);
+    __shared__ double sh[8];
     const int row = blockIdx.x;
     const size_t P = (size_t)nx * ny;
-    // squares summed in groups of 8 in the spinor's precision, groups in FP64: keeps the
-    // FP32 sweeps' reduction off the slow FP64 pipe while the sum stays accurate to ~1e-9
+    // squares summed in groups of 8 (two points of a pair) in the spinor's precision, groups
+    // in FP64: keeps the FP32 sweeps' reduction off the slow FP64 pipe while the sum stays
+    // accurate to ~1e-9
     double acc = 0.0;
-    T part = T(0);
-    int cnt = 0;
-    for (int i = threadIdx.x; i < nx * 8; i += blockDim.x) {
-        const int pair = i / (nx * 4), k = i % (nx * 4);
-        const T v = psi[(pair * P + (size_t)row * nx) * 4 + k];
-        part += v * v;
-        if (++cnt == 8) { acc += (double)part; part = T(0); cnt = 0; }
+    for (int g = threadIdx.x; g < nx; g += blockDim.x) {
+        const int pair = g / (nx / 2), k = g % (nx / 2);
+        const V* q = reinterpret_cast<const V*>(psi + (pair * P + (size_t)row * nx) * 4 + 8 * k);
+        T v[8], part = T(0);
+#pragma unroll
+        for (int i = 0; i < 8 / PER; ++i) {
+            const V u = __ldcg(q + i);
+            memcpy(v + PER * i, &u, 16);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) part += v[i] * v[i];
+        acc += (double)part;
     }
-    acc += (double)part;
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) rowsum[row] = red[0];
+    acc = block_sum(acc, sh);
+    if (threadIdx.x == 0) rowsum[row] = acc;
 }
 
-// Phi(x) = sum_y |psi|^2 dy, one thread per column, rows in order.
+// Phi(x) = sum_y |psi|^2 dy: 32 columns per block, every 32nd row per warp in order, then the
+// warps' sums in order (one thread per column took 103 us for 128 x 128).
 template <typename T>
-__global__ void k_density_x(const T* psi, int nx, int ny, double dy, double* out) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= nx) return;
+__global__ void __launch_bounds__(1024) k_density_x(const T* psi, int nx, int ny, double dy, double* out) {
+    __shared__ double sh[32][33];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, x = blockIdx.x * 32 + lane;
     double acc = 0.0;
     const size_t P = (size_t)nx * ny;
-    for (int y = 0; y < ny; ++y) {
-        double s = 0.0;
-        for (int pair = 0; pair < 2; ++pair) {
-            const T* p = psi + (pair * P + (size_t)y * nx + x) * 4;
-            for (int i = 0; i < 4; ++i) s += (double)p[i] * (double)p[i];
+    if (x < nx)
+        for (int y = g; y < ny; y += 32) {
+            double s = 0.0;
+#pragma unroll
+            for (int pair = 0; pair < 2; ++pair) {
+                const T* p = psi + (pair * P + (size_t)y * nx + x) * 4;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) s += (double)p[i] * (double)p[i];
+            }
+            acc += s;
         }
-        acc += s;
+    sh[g][lane] = acc;
+    __syncthreads();
+    if (g == 0 && x < nx) {
+        for (int w = 1; w < 32; ++w) acc += sh[w][lane];
+        out[x] = acc * dy;
     }
-    out[x] = acc * dy;
 }
 
-// Sum of the row sums times dx dy into scalar[slot]; fixed order.
-__global__ void k_norm(const double* rowsum, int ny, double cell, double* scalar, int slot) {
-    __shared__ double red[256];
+// The row sums' total times dx dy, in every thread of a block; fixed order.
+__device__ __forceinline__ double norm_of(const double* rowsum, int ny, double cell, double* sh) {
     double acc = 0.0;
     for (int i = threadIdx.x; i < ny; i += blockDim.x) acc += rowsum[i];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) scalar[slot] = red[0] * cell;
+    return block_sum(acc, sh) * cell;
+}
+// The norm into scalar[slot].
+__global__ void k_norm(const double* rowsum, int ny, double cell, double* scalar, int slot) {
+    __shared__ double sh[8];
+    const double v = norm_of(rowsum, ny, cell, sh);
+    if (threadIdx.x == 0) scalar[slot] = v;
 }
 
 // Power-of-two operand scales of the tensor-core sweeps from the state's 2-norm
@@ -382,13 +405,29 @@ __global__ void k_tc_scales(const double* rowsum, int nx, int ny, float* out) {
     out[3] = p2(sqrt(P * nx));
 }
 
+// psi / sqrt(norm): every block adds up the row sums itself (a few KB out of L2) instead of
+// waiting for a launch of its own, and takes the FP64 root and quotient once (in every thread
+// they were most of the kernel's 10 us)
 template <typename T>
-__global__ void k_scale_by_norm(T* psi, size_t n, const double* scalar) {
-    const double nr = scalar[0];
-    const T s = (T)(nr > 0.0 ? 1.0 / sqrt(nr) : 0.0);
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x)
-        psi[i] *= s;
+__global__ void __launch_bounds__(256) k_scale_by_norm(T* psi, size_t n, const double* rowsum, int ny, double cell) {
+    using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+    constexpr int PER = 16 / sizeof(T);
+    __shared__ double sh[8];
+    __shared__ T scale;
+    const double nr = norm_of(rowsum, ny, cell, sh);
+    if (threadIdx.x == 0) scale = (T)(nr > 0.0 ? 1.0 / sqrt(nr) : 0.0);
+    __syncthreads();
+    const T s = scale;
+    V* q = reinterpret_cast<V*>(psi);   // n is a multiple of 8
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n / PER; i += (size_t)gridDim.x * blockDim.x) {
+        V u = q[i];
+        T v[PER];
+        memcpy(v, &u, 16);
+#pragma unroll
+        for (int k = 0; k < PER; ++k) v[k] *= s;
+        memcpy(&u, v, 16);
+        q[i] = u;
+    }
 }
 
 // Normalised positive-energy bispinor u^s(pi) of Eq. (Spinors_of_Dirac_equation) with
@@ -429,6 +468,14 @@ __global__ void k_packet(T* psi, int nx, int ny, double dpx, double dpy, double 
     const double pix = px + shx, piy = py + shy;
     const double ddx = pix - p0x, ddy = piy - p0y;
     const double mag = exp(-(ddx * ddx + ddy * ddy) / (4.0 * sig * sig));
+    // far from the packet the values round to zero: most of a large grid
+    if (mag <= (sizeof(T) == 4 ? 1e-50 : 0.0)) {
+        for (int s = 0; s < 4; ++s) {
+            const size_t o = slot_off((size_t)nx * ny, i, s);
+            psi[o] = psi[o + 1] = T(0);
+        }
+        return;
+    }
     double sn, cs;
     sincos(-(rx * px + ry * py) / hbar, &sn, &cs);
     double2 u[4];
@@ -530,48 +577,39 @@ __global__ void k_obs_reduce(const double* rowsum, const double* cells, int nx, 
                              ObsWin w, const StepScalars* steps, const Clock* clock, int n_local,
                              double t_fixed, int64_t obs_every, int64_t cap, kd_obs* out,
                              const double* scalar, double tol, int* status) {
-    __shared__ double red[256];
+    // all ten reductions at once: warps by shuffles, then the eight warps' values in order
+    // (one shared-memory tree per value took 22 us, as long as the rest of a small read-out)
+    __shared__ double sh[8][10], tot[10];
     const int tid = threadIdx.x;
-    auto tree = [&](double v) -> double {
-        red[tid] = v;
-        __syncthreads();
-        for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-            if (tid < s) red[tid] += red[tid + s];
-            __syncthreads();
-        }
-        const double r = red[0];
-        __syncthreads();
-        return r;
-    };
-    auto treemax = [&](double v) -> double {
-        red[tid] = v;
-        __syncthreads();
-        for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-            if (tid < s) red[tid] = fmax(red[tid], red[tid + s]);
-            __syncthreads();
-        }
-        const double r = red[0];
-        __syncthreads();
-        return r;
-    };
-    double acc = 0.0;
-    for (int i = tid; i < ny; i += blockDim.x) acc += rowsum[i];
-    const double norm = tree(acc) * cell;
-    double sums[2][3], mx[3] = {0, 0, 0};
+    double v[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};   // norm, sums [2][3], maxima [3]
+    for (int i = tid; i < ny; i += blockDim.x) v[0] += rowsum[i];
     const int n0 = (w.ihi[0] - w.ilo[0] + 1) * (w.jhi[0] - w.jlo[0] + 1);
     const int n1 = (w.ihi[1] - w.ilo[1] + 1) * (w.jhi[1] - w.jlo[1] + 1);
-    for (int wi = 0; wi < 2; ++wi) {
-        const int nc = wi == 0 ? n0 : n1;
-        const double* base = cells + (wi == 0 ? 0 : (size_t)n0 * 3);
-        double a[3] = {0, 0, 0}, m[3] = {0, 0, 0};
-        for (int q = tid; q < nc; q += blockDim.x) {
-            const double* o = base + (size_t)q * 3;
-            for (int k = 0; k < 3; ++k) { a[k] += o[k]; m[k] = fmax(m[k], o[k]); }
+    for (int q = tid; q < n0; q += blockDim.x)
+        for (int k = 0; k < 3; ++k) v[1 + k] += cells[(size_t)q * 3 + k];
+    for (int q = tid; q < n1; q += blockDim.x)
+        for (int k = 0; k < 3; ++k) {
+            const double o = cells[(size_t)(n0 + q) * 3 + k];
+            v[4 + k] += o;
+            v[7 + k] = fmax(v[7 + k], o);
         }
-        for (int k = 0; k < 3; ++k) sums[wi][k] = tree(a[k]);
-        if (wi == 1)
-            for (int k = 0; k < 3; ++k) mx[k] = treemax(m[k]);
+#pragma unroll
+    for (int k = 0; k < 10; ++k)
+        for (int o = 16; o > 0; o >>= 1) {
+            const double u = __shfl_xor_sync(0xffffffffu, v[k], o);
+            v[k] = k < 7 ? v[k] + u : fmax(v[k], u);
+        }
+    if ((tid & 31) == 0)
+#pragma unroll
+        for (int k = 0; k < 10; ++k) sh[tid >> 5][k] = v[k];
+    __syncthreads();
+    if (tid < 10) {
+        double r = sh[0][tid];
+        for (int i = 1; i < 8; ++i) r = tid < 7 ? r + sh[i][tid] : fmax(r, sh[i][tid]);
+        tot[tid] = r;
     }
+    __syncthreads();
+    const double norm = tot[0] * cell;
     if (tid == 0) {
         int64_t slot = 0;
         double t = t_fixed;
@@ -584,9 +622,9 @@ __global__ void k_obs_reduce(const double* rowsum, const double* cells, int nx, 
         kd_obs r;
         r.t = t;
         r.norm = norm;
-        r.pop_in = sums[0][0]; r.cp_in = sums[0][1]; r.cm_in = sums[0][2];
-        r.pop_diff = sums[1][0]; r.cp_diff = sums[1][1]; r.cm_diff = sums[1][2];
-        r.max_diff = mx[0]; r.cp_max_diff = mx[1]; r.cm_max_diff = mx[2];
+        r.pop_in = tot[1]; r.cp_in = tot[2]; r.cm_in = tot[3];
+        r.pop_diff = tot[4]; r.cp_diff = tot[5]; r.cm_diff = tot[6];
+        r.max_diff = tot[7]; r.cp_max_diff = tot[8]; r.cm_max_diff = tot[9];
         r.p_target = o[0]; r.cp_target = o[1]; r.cm_target = o[2];
         if (slot >= 0 && slot < cap) out[slot] = r;
         int st = 0;
@@ -698,10 +736,11 @@ template <typename T> int upload_tables_t(kd_sim* s) {
     // stage-major twiddle tables, built on the device in FP64 (<= 2N entries of 16 B)
     // for every radix schedule a launch shape may use
     for (int ax = 0; ax < 2; ++ax)
-        for (int le = 2; le <= (sizeof(T) == 4 ? 4 : 3); ++le) {
+        for (int le = 2; le <= 4; ++le) {
             int entries = 0;
             const int logn = ax == 0 ? s->lx : s->ly;
             void* dst = s->tw[ax][le - 2];
+            if (!dst) continue;
             KD_CUDA(sizeof(T) == 4 ? build_twiddles_f32(logn, le, dst, &entries, s->stream)
                                    : build_twiddles_f64(logn, le, dst, &entries, s->stream));
             if (entries > 2 * (1 << logn)) return fail(KD_ERR_CUDA, "twiddle table overflow");
@@ -1074,8 +1113,9 @@ int time_sweep(kd_sim* s, int axis, int reps, double dt, float* ms) {
     } while (0)
 
 int rowsum_launch(kd_sim* s, const void* psi) {   // psi: FP64 for KD_FP64 and KD_DW (view)
-    if (s->prec == KD_FP64) k_rowsum<double><<<s->g.ny, 256, 0, s->stream>>>((const double*)psi, s->g.nx, s->g.ny, s->rowsum);
-    else k_rowsum<float><<<s->g.ny, 256, 0, s->stream>>>((const float*)psi, s->g.nx, s->g.ny, s->rowsum);
+    const int threads = s->g.nx >= 256 ? 256 : (s->g.nx <= 32 ? 32 : s->g.nx);
+    if (s->prec == KD_FP64) k_rowsum<double><<<s->g.ny, threads, 0, s->stream>>>((const double*)psi, s->g.nx, s->g.ny, s->rowsum);
+    else k_rowsum<float><<<s->g.ny, threads, 0, s->stream>>>((const float*)psi, s->g.nx, s->g.ny, s->rowsum);
     KD_CUDA(cudaGetLastError());
     ++s->launches;
     return KD_OK;
@@ -1404,10 +1444,11 @@ int kd_create(const kd_units* units, const kd_grid* grid, const kd_field* field,
             return bail(fail(KD_ERR_CUDA, "event create failed"));
     KD_ALLOC(s->psi, spinor_bytes(s));
     KD_ALLOC(s->work, spinor_bytes(s));
-    for (int le = 0; le < 3; ++le) {
-        KD_ALLOC(s->tw[AXIS_X][le], 2 * (size_t)grid->nx * 16);
-        KD_ALLOC(s->tw[AXIS_Y][le], 2 * (size_t)grid->ny * 16);
-    }
+    for (int le = 0; le < 3; ++le)
+        for (int ax : {(int)AXIS_X, (int)AXIS_Y}) {
+            if (le == 2 && (s->prec == KD_FP64 || form(s, ax) != kFormLarge)) continue;   // radix-16: the large form
+            KD_ALLOC(s->tw[ax][le], 2 * (size_t)(ax == AXIS_X ? grid->nx : grid->ny) * 16);
+        }
     KD_ALLOC(s->xtab, 8 * (size_t)grid->nx * s->tsize);
     KD_ALLOC(s->kxtab, (size_t)grid->nx * s->tsize);
     KD_ALLOC(s->kytab, 4 * (size_t)grid->ny * s->tsize);
@@ -1542,12 +1583,10 @@ int kd_init_packet(kd_sim* s, const kd_packet* pk) {
     KD_LAUNCH(sweep(s, AXIS_X, SHAPE_F1, OP_NONE, s->psi, s->psi, 0, 0.0, true));
     rc = rowsum_launch(s, s->psi);
     if (rc) return rc;
-    k_norm<<<1, 256, 0, s->stream>>>(s->rowsum, s->g.ny, dxdy(s), s->scalar, 0);
-    KD_CUDA(cudaGetLastError());
-    ++s->launches;
     const size_t nreal = s->P * 8;
-    if (s->prec == KD_FP64) k_scale_by_norm<double><<<1024, 256, 0, s->stream>>>((double*)s->psi, nreal, s->scalar);
-    else k_scale_by_norm<float><<<1024, 256, 0, s->stream>>>((float*)s->psi, nreal, s->scalar);
+    const int sb = grid_blocks(nreal, 2048) < 608 ? grid_blocks(nreal, 2048) : 608;
+    if (s->prec == KD_FP64) k_scale_by_norm<double><<<sb, 256, 0, s->stream>>>((double*)s->psi, nreal, s->rowsum, s->g.ny, dxdy(s));
+    else k_scale_by_norm<float><<<sb, 256, 0, s->stream>>>((float*)s->psi, nreal, s->rowsum, s->g.ny, dxdy(s));
     KD_CUDA(cudaGetLastError());
     ++s->launches;
     if (s->dw) {
@@ -2331,8 +2370,8 @@ int kd_get_density_x(kd_sim* s, double* out, int32_t where) {
     const void* st = nullptr;
     rc = state_view(s, &st);
     if (rc) return rc;
-    if (s->prec == KD_FP64) k_density_x<double><<<grid_blocks(s->g.nx, 128), 128, 0, s->stream>>>((const double*)st, s->g.nx, s->g.ny, dy, dst);
-    else k_density_x<float><<<grid_blocks(s->g.nx, 128), 128, 0, s->stream>>>((const float*)s->psi, s->g.nx, s->g.ny, dy, dst);
+    if (s->prec == KD_FP64) k_density_x<double><<<grid_blocks(s->g.nx, 32), 1024, 0, s->stream>>>((const double*)st, s->g.nx, s->g.ny, dy, dst);
+    else k_density_x<float><<<grid_blocks(s->g.nx, 32), 1024, 0, s->stream>>>((const float*)s->psi, s->g.nx, s->g.ny, dy, dst);
     KD_CUDA(cudaGetLastError());
     ++s->launches;
     if (where == KD_HOST) {
