@@ -140,9 +140,10 @@ __host__ __device__ constexpr bool sweep_form_holds(int axis, int form, int logn
 //   x, up to 2^17 points: 64x64 4.9 : 3.2, 256x256 5.6 : 4.2, 1024x128 7.4 : 6.5, 2048x64
 //     7.7 : 7.3; at 2^18 the radix-8 default is ahead (512x512 8.6 : 9.2);
 //   x, 2048 and 4096 points: both pairs per thread (variant 3, the field evaluated once) up to
-//     2^20 points (2048x128 12.9 : 10.9, 2048x256 18.7 : 15.5, 4096x256 40.0 : 33.1), then
-//     large (2048x512 29.7 : 27.8, 4096x2048 288 : 234); 4096x64 is too few rows for
-//     variant 3 (11.1 : 16.7);
+//     2^20 points (2048x128 12.9 : 10.9, 2048x256 18.7 : 15.5, 4096x256 40.0 : 33.1; variant
+//     1 takes 10.3 alone at 2048x128, but its 512-thread CTAs leave no room for the next
+//     sweep's to start under: 21.0 us a step against 18.7), then large (2048x512 29.7 : 27.8,
+//     4096x2048 288 : 234); 4096x64 is too few rows for variant 3 (11.1 : 16.7);
 //   y up to 512 points: small up to 2^16 points (64x64 5.4 : 2.2, 128x128 6.5 : 2.5, 256x256
 //     7.1 : 4.1), radix-4 tiles of both pairs at 2^17 (512x256 7.2 : 5.0);
 //   y from 1024 points (few columns): small up to 2^17 points (128x1024 15.6 : 7.0, 64x2048

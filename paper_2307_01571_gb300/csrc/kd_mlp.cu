@@ -65,7 +65,7 @@ __device__ __forceinline__ float gelu_grad(float x) {
 // or a loader, and a launch starts under its predecessor's tail (programmatic dependent
 // launch).  Chain of a training step: L forward launches, L backward launches, Adam.
 //
-// A step at batch 256 / FP32 went from 22 launches and 396 us to 9 launches and 51 us, at batch
+// A step at batch 256 / FP32 went from 22 launches and 396 us to 9 launches and 43 us, at batch
 // 1024 / BF16 from 401 to 73 us (GB300, the 5-256-256-256-4 network).  What bounds it now is
 // the chain: nine dependent launches of 4-8 us, most of it launch and load latency.
 
@@ -97,7 +97,7 @@ struct Product {
     float* sq;
     float scale;
     int M, N, K, epi;
-    int mt, nt_tiles, splits, kper;
+    int bm, mt, nt_tiles, splits, kper;
 };
 // Column sums out[s][n] = sum over part s of the rows of X [M][N] (32 columns per CTA)
 struct ColSum {
@@ -126,8 +126,16 @@ struct Group {
 // per kind: a kernel of this size runs its code once, from a cold instruction cache, so the
 // kind is decided outside the loop and the loop stays short (unrolled over every kind the
 // BF16 epilogue took 14,000 cycles a tile).
+template <int NE> __device__ __forceinline__ void epi_prefetch(const Product& q, int m, int mstep, int n, int nstep, float (&z)[NE]) {
+    if (q.epi != EPI_GELU_BACK) return;
+#pragma unroll
+    for (int i = 0; i < NE; ++i) {
+        const int mi = m + i * mstep, ni = n + i * nstep;
+        z[i] = mi < q.M && ni < q.N ? __ldg(q.Z + (long)mi * q.N + ni) : 0.0f;
+    }
+}
 template <int NE, int UNROLL, typename F>
-__device__ __forceinline__ void epilogue(const Product& q, int m, int mstep, int n, int nstep, int split, F v) {
+__device__ __forceinline__ void epilogue(const Product& q, int m, int mstep, int n, int nstep, int split, const float (&z)[NE], F v) {
     auto each = [&](auto f) {
 #pragma unroll UNROLL
         for (int i = 0; i < NE; ++i) {
@@ -145,7 +153,11 @@ __device__ __forceinline__ void epilogue(const Product& q, int m, int mstep, int
             q.C[o] = gelu(x);
         });
     } else if (q.epi == EPI_GELU_BACK) {
-        each([&](int, int, long o, float x) { q.C[o] = x * gelu_grad(__ldg(q.Z + o)); });
+#pragma unroll
+        for (int i = 0; i < NE; ++i) {
+            const int mi = m + i * mstep, ni = n + i * nstep;
+            if (mi < q.M && ni < q.N) q.C[(long)mi * q.N + ni] = v(i) * gelu_grad(z[i]);
+        }
     } else if (q.epi == EPI_BIAS) {
         each([&](int, int ni, long o, float x) { q.C[o] = x + __ldg(q.bias + ni); });
     } else {
@@ -197,21 +209,21 @@ __device__ void colsum_block(const ColSum& c, int blk) {
     }
 }
 
-// FP32 products on the CUDA cores: 32 x 32 tiles (64 CTAs for a 256 x 256 output, where
-// 64 x 64 tiles gave 16), 64-deep k slabs in a ring of four shared-memory stages filled by
-// cp.async (zero-filled outside the operand), so that a K = 256 product waits for the load
-// latency once.  A slab's k range is shared by four groups of 64 threads, each with 4 x 4
-// outputs a thread (16-byte shared loads, two per 16 FMAs), whose partial sums are added in
-// a fixed order at the end.  A slab keeps its operand's own contiguous dimension: [32 rows]
-// [64 k] with 68 floats a row, a thread taking rows ty + 8 i (conflict-free 16-byte reads
-// along k), or [64 k][32 rows] with 36 floats, a thread taking rows 4 ty + i.  64 x 64 tiles
-// with one k group and 16-deep slabs of scalar loads took 44 us for 256^3 under
-// ncu; this takes 6.6.
+// FP32 products on the CUDA cores: tiles of 32 columns and 16 or 32 rows (128 or 64 CTAs for a
+// 256 x 256 output, where 64 x 64 tiles gave 16), 64-deep k slabs in a ring of four
+// shared-memory stages filled by cp.async (zero-filled outside the operand), so that a K = 256
+// product waits for the load latency once.  A slab's k range is shared by the eight warps,
+// each with the whole tile (4 or 8 x 4 outputs a thread, 16-byte shared loads, two or one and
+// a half per 16 FMAs), whose partial sums are added in a fixed order at the end.  A slab
+// keeps its operand's own contiguous dimension: [rows][64 k] with 68 floats a row, a thread
+// taking every 4th (columns: 8th) row (conflict-free 16-byte reads along k), or [64 k][rows]
+// with four floats of padding, a thread taking consecutive rows.  64 x 64 tiles with one k
+// group and 16-deep slabs of scalar loads took 44 us for 256^3 under ncu; this takes 5.
 namespace fp32 {
-constexpr int STAGES = 4, KS = 64, KP = KS + 4, RP = 36;
-constexpr int OP = KS * RP;                        // floats of one operand's slab
-constexpr int SMEM = STAGES * 2 * OP * 4;
-static_assert(OP >= 32 * KP && STAGES * 2 * OP >= 4 * 32 * RP, "slab and reduction fit");
+constexpr int STAGES = 4, KS = 64, KP = KS + 4;
+constexpr int BN = 32, PB = BN + 4, OPB = KS * PB;  // floats of an operand's slab of 32 rows
+constexpr int SMEM = STAGES * 2 * OPB * 4;
+static_assert(OPB >= BN * KP && STAGES * 2 * OPB >= 8 * 32 * PB, "slabs and reduction fit");
 
 __device__ __forceinline__ void copy16(float* dst, const float* src, int bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
@@ -221,14 +233,14 @@ __device__ __forceinline__ void copy4(float* dst, const float* src, int bytes) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
                  :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
 }
-// 32 rows x 64 k of an operand into a slab, zeros outside its R rows and [.., kend): 512
-// groups of four contiguous elements, two per thread
-template <bool KC> __device__ __forceinline__ void slab_load(float* sm, const Operand& o, int r0, int R, int k0, int kend) {
+// ROWS rows x 64 k of an operand into a slab, zeros outside its R rows and [.., kend): groups
+// of four contiguous elements, ROWS / 16 per thread
+template <int ROWS, bool KC> __device__ __forceinline__ void slab_load(float* sm, const Operand& o, int r0, int R, int k0, int kend) {
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < ROWS / 16; ++i) {
         const int c = threadIdx.x + 256 * i;
-        const int row = KC ? c >> 4 : 4 * (c & 7), k = KC ? 4 * (c & 15) : c >> 3;
-        float* dst = sm + (KC ? row * KP + k : k * RP + row);
+        const int row = KC ? c >> 4 : 4 * (c % (ROWS / 4)), k = KC ? 4 * (c & 15) : c / (ROWS / 4);
+        float* dst = sm + (KC ? row * KP + k : k * (ROWS + 4) + row);
         const int gr = r0 + row, gk = k0 + k, at = KC ? gk : gr;
         long line = KC ? gr : gk;
         int n = 4;   // elements inside
@@ -247,63 +259,84 @@ template <bool KC> __device__ __forceinline__ void slab_load(float* sm, const Op
         }
     }
 }
-// a thread's four rows (columns) u of a slab at k .. k + 3: element [i][kk]
-template <bool KC> __device__ __forceinline__ void slab_read(const float* sm, int u, int k, float (&v)[4][4]) {
+// a thread's NT of a slab's LN NT rows at k .. k + 3, element [i][kk]: rows u + LN i of a slab
+// contiguous in k, else rows NT u + i
+template <int LN, int NT, bool KC> __device__ __forceinline__ void slab_read(const float* sm, int u, int k, float (&v)[NT][4]) {
+    if constexpr (KC) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float4 q = *reinterpret_cast<const float4*>(KC ? sm + (u + 8 * i) * KP + k : sm + (k + i) * RP + 4 * u);
-        if (KC) { v[i][0] = q.x; v[i][1] = q.y; v[i][2] = q.z; v[i][3] = q.w; }
-        else { v[0][i] = q.x; v[1][i] = q.y; v[2][i] = q.z; v[3][i] = q.w; }
+        for (int i = 0; i < NT; ++i) {
+            const float4 q = *reinterpret_cast<const float4*>(sm + (u + LN * i) * KP + k);
+            v[i][0] = q.x; v[i][1] = q.y; v[i][2] = q.z; v[i][3] = q.w;
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int i = 0; i < NT; i += 4) {
+                const float4 q = *reinterpret_cast<const float4*>(sm + (k + e) * (LN * NT + 4) + NT * u + i);
+                v[i][e] = q.x; v[i + 1][e] = q.y; v[i + 2][e] = q.z; v[i + 3][e] = q.w;
+            }
     }
 }
 
-template <bool AKC, bool BKC> __device__ __forceinline__ void product(const Product& q, int blk, float* sm) {
+template <int BM, bool AKC, bool BKC> __device__ __forceinline__ void product(const Product& q, int blk, float* sm) {
+    constexpr int TM = BM / 4, OPA = KS * (BM + 4), NE = BM / 8;   // rows a thread, A slab, outputs a thread
+    static_assert(OPA >= BM * KP && OPA <= OPB, "A slab");
     const int t = threadIdx.x;
-    const int n0 = (blk % q.nt_tiles) * 32, m0 = blk / q.nt_tiles % q.mt * 32, split = blk / (q.nt_tiles * q.mt);
+    const int n0 = (blk % q.nt_tiles) * BN, m0 = blk / q.nt_tiles % q.mt * BM, split = blk / (q.nt_tiles * q.mt);
     const int kbeg = split * q.kper, kend = min(q.K, kbeg + q.kper);
     const int nslab = (kend - kbeg + KS - 1) / KS;
-    const int g = t >> 6, ty = (t & 63) >> 3, tx = t & 7;
+    const int g = t >> 5, ty = (t & 31) >> 3, tx = t & 7;
     auto fill = [&](int j) {
         if (j < nslab) {
-            float* st = sm + (j % STAGES) * 2 * OP;
-            slab_load<AKC>(st, q.A, m0, q.M, kbeg + KS * j, kend);
-            slab_load<BKC>(st + OP, q.B, n0, q.N, kbeg + KS * j, kend);
+            float* st = sm + (j % STAGES) * (OPA + OPB);
+            slab_load<BM, AKC>(st, q.A, m0, q.M, kbeg + KS * j, kend);
+            slab_load<BN, BKC>(st + OPA, q.B, n0, q.N, kbeg + KS * j, kend);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     for (int j = 0; j < STAGES - 1; ++j) fill(j);
-    float acc[4][4] = {{0.0f}};
+    const int re = t / (BN / NE), ce = NE * (t % (BN / NE));   // this thread's outputs: NE of a row
+    float z[NE];
+    epi_prefetch<NE>(q, m0 + re, 0, n0 + ce, 1, z);
+    float acc[TM][4];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int h = 0; h < 4; ++h) acc[i][h] = 0.0f;
     for (int j = 0; j < nslab; ++j) {
         asm volatile("cp.async.wait_group %0;" :: "n"(STAGES - 2) : "memory");
         __syncthreads();            // slab j has landed, slab j - 1's stage is free
         fill(j + STAGES - 1);
-        const float* as = sm + (j % STAGES) * 2 * OP;
-        const float* bs = as + OP;
+        const float* as = sm + (j % STAGES) * (OPA + OPB);
+        const float* bs = as + OPA;
 #pragma unroll
-        for (int kk = 0; kk < 16; kk += 4) {
-            float av[4][4], bv[4][4];
-            slab_read<AKC>(as, ty, 16 * g + kk, av);
-            slab_read<BKC>(bs, tx, 16 * g + kk, bv);
+        for (int kk = 0; kk < 8; kk += 4) {
+            float av[TM][4], bv[4][4];
+            slab_read<4, TM, AKC>(as, ty, 8 * g + kk, av);
+            slab_read<8, 4, BKC>(bs, tx, 8 * g + kk, bv);
 #pragma unroll
             for (int e = 0; e < 4; ++e)
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < TM; ++i)
 #pragma unroll
                     for (int h = 0; h < 4; ++h) acc[i][h] = fmaf(av[i][e], bv[h][e], acc[i][h]);
         }
     }
-    // the four groups' partial sums, through shared memory, added in order
+    // the eight groups' partial sums, through shared memory, added in order
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
         for (int h = 0; h < 4; ++h)
-            sm[(g * 32 + (AKC ? ty + 8 * i : 4 * ty + i)) * RP + (BKC ? tx + 8 * h : 4 * tx + h)] = acc[i][h];
+            sm[(g * BM + (AKC ? ty + 4 * i : TM * ty + i)) * PB + (BKC ? tx + 8 * h : 4 * tx + h)] = acc[i][h];
     __syncthreads();
-    const float* r = sm + (t >> 3) * RP + 4 * (t & 7);
-    epilogue<4, 4>(q, m0 + (t >> 3), 0, n0 + 4 * (t & 7), 1, split,
-                   [&](int j) { return (r[j] + r[32 * RP + j]) + (r[64 * RP + j] + r[96 * RP + j]); });
+    const float* r = sm + re * PB + ce;
+    constexpr int G = BM * PB;
+    epilogue<NE, NE>(q, m0 + re, 0, n0 + ce, 1, split, z, [&](int j) {
+        return ((r[j] + r[G + j]) + (r[2 * G + j] + r[3 * G + j])) + ((r[4 * G + j] + r[5 * G + j]) + (r[6 * G + j] + r[7 * G + j]));
+    });
 }
 }  // namespace fp32
 
@@ -542,7 +575,9 @@ __device__ __forceinline__ void product_bf16(const Product& q, int blk, int* sta
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (ok && nslab > 0) {
         const float* tr = reinterpret_cast<const float*>(sm) + (t >> 4) * 17 + (t & 15);
-        epilogue<8, 2>(q, m0 + (t >> 4), 16, n0 + (t & 15), 0, split, [&](int i) { return tr[16 * i * 17]; });
+        float z[8];
+        epi_prefetch<8>(q, m0 + (t >> 4), 16, n0 + (t & 15), 0, z);
+        epilogue<8, 2>(q, m0 + (t >> 4), 16, n0 + (t & 15), 0, split, z, [&](int i) { return tr[16 * i * 17]; });
     }
     if (!ok && t == 0) atomicOr(status, 1);
     if (w == 0)
@@ -577,9 +612,15 @@ template <int BF16> __global__ void __launch_bounds__(256) k_group(const __grid_
             else product_bf16<true, false>(q, b, g.status, sm);
         } else {
             float* f = reinterpret_cast<float*>(sm);
-            if (!q.A.kc) fp32::product<false, false>(q, b, f);
-            else if (q.B.kc) fp32::product<true, true>(q, b, f);
-            else fp32::product<true, false>(q, b, f);
+            if (q.bm == 16) {
+                if (!q.A.kc) fp32::product<16, false, false>(q, b, f);
+                else if (q.B.kc) fp32::product<16, true, true>(q, b, f);
+                else fp32::product<16, true, false>(q, b, f);
+            } else {
+                if (!q.A.kc) fp32::product<32, false, false>(q, b, f);
+                else if (q.B.kc) fp32::product<32, true, true>(q, b, f);
+                else fp32::product<32, true, false>(q, b, f);
+            }
         }
     }
 }
@@ -626,11 +667,17 @@ Operand operand(const float* p, long ld, bool kc, const int32_t* idx = nullptr, 
     return Operand{p, ld, idx, nidx, kc ? 1 : 0, vec ? 1 : 0};
 }
 
-// tiles of the product at the network's precision, its k range in `splits` parts
+// Tiles of the product at the network's precision, its k range in `splits` parts.  FP32: 16-row
+// tiles while 32-row ones would leave SMs without one (256 x 256 outputs: 64 tiles), since what
+// counts there is one tile's latency; else 32 rows, which read half as much per output (a step
+// at batch 256 42.9 us against 51.2 with 32 rows only; at batch 1024 78.8 with 16 rows only
+// against 74.6).
 void tile(const kd_mlp* n, Product* q, int splits) {
-    const int bm = n->prec == KD_MLP_BF16 ? 128 : 32, bn = n->prec == KD_MLP_BF16 ? tcg::BN : 32;
-    q->mt = (q->M + bm - 1) / bm;
+    const bool bf = n->prec == KD_MLP_BF16;
+    const int bn = bf ? tcg::BN : fp32::BN;
     q->nt_tiles = (q->N + bn - 1) / bn;
+    q->bm = bf ? 128 : ((q->M + 31) / 32 * q->nt_tiles * splits < 152 ? 16 : 32);
+    q->mt = (q->M + q->bm - 1) / q->bm;
     q->splits = splits;
     q->kper = (q->K + splits - 1) / splits;
 }
