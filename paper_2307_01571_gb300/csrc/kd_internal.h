@@ -114,16 +114,17 @@ __host__ __device__ constexpr int sweep_nc(int axis, int v);
 //   small: radix-4 stages, one or two rows / two columns per CTA.  A small grid is bound by
 //     the latency of one CTA and by idle SMs: 128 columns of 128 points in tiles of eight
 //     columns and both pairs were 16 CTAs on 152 SMs.
-//   large: radix-16 stages (sixteen elements a thread).  A grid of many rounds is bound by the
-//     shared-memory exchanges and twiddle loads together with the FP32 pipe; radix-16 stages
-//     take two thirds of the former, and many rounds make up for the fewer warps.
+//   large (columns): radix-16 stages, sixteen elements a thread.  A grid of many rounds is
+//     bound by the shared-memory exchanges and twiddle loads together with the FP32 pipe;
+//     radix-16 stages take two thirds of the former, and many rounds make up for the fewer
+//     warps.  (Rows gain more from both pairs per thread, which evaluates the field once.)
 //   wide: the small form with column tiles of 256 threads, for small grids in a batch that
 //     fills the SMs anyway.  It differs in threads per CTA alone, so a member still equals
 //     itself run alone, bit for bit.
 constexpr int kFormSmall = 4, kFormLarge = 5, kFormWide = 6, kNumSweepForms = 7;
 __host__ __device__ constexpr SweepVariant sweep_form(int axis, int form) {
     if (form < kNumSweepVariants) return sweep_variant(axis, form);
-    if (axis == AXIS_X) return form == kFormLarge ? SweepVariant{4, 64, 1, 2, 16, 0} : SweepVariant{2, 64, 1, 2, 32, 0};
+    if (axis == AXIS_X) return SweepVariant{2, 64, 1, 2, 32, 0};
     return form == kFormSmall  ? SweepVariant{2, 64, 2, 2, 32, 0}
            : form == kFormWide ? SweepVariant{2, 256, 4, 2, 32, 0}
                                : SweepVariant{4, 256, 2, 2, 16, 0};
@@ -131,40 +132,46 @@ __host__ __device__ constexpr SweepVariant sweep_form(int axis, int form) {
 // axes and lengths a form is compiled for
 __host__ __device__ constexpr bool sweep_form_holds(int axis, int form, int logn) {
     return form == kFormSmall   ? logn <= 11
-           : form == kFormLarge ? logn >= 10
+           : form == kFormLarge ? axis == AXIS_Y && logn >= 10
            : form == kFormWide  ? axis == AXIS_Y && logn <= 9
                                 : true;
 }
 // The form that variant v runs on `lines` lines of 2^logn points.  The lines lie where the
-// measured times cross (GB300, us per sweep, default form against the chosen one):
-//   x, up to 2^17 points: 64x64 4.9 : 3.2, 256x256 5.6 : 4.2, 1024x128 7.4 : 6.5, 2048x64
-//     7.7 : 7.3; at 2^18 the radix-8 default is ahead (512x512 8.6 : 9.2);
-//   x, 2048 and 4096 points: both pairs per thread (variant 3, the field evaluated once) up to
-//     2^20 points (2048x128 12.9 : 10.9, 2048x256 18.7 : 15.5, 4096x256 40.0 : 33.1; variant
-//     1 takes 10.3 alone at 2048x128, but its 512-thread CTAs leave no room for the next
-//     sweep's to start under: 21.0 us a step against 18.7), then large (2048x512 29.7 : 27.8,
-//     4096x2048 288 : 234); 4096x64 is too few rows for variant 3 (11.1 : 16.7);
-//   y up to 512 points: small up to 2^16 points (64x64 5.4 : 2.2, 128x128 6.5 : 2.5, 256x256
-//     7.1 : 4.1), radix-4 tiles of both pairs at 2^17 (512x256 7.2 : 5.0);
-//   y from 1024 points (few columns): small up to 2^17 points (128x1024 15.6 : 7.0, 64x2048
-//     18.7 : 10.1), one pair per CTA at 2^18 (256x1024 15.8 : 9.8, 128x2048 18.8 : 11.2),
-//     then large (1024x1024 30.7 : 29.5, 2048x1024 61.6 : 54.6, 4096x2048 292 : 263).
+// times of whole runs cross (GB300, us per step, both sweeps; a sweep timed alone can mislead:
+// variant 1's 512-thread rows are the fastest at 2048x128 alone, 10.3 against 10.9 us, but leave
+// no room for the next sweep to start under, 21.8 against 19.5 a step).  Variant 0 : chosen:
+//   x small up to 2^16 points, for short rows up to 2^18 (with the chosen columns: 64x64 10.4 :
+//     5.3, 128x128 11.7 : 6.0, 256x256 13.4 : 8.6, 256x1024 21.1 : 17.3, 128x2048 22.0 : 18.8);
+//   x 512 and 1024 points at 2^17: variant 1, the field shared in a CTA (512x256 15.0 : 11.4,
+//     1024x128 15.3 : 11.5); at 2^18 and beyond variant 0 (512x512 18.7, small 22.2);
+//   x 2048 and 4096 points: both pairs per thread (variant 3) from 2^18 and 2^19 points on
+//     (2048x128 23.8 : 19.5, 2048x256 30.9 : 27.7; with large columns 2048x1024 118.2 : 118.0,
+//     2048x2048 267 : 252, 4096x2048 562 : 522; radix-16 rows 129, 265, 529); 4096x64 is too
+//     few rows for it (a sweep 11.1 : 16.7);
+//   y small up to 2^16 points (2^15 at 512), radix-4 tiles of both pairs at 2^17 up to 256
+//     points; one pair per CTA for few long columns (128x512 12.1 : 10.3, 256x512 15.3 : 12.3,
+//     128x1024 20.9 : 15.2, 64x2048 23.5 : 16.3, 256x1024 24.1 : 17.3 with small rows); large
+//     beyond (1024x1024 56.5 : 55.0, 2048x1024 125.5 : 118.2, 4096x2048 589 : 562).
 // crowded: other simulations run beside this one and fill the SMs (a batch).  The small
 // form's narrow column tiles, which spread one small grid over the SMs, then only cost memory
 // transactions: the wide form takes their place.  16 members of 128x128 ... 512x256: 20.5
 // against 21.7 G point-steps/s.
 inline int sweep_form_of(int axis, int v, int logn, int lines, bool crowded) {
     if (v > 1) return v;
-    if (crowded && axis == AXIS_Y && logn <= 9 && ((long long)lines << logn) <= 1 << 16) return kFormWide;
-    const long long points = (long long)lines << logn;
+    int logp = logn;   // log2 of the points (both counts are powers of two)
+    while ((lines >> (logp - logn)) > 1) ++logp;
     if (axis == AXIS_X) {
-        if (logn <= 11 && points <= 1 << 17) return kFormSmall;
-        if (logn <= 10 || points <= 1 << (logn == 11 ? 17 : 18)) return v;
-        return points < 1 << 20 ? 3 : kFormLarge;
+        if (logn <= 8) return logp <= 18 ? kFormSmall : v;
+        if (logn <= 10) return logp <= 16 ? kFormSmall : (logp == 17 ? 1 : v);
+        if (logn == 11) return logp <= 17 ? kFormSmall : 3;
+        return logp <= 18 ? v : 3;
     }
-    if (logn <= 9) return points <= 1 << 16 ? kFormSmall : (points <= 1 << 17 ? 2 : v);
-    if (logn <= 11 && points <= 1 << 17) return kFormSmall;
-    return points <= 1 << 18 ? 3 : kFormLarge;
+    if (logn <= 9) {
+        if (logp <= (logn == 9 ? 15 : 16)) return crowded ? kFormWide : kFormSmall;
+        return logp <= 17 ? (logn == 9 ? 3 : 2) : v;
+    }
+    if (logn <= 11 && logp <= 16) return kFormSmall;
+    return logp <= 18 ? 3 : kFormLarge;
 }
 
 __host__ __device__ constexpr int sweep_nc(int axis, int v) { return sweep_form(axis, v).nc; }
