@@ -501,8 +501,8 @@ def profile_persist(spec: str):
 
 def profile_mlp(spec: str):
     """The surrogate network's BF16 tensor-core GEMMs for a profiler: STEPS training steps
-    of the 5 -> 3 x 256 -> 4 network on BATCH seeded rows (each step: 4 forward, 7 backward
-    GEMMs of k_gemm_bf16)."""
+    of the 5 -> 3 x 256 -> 4 network on BATCH seeded rows (each step: 4 forward and 4 backward
+    launches of k_group<1>, the grouped BF16 products, and Adam)."""
     import torch
     from paper_2307_01571_gb300 import kd, surrogate as S
     batch, steps = (int(v) for v in spec.split(","))

@@ -314,9 +314,11 @@ int kd_bench_sweep(kd_sim* sim, int32_t kind, int32_t reps);
  * KD_TUNE_FORCE times again).  variant_x / variant_y (may be NULL) receive the choice,
  * times_ms (may be NULL, 2 * KD_SWEEP_VARIANTS floats: x then y) the measured ms per
  * launch (the recorded ones when the choice was looked up; -1 for FP64).  FP64
- * simulations have one variant (0).  Synchronises the simulation's stream: KD_ERR_ARG
+ * simulations have one variant (0).  What variants 0 and 1 launch follows the grid's size
+ * (small grids run radix-4 stages in small tiles, long rows both pairs per thread, large
+ * grids radix-16 column stages); 2 and 3 are fixed shapes.  Synchronises the simulation's stream: KD_ERR_ARG
  * while that stream is being captured (kd_set_sweep_variants likewise, when it changes the
- * variants).  Variants 0 and 1 differ only in threads per CTA and give
+ * variants).  Variants 0 and 1 differ at most in threads per CTA and give
  * bitwise identical results; the radix-4 schedule (2) and the components-per-CTA change
  * (3) round differently in the last bits (every variant meets the same accuracy).  A
  * simulation's results are reproducible for fixed variants.  kd_set_sweep_variants selects variants directly

@@ -1,7 +1,7 @@
 """Compiles the CUDA library ``libkd.so`` in-tree for sm_103a.
 
-The translation units (host API, the FP32 sweeps once per launch variant, the
-double-word sweeps once per axis and shape, the FP64 sweeps, the tensor-core sweeps, the allocation-free entry and the MLP kernels) compile in parallel with nvcc; the
+The translation units (host API, the FP32 sweeps once per launch variant and per form beyond
+them, the double-word sweeps once per axis and shape, the FP64 sweeps, the tensor-core sweeps, the allocation-free entry and the MLP kernels) compile in parallel with nvcc; the
 CUDA runtime is linked statically so the library only needs the driver.
 """
 from __future__ import annotations

@@ -78,7 +78,8 @@ struct SweepArgs {
 constexpr int KD_STATUS_NONFINITE = 1, KD_STATUS_DRIFT = 2, KD_STATUS_TC_TIMEOUT = 16;
 
 // Launch variants of the FP32 sweeps, timed per grid by the autotuner (kd_autotune);
-// variant 0 is the default.  A variant fixes the radix schedule (loge = log2 of the
+// variant 0 is the default.  The table is what 2 and 3 always run and 0 and 1 run where
+// sweep_form_of (below) has nothing better for the grid's size.  A variant fixes the radix schedule (loge = log2 of the
 // elements a thread owns: radix-8 or radix-4 Stockham stages), the threads per CTA (a
 // target: at least one whole line), the minimum column-tile width of the y sweep, the
 // spinor components per CTA (2: one 2x2 pair per CTA, the two pairs' CTAs side by side;

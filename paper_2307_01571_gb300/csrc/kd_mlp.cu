@@ -1,9 +1,10 @@
 // kd_mlp.cu -- the surrogate network: a fully connected MLP with exact-erf GELU hidden
 // layers, trained on the batched solver's outputs (seeded parameter draws -> diffraction
 // and spin-flip populations).  Hand-written kernels: tiled products with fused gather, bias,
-// GELU, GELU derivative and loss epilogues (FP32 on the CUDA cores, or BF16 operands on the tcgen05 tensor cores with FP32
-// accumulation in tensor memory), fixed-order column sums, the loss
-// sum and Adam.  Every reduction runs in a fixed order, so training is bitwise reproducible.
+// GELU, GELU derivative and loss epilogues (FP32 on the CUDA cores, or BF16 operands on the
+// tcgen05 tensor cores with FP32 accumulation in tensor memory), fixed-order column sums, the
+// loss sum and Adam.  Every reduction runs in a fixed order, so training is bitwise
+// reproducible.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -63,7 +64,9 @@ __device__ __forceinline__ float gelu_grad(float x) {
 // chain and by the load latency inside each one, not by arithmetic or memory: everything
 // pointwise (gather, bias, GELU and its derivative, the loss' gradient) sits in an epilogue
 // or a loader, and a launch starts under its predecessor's tail (programmatic dependent
-// launch).  Chain of a training step: L forward launches, L backward launches, Adam.
+// launch).  Such a launch may start before its predecessor's stores, so nothing here is read
+// through the non-coherent path.  Chain of a training step: L forward launches, L backward
+// launches, Adam.
 //
 // A step at batch 256 / FP32 went from 22 launches and 396 us to 9 launches and 43 us, at batch
 // 1024 / BF16 from 401 to 73 us (GB300, the 5-256-256-256-4 network).  What bounds it now is
@@ -131,7 +134,7 @@ template <int NE> __device__ __forceinline__ void epi_prefetch(const Product& q,
 #pragma unroll
     for (int i = 0; i < NE; ++i) {
         const int mi = m + i * mstep, ni = n + i * nstep;
-        z[i] = mi < q.M && ni < q.N ? __ldg(q.Z + (long)mi * q.N + ni) : 0.0f;
+        z[i] = mi < q.M && ni < q.N ? *(q.Z + (long)mi * q.N + ni) : 0.0f;
     }
 }
 template <int NE, int UNROLL, typename F>
@@ -148,7 +151,7 @@ __device__ __forceinline__ void epilogue(const Product& q, int m, int mstep, int
         each([&](int, int, long o, float x) { C[o] = x; });
     } else if (q.epi == EPI_BIAS_GELU) {
         each([&](int, int ni, long o, float x) {
-            x += __ldg(q.bias + ni);
+            x += *(q.bias + ni);
             q.Z[o] = x;
             q.C[o] = gelu(x);
         });
@@ -159,12 +162,12 @@ __device__ __forceinline__ void epilogue(const Product& q, int m, int mstep, int
             if (mi < q.M && ni < q.N) q.C[(long)mi * q.N + ni] = v(i) * gelu_grad(z[i]);
         }
     } else if (q.epi == EPI_BIAS) {
-        each([&](int, int ni, long o, float x) { q.C[o] = x + __ldg(q.bias + ni); });
+        each([&](int, int ni, long o, float x) { q.C[o] = x + *(q.bias + ni); });
     } else {
         each([&](int mi, int ni, long o, float x) {
             const long r = q.tidx ? q.tidx[mi] : mi;
-            const float t = !q.tidx || (r >= 0 && r < q.nt) ? __ldg(q.T + r * q.N + ni) : 0.0f;
-            x += __ldg(q.bias + ni);
+            const float t = !q.tidx || (r >= 0 && r < q.nt) ? *(q.T + r * q.N + ni) : 0.0f;
+            x += *(q.bias + ni);
             q.C[o] = x;
             const float d = x - t;
             q.dY[o] = q.scale * d;
@@ -200,7 +203,7 @@ __device__ void colsum_block(const ColSum& c, int blk) {
     const int m1 = min(c.M, (split + 1) * c.mper);
     float s = 0.0f;
     if (n < c.N)
-        for (int m = split * c.mper + g; m < m1; m += 8) s += __ldg(c.X + (long)m * c.N + n);
+        for (int m = split * c.mper + g; m < m1; m += 8) s += *(c.X + (long)m * c.N + n);
     red[g][threadIdx.x & 31] = s;
     __syncthreads();
     if (g == 0 && n < c.N) {
@@ -414,7 +417,7 @@ template <int ROWS, bool KC> __device__ __forceinline__ void tile_load(const Ope
 #pragma unroll
     for (int i = 0; i < ROWS / 8; ++i) {
         const long line = KC ? 8 * i : 64 * (i / KB) + i % KB;
-        s.v[i] = __ldg(reinterpret_cast<const float4*>(p + line * o.ld));
+        s.v[i] = *reinterpret_cast<const float4*>(p + line * o.ld);
     }
 }
 __device__ __forceinline__ float elem(const float4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
@@ -436,7 +439,7 @@ __device__ __forceinline__ void tile_store(unsigned char* dst, const Operand& o,
                     line = o.idx[line];
                     in = line >= 0 && line < o.nidx;
                 }
-                v[e] = in ? __ldg(o.p + line * o.ld + (KC ? k + e : row)) : 0.0f;
+                v[e] = in ? *(o.p + line * o.ld + (KC ? k + e : row)) : 0.0f;
             }
             *reinterpret_cast<uint4*>(cell(dst, row - r0, k - k0)) =
                 make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));

@@ -10,8 +10,9 @@
 // Between sweeps the state lives in (k_x, y) space.  The first and last x sweeps of a
 // run apply a true half step and only one of the two FFTs.
 //
-// FFT engine: Stockham autosort, radix 8/4/2, every thread owns E = 8 (FP32) or 4 (FP64)
-// elements of one line for all four spinor components in registers; butterflies run on
+// FFT engine: Stockham autosort, radix 16/8/4/2, every thread owns E elements (FP32 16, 8 or 4
+// by launch form, FP64 and double-word 4, 8 on long lines) of one line for one 2x2 pair of
+// spinor components, or both, in registers; butterflies run on
 // registers and stages exchange data through shared memory with an XOR swizzle that
 // keeps 16-byte accesses free of bank conflicts.  The last stage of the first FFT and the
 // first stage of the second FFT use the same radix and butterfly-to-thread map, so the
