@@ -110,7 +110,7 @@ __host__ __device__ constexpr SweepVariant sweep_variant(int axis, int v) {
 // spinor components per thread of the FP32 sweeps
 __host__ __device__ constexpr int sweep_nc(int axis, int v);
 
-// The compiled forms of the FP32 sweeps: 0 ... 3 the variants as in the table, and three that
+// The compiled forms of the FP32 sweeps: 0 ... 3 the variants as in the table, and two that
 // the default (variants 0 and 1) becomes by the grid's size, sweep_form_of below.
 //   small: radix-4 stages, one or two rows / two columns per CTA.  A small grid is bound by
 //     the latency of one CTA and by idle SMs: 128 columns of 128 points in tiles of eight
@@ -119,22 +119,16 @@ __host__ __device__ constexpr int sweep_nc(int axis, int v);
 //     bound by the shared-memory exchanges and twiddle loads together with the FP32 pipe;
 //     radix-16 stages take two thirds of the former, and many rounds make up for the fewer
 //     warps.  (Rows gain more from both pairs per thread, which evaluates the field once.)
-//   wide: the small form with column tiles of 256 threads, for small grids in a batch that
-//     fills the SMs anyway.  It differs in threads per CTA alone, so a member still equals
-//     itself run alone, bit for bit.
-constexpr int kFormSmall = 4, kFormLarge = 5, kFormWide = 6, kNumSweepForms = 7;
+constexpr int kFormSmall = 4, kFormLarge = 5, kNumSweepForms = 6;
 __host__ __device__ constexpr SweepVariant sweep_form(int axis, int form) {
     if (form < kNumSweepVariants) return sweep_variant(axis, form);
     if (axis == AXIS_X) return SweepVariant{2, 64, 1, 2, 32, 0};
-    return form == kFormSmall  ? SweepVariant{2, 64, 2, 2, 32, 0}
-           : form == kFormWide ? SweepVariant{2, 256, 4, 2, 32, 0}
-                               : SweepVariant{4, 256, 2, 2, 16, 0};
+    return form == kFormSmall ? SweepVariant{2, 64, 2, 2, 32, 0} : SweepVariant{4, 256, 2, 2, 16, 0};
 }
 // axes and lengths a form is compiled for
 __host__ __device__ constexpr bool sweep_form_holds(int axis, int form, int logn) {
     return form == kFormSmall   ? logn <= 11
            : form == kFormLarge ? axis == AXIS_Y && logn >= 10
-           : form == kFormWide  ? axis == AXIS_Y && logn <= 9
                                 : true;
 }
 // The form that variant v runs on `lines` lines of 2^logn points.  The lines lie where the
@@ -155,8 +149,9 @@ __host__ __device__ constexpr bool sweep_form_holds(int axis, int form, int logn
 //     beyond (1024x1024 56.5 : 55.0, 2048x1024 125.5 : 118.2, 4096x2048 589 : 562).
 // crowded: other simulations run beside this one and fill the SMs (a batch).  The small
 // form's narrow column tiles, which spread one small grid over the SMs, then only cost memory
-// transactions: the wide form takes their place.  16 members of 128x128 ... 512x256: 20.5
-// against 21.7 G point-steps/s.
+// transactions: variant 2's tiles take their place.  Their kinetic step is written to round
+// like the small form's, so a member still equals itself run alone, bit for bit.  16 members
+// of 128x128 ... 512x256: 20.5 against 23.4 G point-steps/s.
 inline int sweep_form_of(int axis, int v, int logn, int lines, bool crowded) {
     if (v > 1) return v;
     int logp = logn;   // log2 of the points (both counts are powers of two)
@@ -168,7 +163,7 @@ inline int sweep_form_of(int axis, int v, int logn, int lines, bool crowded) {
         return logp <= 18 ? v : 3;
     }
     if (logn <= 9) {
-        if (logp <= (logn == 9 ? 15 : 16)) return crowded ? kFormWide : kFormSmall;
+        if (logp <= (logn == 9 ? 15 : 16)) return crowded ? 2 : kFormSmall;
         return logp <= 17 ? (logn == 9 ? 3 : 2) : v;
     }
     if (logn <= 11 && logp <= 16) return kFormSmall;

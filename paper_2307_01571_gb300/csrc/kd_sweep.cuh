@@ -914,6 +914,18 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
                     const int pr = NC == 4 ? q : c.pair;
                     const T piy = pr == 0 ? yv.x : -yv.x;
                     const C u = e[2 * q], l = e[2 * q + 1];
+                    if constexpr (sizeof(T) == 4 && (V == 2 || V == kFormSmall)) {
+                        // the expressions below with every fusion written out, so that these two
+                        // forms, which differ in components per thread, round alike (a crowded
+                        // batch swaps them); psi + (f psi) keeps one rounding around psi itself
+                        const C hu = mk<C>(fmaf(piy, l.y, fmaf(pix, l.x, mc * u.x)), fmaf(-piy, l.x, fmaf(pix, l.y, mc * u.y)));
+                        const C hl = mk<C>(fmaf(-mc, l.x, fmaf(-piy, u.y, pix * u.x)), fmaf(-mc, l.y, fmaf(piy, u.x, pix * u.y)));
+                        const C u1 = mk<C>(fmaf(u.x, invP, fmaf(ab.y, hu.y, ab.x * u.x)), fmaf(u.y, invP, fmaf(-ab.y, hu.x, ab.x * u.y)));
+                        const C l1 = mk<C>(fmaf(l.x, invP, fmaf(ab.y, hl.y, ab.x * l.x)), fmaf(l.y, invP, fmaf(-ab.y, hl.x, ab.x * l.y)));
+                        e[2 * q] = mk<C>(__fadd_rn(u1.x, fmaf(yv.y, u1.x, -yv.z * u1.y)), __fadd_rn(u1.y, fmaf(yv.y, u1.y, yv.z * u1.x)));
+                        e[2 * q + 1] = mk<C>(__fadd_rn(l1.x, fmaf(yv.y, l1.x, -yv.z * l1.y)), __fadd_rn(l1.y, fmaf(yv.y, l1.y, yv.z * l1.x)));
+                        continue;
+                    }
                     // G = H0/c on the pair: (mc u + (pix - i piy) l, (pix + i piy) u - mc l)
                     const C hu = mk<C>(mc * u.x + pix * l.x + piy * l.y, mc * u.y + pix * l.y - piy * l.x);
                     const C hl = mk<C>(pix * u.x - piy * u.y - mc * l.x, pix * u.y + piy * u.x - mc * l.y);
