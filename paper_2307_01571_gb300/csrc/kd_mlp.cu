@@ -701,6 +701,15 @@ cudaError_t launch_pdl(void (*k)(KP...), long grid, int threads, int smem, cudaS
     return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
+// Lets the products' kernel of a precision take its dynamic shared memory on the current
+// device.  The limit belongs to one device's copy of the kernel, so every network sets it for
+// its own device (kd_mlp_create, kd_mlp_set_precision) and nothing remembers it.
+cudaError_t allow_smem(int precision) {
+    return precision == KD_MLP_BF16
+        ? cudaFuncSetAttribute(k_group<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tcg::SMEM)
+        : cudaFuncSetAttribute(k_group<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, fp32::SMEM);
+}
+
 cudaError_t launch_group(const kd_mlp* n, Group& g, int nprod, cudaStream_t s) {
     long b = 0;
     for (int i = 0; i < 2; ++i) {
@@ -718,10 +727,6 @@ cudaError_t launch_group(const kd_mlp* n, Group& g, int nprod, cudaStream_t s) {
     // BF16: two 41 KB stages and 32 columns of tensor memory per CTA: two CTAs per SM, whose
     // columns fit the SM's 512, so no allocation waits
     const int smem = bf ? (int)tcg::SMEM : fp32::SMEM;
-    static const cudaError_t attr[2] = {
-        cudaFuncSetAttribute(k_group<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, fp32::SMEM),
-        cudaFuncSetAttribute(k_group<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tcg::SMEM)};
-    if (attr[bf] != cudaSuccess) return attr[bf];
     return bf ? launch_pdl(k_group<1>, b, 256, smem, s, g) : launch_pdl(k_group<0>, b, 256, smem, s, g);
 }
 
@@ -940,6 +945,7 @@ int kd_mlp_create(const int32_t* widths, int32_t nlayers, kd_mlp** out) {
     }
     n->nparam = off;
     auto bail = [&](int rc) { kd_mlp_destroy(n); return rc; };
+    if (allow_smem(KD_MLP_FP32) != cudaSuccess) return bail(err(KD_ERR_CUDA, "kd_mlp_create: shared-memory limit refused"));
     if (cudaMalloc(&n->param, off * sizeof(float)) != cudaSuccess || cudaMalloc(&n->grad, off * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&n->m1, off * sizeof(float)) != cudaSuccess || cudaMalloc(&n->m2, off * sizeof(float)) != cudaSuccess)
         return bail(err(KD_ERR_NOMEM, "kd_mlp_create: allocation failed"));
@@ -1002,6 +1008,10 @@ int kd_mlp_get_params(kd_mlp* n, float* p, int32_t where) {
 int kd_mlp_set_precision(kd_mlp* n, int32_t precision) {
     if (!n || (precision != KD_MLP_FP32 && precision != KD_MLP_BF16))
         return err(KD_ERR_ARG, "kd_mlp_set_precision: KD_MLP_FP32 or KD_MLP_BF16");
+    if (precision != n->prec) {
+        MLP_CUDA(cudaSetDevice(n->device));
+        MLP_CUDA(allow_smem(precision));
+    }
     n->prec = precision;
     return KD_OK;
 }

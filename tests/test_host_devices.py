@@ -1,0 +1,84 @@
+"""The library's host code on a fake CUDA runtime with two devices (tests/fake/cudart.cpp),
+without a GPU: the compiled objects of the build linked with the fake in place of the CUDA
+runtime, kernels checked against their launch limits and not run."""
+import ctypes as C
+import glob
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2307_01571_gb300 import _build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+KD_DEVICE, KD_HOST = 1, 0
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    objs = [os.path.join(_build.BUILD, o) for _, o, _ in _build.UNITS]
+    _build.build(force=not all(os.path.exists(o) for o in objs))
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_build._nvcc())))
+    inc = [d for d in glob.glob(os.path.join(cuda, "include")) + glob.glob(os.path.join(cuda, "targets", "*", "include"))
+           if os.path.exists(os.path.join(d, "cuda_runtime_api.h"))]
+    out = str(tmp_path_factory.mktemp("fake") / "libkd_fake.so")
+    r = subprocess.run([shutil.which("g++"), "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-Wl,-z,defs",
+                        *[f"-I{d}" for d in inc], os.path.join(HERE, "fake", "cudart.cpp"), *objs, "-o", out],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
+    return C.CDLL(out)
+
+
+@pytest.fixture
+def fake(lib):
+    yield lib
+    lib.fake_fail_malloc(-1)
+    lib.fake_capture_query_error(0)
+    lib.fake_refuse_attribute(0)
+    lib.fake_set_device(0)
+
+
+def _net(lib, widths):
+    h = C.c_void_p()
+    arr = (C.c_int32 * len(widths))(*widths)
+    return lib.kd_mlp_create(arr, len(widths) - 1, C.byref(h)), h
+
+
+def _train(lib, h, batch=8):
+    x = np.zeros(1 << 16, np.float32)
+    p = C.c_void_p(x.ctypes.data)
+    return lib.kd_mlp_train_step(h, p, p, batch, C.c_float(1e-3), None, None)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_networks_train_on_every_device(fake, precision):
+    """The shared-memory limit that the products' kernels need is set on each device that holds
+    a network, whichever device held the first one."""
+    for dev in (0, 1, 0):
+        assert fake.fake_set_device(dev) == 0
+        rc, h = _net(fake, [5, 64, 4])
+        assert rc == 0
+        assert fake.kd_mlp_set_precision(h, precision) == 0
+        before = fake.fake_launches()
+        assert _train(fake, h) == 0, dev
+        assert fake.fake_launches() > before
+        fake.kd_mlp_destroy(h)
+
+
+def test_a_refused_limit_is_not_remembered(fake):
+    """A network whose device refuses the limit is not made (or not switched to BF16); later
+    ones are."""
+    fake.fake_refuse_attribute(1)
+    rc, h = _net(fake, [5, 64, 4])
+    assert rc != 0 and not h
+    fake.fake_refuse_attribute(0)
+    rc, h = _net(fake, [5, 64, 4])
+    assert rc == 0
+    fake.fake_refuse_attribute(1)
+    assert fake.kd_mlp_set_precision(h, 1) != 0
+    assert _train(fake, h) == 0            # still an FP32 network
+    fake.fake_refuse_attribute(0)
+    assert fake.kd_mlp_set_precision(h, 1) == 0 and _train(fake, h) == 0
+    fake.kd_mlp_destroy(h)
