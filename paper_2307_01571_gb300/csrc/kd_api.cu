@@ -42,6 +42,7 @@ int fail(int code, const char* fmt, ...) {
     vsnprintf(buf, sizeof buf, fmt, ap);
     va_end(ap);
     g_err = buf;
+    cudaGetLastError();   // reported here: a later call's launch check must not report it again
     return code;
 }
 
@@ -2020,9 +2021,12 @@ int kd_batch_create(kd_sim* const* sims, int32_t n, void* cuda_stream, kd_batch*
         std::map<std::pair<int, int>, int> seen;
         for (kd_sim* s : b->sims) {
             cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-            if (s->prec == KD_FP64 || seen[{s->lx, s->ly}]++ || cudaStreamIsCapturing(s->stream, &cs) != cudaSuccess ||
-                cs != cudaStreamCaptureStatusNone)
+            if (s->prec == KD_FP64 || seen[{s->lx, s->ly}]++) continue;
+            if (cudaStreamIsCapturing(s->stream, &cs) != cudaSuccess) {
+                cudaGetLastError();
                 continue;
+            }
+            if (cs != cudaStreamCaptureStatusNone) continue;
             s->crowded = true;
             int rc = warm_variants(s);
             s->crowded = false;

@@ -82,3 +82,34 @@ def test_a_refused_limit_is_not_remembered(fake):
     fake.fake_refuse_attribute(0)
     assert fake.kd_mlp_set_precision(h, 1) == 0 and _train(fake, h) == 0
     fake.kd_mlp_destroy(h)
+
+
+def _sim(lib, nx, ny, precision):
+    from paper_2307_01571_gb300 import kd, workloads as W
+    wl = W.small(nx, ny, W.GAUSS, units=W.ATOMIC)
+    h = C.c_void_p()
+    rc = lib.kd_create(C.byref(kd._fill(kd.kd_units, wl.units)), C.byref(kd._fill(kd.kd_grid, wl.grid)),
+                       C.byref(kd._fill(kd.kd_field, wl.field)), precision, None, C.byref(h))
+    return rc, h, wl
+
+
+def test_an_error_is_reported_once(fake):
+    """A call that failed inside the runtime, or a query whose failure a call gets over, leaves
+    nothing behind that a later call's launch check would report as its own."""
+    rc, h = _net(fake, [5, 64, 4])
+    assert rc == 0
+    fake.fake_fail_malloc(0)
+    assert _train(fake, h) != 0
+    assert fake.fake_last_error() == 0
+    made = [_sim(fake, 512, 512, 1) for _ in range(2)]          # together they fill the SMs
+    assert all(rc == 0 for rc, _, _ in made)
+    fake.fake_capture_query_error(1)
+    b = C.c_void_p()
+    assert fake.kd_batch_create((C.c_void_p * 2)(*[s for _, s, _ in made]), 2, None, C.byref(b)) == 0
+    assert fake.fake_last_error() == 0
+    fake.fake_capture_query_error(0)
+    assert fake.kd_get_density_x(made[0][1], np.zeros(512).ctypes.data_as(C.c_void_p), KD_HOST) == 0
+    fake.kd_batch_destroy(b)
+    for _, s, _ in made:
+        fake.kd_destroy(s)
+    fake.kd_mlp_destroy(h)
