@@ -4,7 +4,23 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace kd {
+
+// Lets kernel k take `bytes` of dynamic shared memory on the current device.  The limit belongs
+// to one device's copy of the kernel: `done` holds one bit per device that accepted it (devices
+// beyond the 64th are asked every time).
+template <typename K> cudaError_t allow_smem(K k, int bytes, std::atomic<uint64_t>& done) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev < 64 ? (uint64_t)1 << dev : 0;
+    if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+}
 
 // Internal spinor layout: two pair planes [pair][ny][nx][2] complex.  In 2D with
 // A = (A_x, A_y) and p = (p_x, p_y) both alpha.A and alpha.p + beta couple only

@@ -255,26 +255,23 @@ void persist_variants(int axis, int logn, int* v0, int* v1) {
 }
 
 cudaError_t launch_persist(const PersistPlan& p, cudaStream_t s) {
-    static int smem = 0, grid = 0;
-    if (grid == 0) {
-        int m = 0;
-        const int sm[] = {max_smem<4>(), max_smem<5>(), max_smem<6>(), max_smem<7>(),
-                          max_smem<8>(), max_smem<9>()};
-        for (int v : sm) m = v > m ? v : m;
-        cudaError_t e = cudaFuncSetAttribute(k_persist, cudaFuncAttributeMaxDynamicSharedMemorySize, m);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, dev = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_persist, kThreads, m);
-        if (e != cudaSuccess) return e;
-        e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        if (per_sm < 1) return cudaErrorInvalidConfiguration;
-        smem = m;
-        grid = per_sm * sms;
-    }
-    k_persist<<<grid, kThreads, smem, s>>>(p);
+    static std::atomic<uint64_t> allowed{0};
+    int smem = 0;
+    const int sm[] = {max_smem<4>(), max_smem<5>(), max_smem<6>(), max_smem<7>(),
+                      max_smem<8>(), max_smem<9>()};
+    for (int v : sm) smem = v > smem ? v : smem;
+    cudaError_t e = allow_smem(k_persist, smem, allowed);
+    if (e != cudaSuccess) return e;
+    // as many CTAs as the current device holds (asked once per captured graph)
+    int per_sm = 0, dev = 0, sms = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_persist, kThreads, smem);
+    if (e != cudaSuccess) return e;
+    e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    k_persist<<<per_sm * sms, kThreads, smem, s>>>(p);
     return cudaGetLastError();
 }
 

@@ -1002,14 +1002,10 @@ sweep_kernel(const SweepArgs a) {
 template <typename T, int LOGN, int AXIS, int SHAPE, int V>
 cudaError_t launch_one(const SweepArgs& a, cudaStream_t s) {
     using Cf = Cfg<T, LOGN, AXIS, V>;
-    static bool attr_done = false;
+    static std::atomic<uint64_t> allowed{0};
     auto k = sweep_kernel<T, LOGN, AXIS, SHAPE, V>;
-    if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              Cf::SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        attr_done = true;
-    }
+    cudaError_t e = allow_smem(k, Cf::SMEM_BYTES, allowed);
+    if (e != cudaSuccess) return e;
     const int lines = AXIS == AXIS_X ? a.ny : a.nx;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(((lines + Cf::BATCH - 1) / Cf::BATCH) * Cf::NPAIRS);

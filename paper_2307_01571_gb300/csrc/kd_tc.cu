@@ -450,20 +450,13 @@ __global__ void __launch_bounds__(THREADS, 2) tc_sweep(const SweepArgs a) {
 bool tc_supported(int logn) { return logn == 10; }
 
 cudaError_t launch_tc_sweep(int axis, const SweepArgs& a, cudaStream_t s) {
-    static bool attr_done[2] = {false, false};
-    static int nsm = 0;
+    static std::atomic<uint64_t> allowed[2];
     auto k = axis == AXIS_X ? tc::tc_sweep<AXIS_X> : tc::tc_sweep<AXIS_Y>;
-    if (!attr_done[axis]) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM);
-        if (e != cudaSuccess) return e;
-        attr_done[axis] = true;
-    }
-    if (nsm == 0) {
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-    }
+    int nsm = 0, dev = 0;
+    cudaError_t e = allow_smem(k, tc::SMEM, allowed[axis]);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
     const int lines = axis == AXIS_X ? a.ny : a.nx;
     const int items = 2 * (lines / tc::LC);
     const int grid = items < 2 * nsm ? items : 2 * nsm;

@@ -113,3 +113,30 @@ def test_an_error_is_reported_once(fake):
     for _, s, _ in made:
         fake.kd_destroy(s)
     fake.kd_mlp_destroy(h)
+
+
+# FP64, FP32, FP32 on the tensor cores, double-word; sizes whose sweeps need the raised limit
+@pytest.mark.parametrize("precision,nx,ny", [(0, 2048, 1024), (1, 1024, 512), (2, 1024, 64), (3, 1024, 1024)])
+def test_simulations_step_on_every_device(fake, precision, nx, ny):
+    """As for the networks: the sweeps' limits on both devices."""
+    for dev in (0, 1, 0):
+        assert fake.fake_set_device(dev) == 0
+        rc, h, wl = _sim(fake, nx, ny, precision)
+        assert rc == 0, dev
+        assert fake.kd_step(h, C.c_double(wl.dt), C.c_int64(3), C.c_int64(0), None, C.c_int64(0), None) == 0, dev
+        fake.kd_destroy(h)
+
+
+def test_persistent_batches_step_on_every_device(fake):
+    for dev in (0, 1):
+        assert fake.fake_set_device(dev) == 0
+        made = [_sim(fake, 512, 64, 1) for _ in range(2)]
+        assert all(rc == 0 for rc, _, _ in made)
+        b = C.c_void_p()
+        assert fake.kd_batch_create((C.c_void_p * 2)(*[h for _, h, _ in made]), 2, None, C.byref(b)) == 0
+        assert fake.kd_batch_set_mode(b, 1) == 0
+        dt = (C.c_double * 2)(made[0][2].dt, made[0][2].dt)
+        assert fake.kd_batch_step(b, dt, C.c_int64(3), C.c_int64(0), None, C.c_int64(0), None) == 0, dev
+        fake.kd_batch_destroy(b)
+        for _, h, _ in made:
+            fake.kd_destroy(h)
