@@ -753,6 +753,9 @@ int ensure_cap(kd_mlp* n, int batch) {
     cudaFree(n->dbuf0);
     cudaFree(n->dbuf1);
     cudaFree(n->lossbuf);
+    // nothing is left to use or free again if one of the allocations below fails
+    n->cap = 0;
+    n->dbuf0 = n->dbuf1 = n->lossbuf = nullptr;
     n->z.assign(n->L, nullptr);
     n->a.assign(n->L + 1, nullptr);
     for (int l = 0; l < n->L; ++l) {

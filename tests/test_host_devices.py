@@ -140,3 +140,25 @@ def test_persistent_batches_step_on_every_device(fake):
         fake.kd_batch_destroy(b)
         for _, h, _ in made:
             fake.kd_destroy(h)
+
+
+def test_batch_buffers_after_a_failed_allocation(fake):
+    """Every allocation that a larger batch needs fails in turn: the call reports it, and the
+    next calls, at the old batch size and at the new one, use and free no buffer of the old
+    set (the fake runtime counts frees of memory that is not live)."""
+    for k in range(16):
+        rc, h = _net(fake, [5, 64, 64, 4])
+        assert rc == 0 and _train(fake, h, 8) == 0
+        live = fake.fake_live()
+        fake.fake_fail_malloc(k)
+        rc = _train(fake, h, 300)
+        fake.fake_fail_malloc(-1)
+        if rc == 0:             # more than the call allocates
+            fake.kd_mlp_destroy(h)
+            break
+        assert rc == -8, (k, rc)      # KD_ERR_NOMEM
+        assert _train(fake, h, 8) == 0 and fake.fake_live() >= live
+        assert _train(fake, h, 300) == 0
+        fake.kd_mlp_destroy(h)
+        assert fake.fake_bad_frees() == 0, k
+    assert k > 6 and fake.fake_bad_frees() == 0
