@@ -81,10 +81,11 @@ def peaks():
 
 
 def kernel_source_hash() -> str:
+    """Hash of every source that the sweep kernels are compiled from."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2307_01571_gb300", "csrc")
-    for f in ("kd_sweep.cuh", "kd_sweep_f32.cu", "kd_sweep_f64.cu", "kd_internal.h", "kd_dw.cuh",
-              "kd_sweep_dw.cu"):
+    for f in ("kd_sweep.cuh", "kd_sweep_f32.cu", "kd_sweep_f32_forms.cu", "kd_sweep_f64.cu", "kd_internal.h",
+              "kd_dw.cuh", "kd_sweep_dw.cu"):
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

@@ -65,3 +65,29 @@ def test_issue_bound_reads_the_committed_counts_only_for_the_current_source():
     # launch variants other than the profiled ones: no count
     r2 = bench.roofline_issue("fp32", {"x_sweep": 0.0131}, 2070.0, 152, profiled_variants=False)
     assert r2["kernels"]["x_sweep"]["frac"] is None
+
+
+def test_kernel_hash_covers_every_source_of_the_sweeps(tmp_path, monkeypatch):
+    """A change of any file that a sweep object is compiled from, its own includes with it,
+    makes the committed counts of another source unreadable."""
+    import os
+    import re
+    import shutil
+
+    import bench
+    from paper_2307_01571_gb300 import _build
+    csrc = os.path.join(str(tmp_path), "paper_2307_01571_gb300", "csrc")
+    shutil.copytree(_build.CSRC, csrc)
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    files, todo = set(), {src for src, _, _ in _build.UNITS if "sweep" in src}
+    while todo:
+        f = todo.pop()
+        files.add(f)
+        text = open(os.path.join(csrc, f)).read()
+        todo |= {i for i in re.findall(r'#include "(kd_[^"]+)"', text) if i not in files}
+    assert len(files) >= 6
+    for f in sorted(files):
+        before = bench.kernel_source_hash()
+        with open(os.path.join(csrc, f), "a") as fh:
+            fh.write("// changed\n")
+        assert bench.kernel_source_hash() != before, f
