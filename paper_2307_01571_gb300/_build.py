@@ -21,7 +21,7 @@ SWEEP_VARIANTS = 4    # KD_SWEEP_VARIANTS in csrc/kd_internal.h
 UNITS = ([("kd_api.cu", "kd_api.o", [])]
          + [("kd_sweep_f32.cu", f"kd_sweep_f32_v{v}.o", [f"-DKD_SWEEP_VARIANT={v}"])
             for v in range(SWEEP_VARIANTS)]
-         + [("kd_sweep_f32_forms.cu", f"kd_sweep_f32_form{v}.o", [f"-DKD_SWEEP_FORM={v}"]) for v in (4, 5)]
+         + [("kd_sweep_f32_forms.cu", f"kd_sweep_f32_form{v}.o", [f"-DKD_SWEEP_FORM={v}"]) for v in (4, 5, 6, 7, 8)]
          + [("kd_sweep_dw.cu", f"kd_sweep_dw_p{p}.o", [f"-DKD_DW_PART={p}"]) for p in range(6)]
          + [("kd_sweep_f64.cu", "kd_sweep_f64.o", []), ("kd_tc.cu", "kd_tc.o", []),
             ("kd_noalloc.cu", "kd_noalloc.o", []), ("kd_mlp.cu", "kd_mlp.o", []),

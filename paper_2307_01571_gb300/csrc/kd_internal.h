@@ -126,26 +126,41 @@ __host__ __device__ constexpr SweepVariant sweep_variant(int axis, int v) {
 // spinor components per thread of the FP32 sweeps
 __host__ __device__ constexpr int sweep_nc(int axis, int v);
 
-// The compiled forms of the FP32 sweeps: 0 ... 3 the variants as in the table, and two that
+// The compiled forms of the FP32 sweeps: 0 ... 3 the variants as in the table, and those that
 // the default (variants 0 and 1) becomes by the grid's size, sweep_form_of below.
 //   small: radix-4 stages, one or two rows / two columns per CTA.  A small grid is bound by
 //     the latency of one CTA and by idle SMs: 128 columns of 128 points in tiles of eight
 //     columns and both pairs were 16 CTAs on 152 SMs.
+//   tall (columns): radix-8 stages, one column per CTA, for at most 32 columns of 1024 and 2048
+//     points, where three stages instead of five or six outweigh the 16-byte rows of the tile
+//     (us a step, small : tall: 16x1024 9.91 : 9.46, 32x1024 10.00 : 9.75, 32x2048 13.85 :
+//     13.59; but 64x1024 11.1 : 14.8).
 //   large (columns): radix-16 stages, sixteen elements a thread.  A grid of many rounds is
 //     bound by the shared-memory exchanges and twiddle loads together with the FP32 pipe;
 //     radix-16 stages take two thirds of the former, and many rounds make up for the fewer
 //     warps.  (Rows gain more from both pairs per thread, which evaluates the field once.)
-constexpr int kFormSmall = 4, kFormLarge = 5, kNumSweepForms = 6;
+//   wide, tall wide: what members of a batch that fills the SMs run in the place of small and of
+//     the long columns' forms: both pairs per thread, rows in CTAs of 256 threads, columns in
+//     tiles of 256 threads (two columns at 512 points, where four would take 512).
+// Radix-4 forms, and tall with its stand-in, round alike: their pointwise steps have every
+// fusion written out, so that components per thread do not change a bit.
+constexpr int kFormSmall = 4, kFormLarge = 5, kFormWide = 6, kFormTall = 7, kFormTallWide = 8, kNumSweepForms = 9;
 __host__ __device__ constexpr SweepVariant sweep_form(int axis, int form) {
     if (form < kNumSweepVariants) return sweep_variant(axis, form);
+    if (form == kFormWide) return axis == AXIS_X ? SweepVariant{2, 256, 1, 4, 24, 0} : SweepVariant{2, 256, 2, 4, 24, 0};
+    if (form == kFormTall) return SweepVariant{3, 64, 1, 2, 28, 0};
+    if (form == kFormTallWide) return SweepVariant{3, 256, 4, 4, 16, 0};
     if (axis == AXIS_X) return SweepVariant{2, 64, 1, 2, 32, 0};
     return form == kFormSmall ? SweepVariant{2, 64, 2, 2, 32, 0} : SweepVariant{4, 256, 2, 2, 16, 0};
 }
 // axes and lengths a form is compiled for
 __host__ __device__ constexpr bool sweep_form_holds(int axis, int form, int logn) {
-    return form == kFormSmall   ? logn <= 11
-           : form == kFormLarge ? axis == AXIS_Y && logn >= 10
-                                : true;
+    return form == kFormSmall      ? logn <= (axis == AXIS_X ? 11 : 10)
+           : form == kFormWide     ? logn <= (axis == AXIS_X ? 11 : 9)
+           : form == kFormTall     ? axis == AXIS_Y && (logn == 10 || logn == 11)
+           : form == kFormTallWide ? axis == AXIS_Y && logn >= 10
+           : form == kFormLarge    ? axis == AXIS_Y && logn >= 10
+                                   : true;
 }
 // The form that variant v runs on `lines` lines of 2^logn points.  The lines lie where the
 // times of whole runs cross (GB300, us per step, both sweeps; a sweep timed alone can mislead:
@@ -159,31 +174,43 @@ __host__ __device__ constexpr bool sweep_form_holds(int axis, int form, int logn
 //     (2048x128 23.8 : 19.5, 2048x256 30.9 : 27.7; with large columns 2048x1024 118.2 : 118.0,
 //     2048x2048 267 : 252, 4096x2048 562 : 522; radix-16 rows 129, 265, 529); 4096x64 is too
 //     few rows for it (a sweep 11.1 : 16.7);
-//   y small up to 2^16 points (2^15 at 512), radix-4 tiles of both pairs at 2^17 up to 256
-//     points; one pair per CTA for few long columns (128x512 12.1 : 10.3, 256x512 15.3 : 12.3,
+//   x 2048 points at 2^17: variant 0 (13.1 with small rows, 11.9);
+//   y small up to 2^16 points (2^15 at 512, tall for few columns of 1024 and more), radix-4
+//     tiles of both pairs (wide) at 2^17 up to 256 points; one pair per CTA for few long columns (128x512 12.1 : 10.3, 256x512 15.3 : 12.3,
 //     128x1024 20.9 : 15.2, 64x2048 23.5 : 16.3, 256x1024 24.1 : 17.3 with small rows); large
 //     beyond (1024x1024 56.5 : 55.0, 2048x1024 125.5 : 118.2, 4096x2048 589 : 562).
-// crowded: other simulations run beside this one and fill the SMs (a batch).  The small
-// form's narrow column tiles, which spread one small grid over the SMs, then only cost memory
-// transactions: variant 2's tiles take their place.  Their kinetic step is written to round
-// like the small form's, so a member still equals itself run alone, bit for bit.  16 members
-// of 128x128 ... 512x256: 20.5 against 23.4 G point-steps/s.
+// crowded: other simulations run beside this one and fill the SMs (a batch).  The narrow tiles
+// that spread one small grid over the SMs then only cost: the field, the twiddles and the index
+// work of each pair of components, and memory transactions.  The wide forms take their place,
+// with the same arithmetic, so that a member still equals itself run alone, bit for bit (which
+// rules the radix-8 shapes out where a grid alone runs radix-4 stages).  G point-steps/s of a
+// batch, its members' forms when alone (columns: variant 2's tiles) : radix-8 shapes of the
+// table's variant 0 : here:
+//   256 of 256x128 20.9 : 22.7 : 22.8, 256 of 128x128 17.3 : 18.0 : 18.6, 64 of 256x256 20.4 :
+//   22.1 : 21.9, 64 of 128x512 19.8 : 21.0 : 21.7, 64 of 1024x64 20.4 : 23.0 : 24.1, 32 of
+//   32x2048 14.3 : 19.7 : 20.3, 32 of 128x1024 17.7 : 19.3 : 19.6, 64 mixed 20.1 : 19.4 : 20.6;
+//   radix-4 stages of 512 points and more, and 256-point columns at 2^17 points, stay behind:
+//   64 of 64x512 18.6 : 24.3 : 21.4, 64 of 64x1024 16.6 : 19.3 : 16.7, 32 of 512x256 22.4 :
+//   23.3 : 22.5 (alone these grids take 7.5, 11.1 and 11.6 us a step; variant 0's shapes 12.9,
+//   20.6 and 15.0).
 inline int sweep_form_of(int axis, int v, int logn, int lines, bool crowded) {
     if (v > 1) return v;
     int logp = logn;   // log2 of the points (both counts are powers of two)
     while ((lines >> (logp - logn)) > 1) ++logp;
     if (axis == AXIS_X) {
-        if (logn <= 8) return logp <= 18 ? kFormSmall : v;
-        if (logn <= 10) return logp <= 16 ? kFormSmall : (logp == 17 ? 1 : v);
-        if (logn == 11) return logp <= 17 ? kFormSmall : 3;
+        const int small = crowded ? kFormWide : kFormSmall;
+        if (logn <= 8) return logp <= 18 ? small : v;
+        if (logn <= 10) return logp <= 16 ? small : (logp == 17 ? 1 : v);
+        if (logn == 11) return logp <= 16 ? small : (logp == 17 ? v : 3);
         return logp <= 18 ? v : 3;
     }
     if (logn <= 9) {
-        if (logp <= (logn == 9 ? 15 : 16)) return crowded ? 2 : kFormSmall;
-        return logp <= 17 ? (logn == 9 ? 3 : 2) : v;
+        if (logp <= (logn == 9 ? 15 : 16)) return crowded ? kFormWide : kFormSmall;
+        return logp <= 17 ? (logn == 9 ? 3 : kFormWide) : v;
     }
-    if (logn <= 11 && logp <= 16) return kFormSmall;
-    return logp <= 18 ? 3 : kFormLarge;
+    if (logp > 18) return kFormLarge;
+    if (lines == 64 && logn == 10) return kFormSmall;
+    return crowded ? kFormTallWide : (logp <= 16 && logn <= 11 ? kFormTall : 3);
 }
 
 __host__ __device__ constexpr int sweep_nc(int axis, int v) { return sweep_form(axis, v).nc; }

@@ -226,8 +226,9 @@ template <typename T, int LOGN, int AXIS, int V> struct Cfg {
     static constexpr int E = 1 << LOGE;                          // elements per thread
     static constexpr int TF = N / E;                             // threads per line
     // lines per CTA (FP32): rows are batched up to the variant's thread count; column tiles
-    // take that many threads and at least MINB columns, i.e. >= 64 contiguous bytes per tile
-    // row, within 512 threads
+    // take that many threads and at least MINB columns, within 512 threads: the table's shapes
+    // read 64 contiguous bytes of a tile row and more, the narrow forms 16 (one column of a
+    // pair) or 32
     static constexpr int MINB = DWT ? 2 : VS.minb;
     // field sharing between the two pairs of a line (x axis, one pair per thread)
     static constexpr bool SHARE = AXIS == AXIS_X && NC == 2 && (DWT ? TF <= 128 : !F64 && TF <= 256 && VS.share != 0);
@@ -823,6 +824,14 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
             const int pr = NC == 4 ? q : c.pair;
             const T sy = pr == 0 ? say : -say;
             const C u = e[2 * q], l = e[2 * q + 1];
+            if constexpr (sizeof(T) == 4 && Cf::LOGE == 2) {
+                // the expressions below with every fusion written out: the radix-4 forms
+                // differ in components per thread and stand in for one another (a crowded
+                // batch swaps them, a persistent batch runs wide rows for all of them)
+                e[2 * q] = mk<C>(__fadd_rn(u.x, fmaf(c1, u.x, fmaf(sy, l.x, -sax * l.y))), __fadd_rn(u.y, fmaf(c1, u.y, fmaf(sy, l.y, sax * l.x))));
+                e[2 * q + 1] = mk<C>(__fadd_rn(l.x, fmaf(c1, l.x, fmaf(-sy, u.x, -sax * u.y))), __fadd_rn(l.y, fmaf(c1, l.y, fmaf(-sy, u.y, sax * u.x))));
+                continue;
+            }
             const C q1 = mk<C>(sy, sax);
             const C q2 = mk<C>(-sy, sax);
             const C du = cadd(mk<C>(c1 * u.x, c1 * u.y), cmul(q1, l));
@@ -914,10 +923,13 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
                     const int pr = NC == 4 ? q : c.pair;
                     const T piy = pr == 0 ? yv.x : -yv.x;
                     const C u = e[2 * q], l = e[2 * q + 1];
-                    if constexpr (sizeof(T) == 4 && (V == 2 || V == kFormSmall)) {
-                        // the expressions below with every fusion written out, so that these two
-                        // forms, which differ in components per thread, round alike (a crowded
-                        // batch swaps them); psi + (f psi) keeps one rounding around psi itself
+                    if constexpr (sizeof(T) == 4 && (V == kFormWide || V == kFormSmall || V == kFormTall || V == kFormTallWide || (V == 3 && LOGN >= 10))) {
+                        // the expressions below with every fusion written out, so that forms
+                        // that differ in components per thread round alike (a crowded batch
+                        // swaps them; variant 3 is the long columns' lone form); psi + (f psi)
+                        // keeps one rounding around psi itself.  Where no form needs it the
+                        // compiler's choice stays: 3 % faster at 512-point columns (128x512
+                        // 10.34 us a step against 10.68)
                         const C hu = mk<C>(fmaf(piy, l.y, fmaf(pix, l.x, mc * u.x)), fmaf(-piy, l.x, fmaf(pix, l.y, mc * u.y)));
                         const C hl = mk<C>(fmaf(-mc, l.x, fmaf(-piy, u.y, pix * u.x)), fmaf(-mc, l.y, fmaf(piy, u.x, pix * u.y)));
                         const C u1 = mk<C>(fmaf(u.x, invP, fmaf(ab.y, hu.y, ab.x * u.x)), fmaf(u.y, invP, fmaf(-ab.y, hu.x, ab.x * u.y)));

@@ -21,10 +21,13 @@ extern template cudaError_t launch_sweep_f32_v<2>(int, int, int, const SweepArgs
 extern template cudaError_t launch_sweep_f32_v<3>(int, int, int, const SweepArgs&, cudaStream_t);
 extern template cudaError_t launch_sweep_f32_v<kFormSmall>(int, int, int, const SweepArgs&, cudaStream_t);
 extern template cudaError_t launch_sweep_f32_v<kFormLarge>(int, int, int, const SweepArgs&, cudaStream_t);
+extern template cudaError_t launch_sweep_f32_v<kFormWide>(int, int, int, const SweepArgs&, cudaStream_t);
+extern template cudaError_t launch_sweep_f32_v<kFormTall>(int, int, int, const SweepArgs&, cudaStream_t);
+extern template cudaError_t launch_sweep_f32_v<kFormTallWide>(int, int, int, const SweepArgs&, cudaStream_t);
 
 cudaError_t launch_sweep_f32(int form, int axis, int shape, int logn, const SweepArgs& a,
                              cudaStream_t s) {
-    static_assert(kNumSweepVariants == 4 && kNumSweepForms == 6, "one case per compiled form");
+    static_assert(kNumSweepVariants == 4 && kNumSweepForms == 9, "one case per compiled form");
     switch (form) {
         case 0: return launch_sweep_f32_v<0>(axis, shape, logn, a, s);
         case 1: return launch_sweep_f32_v<1>(axis, shape, logn, a, s);
@@ -32,6 +35,9 @@ cudaError_t launch_sweep_f32(int form, int axis, int shape, int logn, const Swee
         case 3: return launch_sweep_f32_v<3>(axis, shape, logn, a, s);
         case kFormSmall: return launch_sweep_f32_v<kFormSmall>(axis, shape, logn, a, s);
         case kFormLarge: return launch_sweep_f32_v<kFormLarge>(axis, shape, logn, a, s);
+        case kFormWide: return launch_sweep_f32_v<kFormWide>(axis, shape, logn, a, s);
+        case kFormTall: return launch_sweep_f32_v<kFormTall>(axis, shape, logn, a, s);
+        case kFormTallWide: return launch_sweep_f32_v<kFormTallWide>(axis, shape, logn, a, s);
         default: return cudaErrorInvalidValue;
     }
 }

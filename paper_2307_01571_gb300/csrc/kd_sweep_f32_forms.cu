@@ -1,5 +1,5 @@
-// The FP32 sweeps' forms beyond the launch variants (sweep_form in kd_internal.h: small and
-// large), compiled once per KD_SWEEP_FORM for the axis lengths that use them.
+// The FP32 sweeps' forms beyond the launch variants (sweep_form in kd_internal.h: small,
+// tall, large and the wide ones), compiled once per KD_SWEEP_FORM for the axis lengths that use them.
 #include "kd_sweep.cuh"
 
 namespace kd {

@@ -121,3 +121,40 @@ def test_runs_from_new_states_and_times_replay_the_same_steps(kd, prec):
                 ref, ref_obs, ref_t = run(fresh, k)
             spec_basis = 1 if k == 1 else (0 if k == 0 else spec_basis)
             assert np.array_equal(psi, ref) and obs == ref_obs and t == ref_t
+
+
+@pytest.mark.parametrize("nx,ny", [(4, 1024), (32, 1024), (16, 2048), (32, 2048), (64, 2048), (16, 4096),
+                                   (2048, 32), (1024, 64), (1024, 128), (1024, 256)])
+def test_more_default_forms_match_oracle(kd, nx, ny):
+    """Tall columns on both sides of their line, and 1024-point rows in each of their forms."""
+    test_default_form_matches_oracle(kd, nx, ny)
+
+
+@pytest.mark.parametrize("shapes", [
+    [(512, 128), (1024, 64), (2048, 32), (2048, 64), (512, 256), (1024, 128), (8, 8)],
+    [(64, 512), (128, 512), (256, 512), (64, 1024), (32, 1024), (4, 1024), (32, 2048)],
+    [(128, 1024), (256, 1024), (64, 2048), (16, 4096), (64, 4096), (8, 2048)]])
+@pytest.mark.parametrize("variants", [None, (0, 3), (1, 2)])
+def test_long_lines_in_a_crowded_batch_equal_members_alone(kd, shapes, variants):
+    """As test_members_of_a_crowded_batch_equal_members_alone, at every length and size whose
+    form a crowd changes, with the default variants and others beside them."""
+    wls = [W.small(nx, ny, W.GAUSS, units=W.ATOMIC, a0=0.3).with_(precision=1) for nx, ny in shapes]
+    assert sum(w.points for w in wls) > 1 << 18
+
+    def make(wl):
+        sim = kd.Sim.from_workload(wl)
+        if variants:
+            sim.sweep_variants = variants
+        sim.init_packet(wl.packet)
+        return sim
+
+    alone = []
+    for wl in wls:
+        with make(wl) as sim:
+            alone.append((sim.step(wl.dt, 6, obs_every=3), sim.get_spinor()))
+    sims = [make(wl) for wl in wls]
+    with kd.Batch(sims) as b:
+        obs = b.step([wl.dt for wl in wls], 6, obs_every=3)
+    for s, o, (ref_obs, ref) in zip(sims, obs, alone):
+        assert np.array_equal(s.get_spinor(), ref) and o == ref_obs
+        s.close()
