@@ -153,9 +153,11 @@ __host__ __device__ constexpr SweepVariant sweep_form(int axis, int form) {
     if (axis == AXIS_X) return SweepVariant{2, 64, 1, 2, 32, 0};
     return form == kFormSmall ? SweepVariant{2, 64, 2, 2, 32, 0} : SweepVariant{4, 256, 2, 2, 16, 0};
 }
-// axes and lengths a form is compiled for
+// axes and lengths a form is compiled for: those at which sweep_form_of gives it on some grid
+// (axes end at 4096 points)
 __host__ __device__ constexpr bool sweep_form_holds(int axis, int form, int logn) {
-    return form == kFormSmall      ? logn <= (axis == AXIS_X ? 11 : 10)
+    return form <= 1               ? (axis == AXIS_X ? logn >= 7 : logn >= 6 && logn <= 9)
+           : form == kFormSmall      ? logn <= (axis == AXIS_X ? 11 : 10)
            : form == kFormWide     ? logn <= (axis == AXIS_X ? 11 : 9)
            : form == kFormTall     ? axis == AXIS_Y && (logn == 10 || logn == 11)
            : form == kFormTallWide ? axis == AXIS_Y && logn >= 10

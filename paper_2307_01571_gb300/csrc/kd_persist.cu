@@ -32,6 +32,7 @@ constexpr int kThreads = 256;            // CTA size of the persistent kernel
 // latter up to 256 points (at 512 points it needs 512-thread CTAs)
 constexpr int kVX0 = 0, kVX1 = kFormWide, kVY0 = 3, kVY1 = 2;
 constexpr int kMinLog = 4, kMaxLog = 9, kMaxLogVY1 = 8;
+constexpr int kMinLogVX0 = 9;   // shorter rows of a persistent member's grid are radix-4 in every variant
 
 static_assert(sizeof(SweepArgs) % sizeof(int4) == 0, "SweepArgs copies as int4");
 
@@ -86,8 +87,9 @@ __device__ __forceinline__ void run_logn_y1(int logn, const SweepArgs& a, int g,
 template <int AXIS, int SHAPE>
 __device__ __forceinline__ void run_logn(int logn, int alt, const SweepArgs& a, int g, unsigned char* smem, int nl) {
     if constexpr (AXIS == AXIS_X) {
-        if (alt) run_logn_v<AXIS, SHAPE, kVX1>(logn, a, g, smem, nl);
-        else run_logn_v<AXIS, SHAPE, kVX0>(logn, a, g, smem, nl);
+        static_assert(kMinLogVX0 == kMaxLog, "one length of radix-8 rows");
+        if (alt || logn < kMinLogVX0) run_logn_v<AXIS, SHAPE, kVX1>(logn, a, g, smem, nl);
+        else run_group<kMinLogVX0, AXIS, SHAPE, kVX0>(a, g, smem, nl);
     } else {
         if (alt && logn <= kMaxLogVY1) run_logn_y1<SHAPE>(logn, a, g, smem, nl);
         else run_logn_v<AXIS, SHAPE, kVY0>(logn, a, g, smem, nl);
@@ -209,7 +211,10 @@ template <int LOGN, int AXIS, int VAR> void geo_v(int lines, int* ctas) {
 }
 template <int LOGN> void geo_axis(int axis, int alt, int lines, int* ctas) {
     if (axis == AXIS_X) {
-        if (alt) geo_v<LOGN, AXIS_X, kVX1>(lines, ctas); else geo_v<LOGN, AXIS_X, kVX0>(lines, ctas);
+        if constexpr (LOGN >= kMinLogVX0) {
+            if (!alt) { geo_v<LOGN, AXIS_X, kVX0>(lines, ctas); return; }
+        }
+        geo_v<LOGN, AXIS_X, kVX1>(lines, ctas);
     } else {
         if constexpr (LOGN <= kMaxLogVY1) {
             if (alt) { geo_v<LOGN, AXIS_Y, kVY1>(lines, ctas); return; }
@@ -219,10 +224,10 @@ template <int LOGN> void geo_axis(int axis, int alt, int lines, int* ctas) {
 }
 
 template <int LOGN> int max_smem() {
-    int y1 = 0;
+    int y1 = 0, x0 = 0;
     if constexpr (LOGN <= kMaxLogVY1) y1 = Geo<LOGN, AXIS_Y, kVY1>::SMEM;
-    const int s[4] = {Geo<LOGN, AXIS_X, kVX0>::SMEM, Geo<LOGN, AXIS_X, kVX1>::SMEM,
-                      Geo<LOGN, AXIS_Y, kVY0>::SMEM, y1};
+    if constexpr (LOGN >= kMinLogVX0) x0 = Geo<LOGN, AXIS_X, kVX0>::SMEM;
+    const int s[4] = {x0, Geo<LOGN, AXIS_X, kVX1>::SMEM, Geo<LOGN, AXIS_Y, kVY0>::SMEM, y1};
     int m = 0;
     for (int v : s) m = v > m ? v : m;
     return m;

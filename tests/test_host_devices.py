@@ -162,3 +162,38 @@ def test_batch_buffers_after_a_failed_allocation(fake):
         fake.kd_mlp_destroy(h)
         assert fake.fake_bad_frees() == 0, k
     assert k > 6 and fake.fake_bad_frees() == 0
+
+
+def _batch_step(lib, sims, dt):
+    b = C.c_void_p()
+    assert lib.kd_batch_create((C.c_void_p * len(sims))(*sims), len(sims), None, C.byref(b)) == 0
+    rc = lib.kd_batch_step(b, (C.c_double * len(sims))(*[dt] * len(sims)), C.c_int64(2), C.c_int64(0), None, C.c_int64(0), None)
+    lib.kd_batch_destroy(b)
+    return rc
+
+
+def test_every_grid_and_variant_has_its_kernels(fake):
+    """The kernels that the launch rule names for a grid are among those compiled, for every
+    pair of axis lengths and every variant, alone and in a batch that fills the SMs (one that
+    is not compiled is refused with an error)."""
+    rc, big, _ = _sim(fake, 1024, 512, 1)
+    assert rc == 0
+    sizes = [1 << k for k in range(2, 13)]
+    for nx in sizes:
+        for ny in sizes:
+            if nx * ny > 1 << 20:
+                continue
+            rc, h, wl = _sim(fake, nx, ny, 1)
+            assert rc == 0, (nx, ny)
+            for v in range(4):
+                assert fake.kd_set_sweep_variants(h, v, v) == 0, (nx, ny, v)
+                assert fake.kd_step(h, C.c_double(wl.dt), C.c_int64(2), C.c_int64(0), None, C.c_int64(0), None) == 0
+                assert _batch_step(fake, [h, big], wl.dt) == 0, (nx, ny, v)
+            if 16 <= nx <= 512 and 16 <= ny <= 512:
+                b = C.c_void_p()
+                assert fake.kd_batch_create((C.c_void_p * 1)(h), 1, None, C.byref(b)) == 0
+                assert fake.kd_batch_set_mode(b, 1) == 0
+                assert fake.kd_batch_step(b, (C.c_double * 1)(wl.dt), C.c_int64(2), C.c_int64(0), None, C.c_int64(0), None) == 0
+                fake.kd_batch_destroy(b)
+            fake.kd_destroy(h)
+    fake.kd_destroy(big)
