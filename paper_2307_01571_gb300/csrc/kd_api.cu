@@ -1047,14 +1047,34 @@ int reject_capture(kd_sim* s, const char* what) {
 }
 
 // First launch of every sweep shape of the current variants outside any stream capture
-// (sets the kernels' shared-memory attributes); reads psi, writes only the work buffer.
+// (sets the kernels' shared-memory attributes); reads psi, writes only the work buffer.  With
+// them the forms that stand in for these in a batch that fills the SMs, whose first launch would
+// otherwise be inside the batch's capture: once per device, form and length.
 int warm_variants(kd_sim* s) {
+    static std::atomic<uint64_t> crowd[2][kNumSweepForms][13];
+    const uint64_t bit = s->device < 64 ? (uint64_t)1 << s->device : 0;
     const int shapes[3] = {SHAPE_F1, SHAPE_F2, SHAPE_F1F2};
-    for (int ax = 0; ax < 2; ++ax)
-        for (int sh : shapes) {
-            cudaError_t el = sweep(s, ax, sh, OP_NONE, s->psi, s->work, 0, 0.0);
+    for (int ax = 0; ax < 2; ++ax) {
+        std::atomic<uint64_t>* once = nullptr;
+        for (bool crowded : {false, true}) {
+            if (crowded) {
+                if (s->prec == KD_FP64) break;
+                const int lone = form(s, ax);
+                s->crowded = true;
+                const int f = form(s, ax);
+                s->crowded = false;
+                once = &crowd[ax][f][ax == AXIS_X ? s->lx : s->ly];
+                if (f == lone || (once->load(std::memory_order_relaxed) & bit)) break;
+            }
+            cudaError_t el = cudaSuccess;
+            s->crowded = crowded;
+            for (int sh : shapes)
+                if (el == cudaSuccess) el = sweep(s, ax, sh, OP_NONE, s->psi, s->work, 0, 0.0);
+            s->crowded = false;
             if (el != cudaSuccess) return fail(KD_ERR_CUDA, "sweep launch: %s", cudaGetErrorString(el));
+            if (crowded && !s->tc) once->fetch_or(bit, std::memory_order_relaxed);   // (tc: not every shape)
         }
+    }
     KD_CUDA(cudaStreamSynchronize(s->stream));
     return KD_OK;
 }
@@ -2017,25 +2037,6 @@ int kd_batch_create(kd_sim* const* sims, int32_t n, void* cuda_stream, kd_batch*
         return fail(KD_ERR_CUDA, "stream/event creation failed");
     }
     b->gens.assign(n, ~0ull);
-    if (b->crowded) {   // first launches of the forms that only a crowded batch runs, once per shape
-        std::map<std::pair<int, int>, int> seen;
-        for (kd_sim* s : b->sims) {
-            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-            if (s->prec == KD_FP64 || seen[{s->lx, s->ly}]++) continue;
-            if (cudaStreamIsCapturing(s->stream, &cs) != cudaSuccess) {
-                cudaGetLastError();
-                continue;
-            }
-            if (cs != cudaStreamCaptureStatusNone) continue;
-            s->crowded = true;
-            int rc = warm_variants(s);
-            s->crowded = false;
-            if (rc) {
-                kd_batch_destroy(b);
-                return rc;
-            }
-        }
-    }
     *out = b;
     return KD_OK;
 }

@@ -21,6 +21,9 @@ std::map<std::pair<int, const void*>, int> limit;   // dynamic shared memory per
 std::set<void*> live;
 int bad_frees = 0, fail_after = -1, capturing_error = 0, refuse_attr = 0;
 long launches = 0;
+bool capturing = false;
+int first_in_capture = 0;                           // kernels first launched inside a capture
+std::set<std::pair<int, const void*>> seen;
 struct Config {
     dim3 grid, block;
     size_t shared;
@@ -38,6 +41,7 @@ cudaError_t launch(const void* k, size_t shared) {
     const size_t most = it == limit.end() ? kStaticLimit : it->second;
     if (shared > most && shared > (size_t)kStaticLimit) return done(cudaErrorInvalidValue);
     ++launches;
+    if (seen.insert({device, k}).second && capturing) ++first_in_capture;
     return cudaSuccess;
 }
 
@@ -54,6 +58,7 @@ void fake_capture_query_error(int on) { capturing_error = on; }
 void fake_refuse_attribute(int on) { refuse_attr = on; }
 int fake_set_device(int d) { return cudaSetDevice(d); }
 int fake_last_error() { return last; }
+int fake_first_in_capture() { return first_in_capture; }
 
 cudaError_t cudaGetDeviceCount(int* n) { *n = kDevices; return cudaSuccess; }
 cudaError_t cudaGetDevice(int* d) { *d = device; return cudaSuccess; }
@@ -98,8 +103,8 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* c) {
     *c = cudaStreamCaptureStatusNone;
     return capturing_error ? done(cudaErrorStreamCaptureImplicit) : cudaSuccess;
 }
-cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaSuccess; }
-cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { *g = (cudaGraph_t)malloc(1); return cudaSuccess; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { capturing = true; return cudaSuccess; }
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { capturing = false; *g = (cudaGraph_t)malloc(1); return cudaSuccess; }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t* x, cudaGraph_t, unsigned long long) { *x = (cudaGraphExec_t)malloc(1); return cudaSuccess; }
 cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaGraphDestroy(cudaGraph_t g) { free(g); return cudaSuccess; }

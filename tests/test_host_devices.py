@@ -197,3 +197,27 @@ def test_every_grid_and_variant_has_its_kernels(fake):
                 fake.kd_batch_destroy(b)
             fake.kd_destroy(h)
     fake.kd_destroy(big)
+
+
+def test_no_sweep_kernel_is_first_launched_in_a_capture(fake):
+    """What a crowded batch launches has run before its graph is captured, whatever variants the
+    first member of a shape has and whether a member's variants change after the batch is made."""
+    from paper_2307_01571_gb300 import kd, workloads as W
+    assert fake.fake_set_device(1) == 0
+    rc, big, wl = _sim(fake, 1024, 512, 1)
+    assert rc == 0
+    sims = [_sim(fake, 128, 64, 1)[1] for _ in range(3)]
+    assert fake.kd_set_sweep_variants(sims[0], 2, 3) == 0
+    b = C.c_void_p()
+    assert fake.kd_batch_create((C.c_void_p * 4)(*sims, big), 4, None, C.byref(b)) == 0
+    dt = (C.c_double * 4)(*[wl.dt] * 4)
+    # the small kernels of the step loop have no first launch of their own: a lone run's
+    assert fake.kd_step(sims[1], C.c_double(wl.dt), C.c_int64(2), C.c_int64(0), None, C.c_int64(0), None) == 0
+    before = fake.fake_first_in_capture()
+    assert fake.kd_batch_step(b, dt, C.c_int64(2), C.c_int64(0), None, C.c_int64(0), None) == 0
+    assert fake.kd_set_sweep_variants(sims[0], 0, 0) == 0
+    assert fake.kd_batch_step(b, dt, C.c_int64(2), C.c_int64(0), None, C.c_int64(0), None) == 0
+    assert fake.fake_first_in_capture() == before
+    fake.kd_batch_destroy(b)
+    for s in (*sims, big):
+        fake.kd_destroy(s)
