@@ -403,30 +403,72 @@ __device__ __forceinline__ unsigned char* cell(unsigned char* dst, int row, int 
 }
 // 16-deep products of the slab at k0
 __device__ __forceinline__ int steps_of(int k0, int kend) { return min(KS, kend - k0 + 15) / 16; }
+// A tile is whole (every line and k inside, 16-byte loads), or so small that there is little to
+// wait for (few rows, or a single 16-deep step: read element by element at the store), or
+// neither: edges, gathered rows, odd strides.  The last kind exists in the CHECKED kernel only,
+// which the host picks where such a tile can occur (needs_checks): there too all of a thread's
+// loads of the slab are in flight together, with every bound checked, 16-byte ones where the
+// lines allow it, else scalar ones side by side across the warp.  (In one kernel with the whole
+// tiles' short path the checks cost the 256-wide network's steps 3-4 %.)  With these tiles read
+// element by element as well, a load latency per eight, a training step took, us: widths 1024,
+// 2048, 2048, 64 on 1024 gathered rows 1361 (now 891), on 32 plain ones 399 (254); widths 511,
+// 1023, 1023, 7 at batch 1024 620 (367); widths 5, 256, 256, 256, 4 at batch 200 116 (84).
 template <int ROWS> struct Tile {
     float4 v[ROWS / 8];
-    bool whole;      // v holds the tile; else it is read element by element at the store
+    bool held;       // v holds the tile; else it is read element by element at the store
 };
-template <int ROWS, bool KC> __device__ __forceinline__ void tile_load(const Operand& o, int r0, int R, int k0, int kend, Tile<ROWS>& s) {
+__host__ __device__ constexpr bool small_tile(int rows, int k) { return rows < 16 || k <= 16; }
+template <int ROWS, bool KC, bool CHECKED>
+__device__ __forceinline__ void tile_load(const Operand& o, int r0, int R, int k0, int kend, Tile<ROWS>& s) {
     const int t = threadIdx.x;
-    s.whole = o.vec && !o.idx && r0 + ROWS <= R && k0 + KS <= kend;
-    if (!s.whole) return;
     constexpr int KB = ROWS == 128 ? 8 : 2;
-    const float* p = o.p + (KC ? (long)(r0 + (t >> 5)) * o.ld + k0 + 4 * (t & 31)
-                               : (long)(k0 + KB * (t / (ROWS / 4))) * o.ld + r0 + 4 * (t % (ROWS / 4)));
+    // this thread's first line (row, or k if !KC) and its place along the lines: four elements
+    // there, side by side or (scalar loads) a quarter of the tile apart
+    constexpr int Q = KC ? KS / 4 : ROWS / 4;
+    const int line0 = KC ? r0 + (t >> 5) : k0 + KB * (t / Q), at = (KC ? k0 : r0) + (!CHECKED || o.vec ? 4 : 1) * (t % Q);
+    const bool whole = o.vec && !o.idx && r0 + ROWS <= R && k0 + KS <= kend;
+    s.held = CHECKED ? whole || !small_tile(R - r0, kend - k0) : whole;
+    if (!s.held) return;
+    if (!CHECKED || whole) {
+        const float* p = o.p + (long)line0 * o.ld + at;
 #pragma unroll
-    for (int i = 0; i < ROWS / 8; ++i) {
-        const long line = KC ? 8 * i : 64 * (i / KB) + i % KB;
-        s.v[i] = *reinterpret_cast<const float4*>(p + line * o.ld);
+        for (int i = 0; i < ROWS / 8; ++i) {
+            const long line = KC ? 8 * i : 64 * (i / KB) + i % KB;
+            s.v[i] = *reinterpret_cast<const float4*>(p + line * o.ld);
+        }
+    } else {
+        const int lines = KC ? R : kend, left = (KC ? kend : R) - at;   // elements along the lines
+#pragma unroll
+        for (int i = 0; i < ROWS / 8; ++i) {
+            long line = line0 + (KC ? 8 * i : 64 * (i / KB) + i % KB);
+            bool in = line < lines && left > 0;
+            if (in && o.idx) {
+                line = o.idx[line];
+                in = line >= 0 && line < o.nidx;
+            }
+            float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (in) {
+                const float* p = o.p + line * o.ld + at;
+                if (o.vec) {   // the extent is a multiple of four, as the stride is
+                    x = *reinterpret_cast<const float4*>(p);
+                } else {
+                    x.x = p[0];
+                    if (left > Q) x.y = p[Q];
+                    if (left > 2 * Q) x.z = p[2 * Q];
+                    if (left > 3 * Q) x.w = p[3 * Q];
+                }
+            }
+            s.v[i] = x;
+        }
     }
 }
 __device__ __forceinline__ float elem(const float4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
-template <int ROWS, bool KC>
+template <int ROWS, bool KC, bool CHECKED>
 __device__ __forceinline__ void tile_store(unsigned char* dst, const Operand& o, int r0, int R, int k0, int kend, const Tile<ROWS>& s) {
     const int t = threadIdx.x;
-    if (!s.whole) {
-        // edges, gathered rows, odd strides: element by element, zeros outside, up to the
-        // last 16-deep step that holds any k
+    const bool side = !CHECKED || o.vec;   // a thread's four elements of a line lie side by side
+    if (!s.held) {
+        // element by element, zeros outside, up to the last 16-deep step that holds any k
 #pragma unroll 1
         for (int c = t; c < ROWS * 2 * steps_of(k0, kend); c += 256) {
             const int row = r0 + c % ROWS, k = k0 + 8 * (c / ROWS);
@@ -445,16 +487,24 @@ __device__ __forceinline__ void tile_store(unsigned char* dst, const Operand& o,
                 make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
         }
     } else if constexpr (KC) {
+        if (side) {
 #pragma unroll
-        for (int i = 0; i < ROWS / 8; ++i)
-            *reinterpret_cast<uint2*>(cell(dst, (t >> 5) + 8 * i, 4 * (t & 31))) =
-                make_uint2(pack_bf16(s.v[i].x, s.v[i].y), pack_bf16(s.v[i].z, s.v[i].w));
+            for (int i = 0; i < ROWS / 8; ++i)
+                *reinterpret_cast<uint2*>(cell(dst, (t >> 5) + 8 * i, 4 * (t & 31))) =
+                    make_uint2(pack_bf16(s.v[i].x, s.v[i].y), pack_bf16(s.v[i].z, s.v[i].w));
+        } else {
+#pragma unroll
+            for (int i = 0; i < ROWS / 8; ++i)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    *reinterpret_cast<__nv_bfloat16*>(cell(dst, (t >> 5) + 8 * i, (t & 31) + 32 * e)) = __float2bfloat16_rn(elem(s.v[i], e));
+        }
     } else if constexpr (ROWS == 128) {
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-                *reinterpret_cast<uint4*>(cell(dst, 4 * (t & 31) + e, 8 * (t >> 5) + 64 * i)) =
+                *reinterpret_cast<uint4*>(cell(dst, side ? 4 * (t & 31) + e : (t & 31) + 32 * e, 8 * (t >> 5) + 64 * i)) =
                     make_uint4(pack_bf16(elem(s.v[8 * i + 0], e), elem(s.v[8 * i + 1], e)),
                                pack_bf16(elem(s.v[8 * i + 2], e), elem(s.v[8 * i + 3], e)),
                                pack_bf16(elem(s.v[8 * i + 4], e), elem(s.v[8 * i + 5], e)),
@@ -462,12 +512,12 @@ __device__ __forceinline__ void tile_store(unsigned char* dst, const Operand& o,
     } else {
 #pragma unroll
         for (int e = 0; e < 4; ++e)
-            *reinterpret_cast<uint32_t*>(cell(dst, 4 * (t & 3) + e, 2 * (t >> 2))) = pack_bf16(elem(s.v[0], e), elem(s.v[1], e));
+            *reinterpret_cast<uint32_t*>(cell(dst, side ? 4 * (t & 3) + e : (t & 3) + 4 * e, 2 * (t >> 2))) = pack_bf16(elem(s.v[0], e), elem(s.v[1], e));
     }
 }
 }  // namespace tcg
 
-template <bool AKC, bool BKC>
+template <bool AKC, bool BKC, bool CHECKED>
 __device__ __forceinline__ void product_bf16(const Product& q, int blk, int* status, unsigned char* sm) {
     const int t = threadIdx.x, w = t >> 5;
     const int n0 = (blk % q.nt_tiles) * tcg::BN, m0 = blk / q.nt_tiles % q.mt * 128, split = blk / (q.nt_tiles * q.mt);
@@ -492,10 +542,10 @@ __device__ __forceinline__ void product_bf16(const Product& q, int blk, int* sta
     tcg::Tile<128> ta;
     tcg::Tile<tcg::BN> tb;
     if (nslab > 0) {
-        tcg::tile_load<128, AKC>(q.A, m0, q.M, kbeg, kend, ta);
-        tcg::tile_load<tcg::BN, BKC>(q.B, n0, q.N, kbeg, kend, tb);
-        tcg::tile_store<128, AKC>(sm, q.A, m0, q.M, kbeg, kend, ta);
-        tcg::tile_store<tcg::BN, BKC>(sm + tcg::A_BYTES, q.B, n0, q.N, kbeg, kend, tb);
+        tcg::tile_load<128, AKC, CHECKED>(q.A, m0, q.M, kbeg, kend, ta);
+        tcg::tile_load<tcg::BN, BKC, CHECKED>(q.B, n0, q.N, kbeg, kend, tb);
+        tcg::tile_store<128, AKC, CHECKED>(sm, q.A, m0, q.M, kbeg, kend, ta);
+        tcg::tile_store<tcg::BN, BKC, CHECKED>(sm + tcg::A_BYTES, q.B, n0, q.N, kbeg, kend, tb);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -522,8 +572,8 @@ __device__ __forceinline__ void product_bf16(const Product& q, int blk, int* sta
         issued = j + 1;
         // the next slab's global loads run while these products do
         if (j + 1 < nslab) {
-            tcg::tile_load<128, AKC>(q.A, m0, q.M, kbeg + tcg::KS * (j + 1), kend, ta);
-            tcg::tile_load<tcg::BN, BKC>(q.B, n0, q.N, kbeg + tcg::KS * (j + 1), kend, tb);
+            tcg::tile_load<128, AKC, CHECKED>(q.A, m0, q.M, kbeg + tcg::KS * (j + 1), kend, ta);
+            tcg::tile_load<tcg::BN, BKC, CHECKED>(q.B, n0, q.N, kbeg + tcg::KS * (j + 1), kend, tb);
         }
         bool got = true;
         if (j >= 1) {   // slab j - 1's products read the stage slab j + 1 goes to
@@ -535,8 +585,8 @@ __device__ __forceinline__ void product_bf16(const Product& q, int blk, int* sta
         }
         if (got && j + 1 < nslab) {
             unsigned char* st = sm + (uint32_t)(b ^ 1) * tcg::STAGE;
-            tcg::tile_store<128, AKC>(st, q.A, m0, q.M, kbeg + tcg::KS * (j + 1), kend, ta);
-            tcg::tile_store<tcg::BN, BKC>(st + tcg::A_BYTES, q.B, n0, q.N, kbeg + tcg::KS * (j + 1), kend, tb);
+            tcg::tile_store<128, AKC, CHECKED>(st, q.A, m0, q.M, kbeg + tcg::KS * (j + 1), kend, ta);
+            tcg::tile_store<tcg::BN, BKC, CHECKED>(st + tcg::A_BYTES, q.B, n0, q.N, kbeg + tcg::KS * (j + 1), kend, tb);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -588,8 +638,8 @@ __device__ __forceinline__ void product_bf16(const Product& q, int blk, int* sta
 }
 
 // One launch of a pass: the block index selects the product (and its tile and part), the
-// column sums or the loss.
-template <int BF16> __global__ void __launch_bounds__(256) k_group(const __grid_constant__ Group g) {
+// column sums or the loss.  KIND 0: FP32; 1: BF16, whole or small tiles; 2: BF16, checked tiles.
+template <int KIND> __global__ void __launch_bounds__(256, 2) k_group(const __grid_constant__ Group g) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
     const int blk = blockIdx.x;
@@ -609,10 +659,10 @@ template <int BF16> __global__ void __launch_bounds__(256) k_group(const __grid_
             b -= g.first[1];
         }
         extern __shared__ __align__(1024) unsigned char sm[];
-        if constexpr (BF16) {
-            if (!q.A.kc) product_bf16<false, false>(q, b, g.status, sm);
-            else if (q.B.kc) product_bf16<true, true>(q, b, g.status, sm);
-            else product_bf16<true, false>(q, b, g.status, sm);
+        if constexpr (KIND != 0) {
+            if (!q.A.kc) product_bf16<false, false, KIND == 2>(q, b, g.status, sm);
+            else if (q.B.kc) product_bf16<true, true, KIND == 2>(q, b, g.status, sm);
+            else product_bf16<true, false, KIND == 2>(q, b, g.status, sm);
         } else {
             float* f = reinterpret_cast<float*>(sm);
             if (q.bm == 16) {
@@ -674,7 +724,10 @@ Operand operand(const float* p, long ld, bool kc, const int32_t* idx = nullptr, 
 // tiles while 32-row ones would leave SMs without one (256 x 256 outputs: 64 tiles), since what
 // counts there is one tile's latency; else 32 rows, which read half as much per output (a step
 // at batch 256 42.9 us against 51.2 with 32 rows only; at batch 1024 78.8 with 16 rows only
-// against 74.6).
+// against 74.6).  The tiles are drawn for the 256-wide network.  Wider ones read an operand more
+// often than 64 x 64 (FP32) and 128 x 32 (BF16) tiles did, and are still faster (widths 1024,
+// 2048, 2048, 64 at batch 4096: FP32 10.1 -> 4.8 ms, BF16 3.7 -> 2.7), but for BF16 with rows
+// of odd length from 2049 on at batch 1024 and more (1.29 -> 1.50 ms).
 void tile(const kd_mlp* n, Product* q, int splits) {
     const bool bf = n->prec == KD_MLP_BF16;
     const int bn = bf ? tcg::BN : fp32::BN;
@@ -705,12 +758,35 @@ cudaError_t launch_pdl(void (*k)(KP...), long grid, int threads, int smem, cudaS
 // device.  The limit belongs to one device's copy of the kernel, so every network sets it for
 // its own device (kd_mlp_create, kd_mlp_set_precision) and nothing remembers it.
 cudaError_t allow_smem(int precision) {
-    return precision == KD_MLP_BF16
-        ? cudaFuncSetAttribute(k_group<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tcg::SMEM)
-        : cudaFuncSetAttribute(k_group<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, fp32::SMEM);
+    constexpr cudaFuncAttribute attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if (precision != KD_MLP_BF16) return cudaFuncSetAttribute(k_group<0>, attr, fp32::SMEM);
+    const cudaError_t e = cudaFuncSetAttribute(k_group<1>, attr, (int)tcg::SMEM);
+    return e == cudaSuccess ? cudaFuncSetAttribute(k_group<2>, attr, (int)tcg::SMEM) : e;
 }
 
-cudaError_t launch_group(const kd_mlp* n, Group& g, int nprod, cudaStream_t s) {
+// Whether a tile of a BF16 product can be neither whole nor small (tcg::Tile): its operand has
+// rows x k elements, k in parts of kper.
+bool needs_checks(const Operand& o, int tile_rows, int rows, int k, int kper) {
+    if (tcg::small_tile(rows, kper)) return false;
+    return !o.vec || o.idx || rows % tile_rows != 0 || k % tcg::KS != 0 || kper % tcg::KS != 0;
+}
+bool needs_checks(const Group& g, int nprod) {
+    for (int i = 0; i < nprod; ++i) {
+        const Product& q = g.prod[i];
+        if (needs_checks(q.A, 128, q.M, q.K, q.kper) || needs_checks(q.B, tcg::BN, q.N, q.K, q.kper)) return true;
+    }
+    return false;
+}
+
+// A pass's launches in order, all by one kernel: the BF16 kernel with checks for every launch
+// if any needs it (alternating between the two, each with a cold instruction cache, a forward
+// pass of the 256-wide network at batch 32 took 47 us; 35 with one).
+struct Pass {
+    Group g[16];
+    int nprod[16];
+    int n = 0;
+};
+cudaError_t launch_group(const kd_mlp* n, Group& g, int nprod, bool checks, cudaStream_t s) {
     long b = 0;
     for (int i = 0; i < 2; ++i) {
         g.first[i] = (int)b;
@@ -727,7 +803,18 @@ cudaError_t launch_group(const kd_mlp* n, Group& g, int nprod, cudaStream_t s) {
     // BF16: two 41 KB stages and 32 columns of tensor memory per CTA: two CTAs per SM, whose
     // columns fit the SM's 512, so no allocation waits
     const int smem = bf ? (int)tcg::SMEM : fp32::SMEM;
-    return bf ? launch_pdl(k_group<1>, b, 256, smem, s, g) : launch_pdl(k_group<0>, b, 256, smem, s, g);
+    if (!bf) return launch_pdl(k_group<0>, b, 256, smem, s, g);
+    return checks ? launch_pdl(k_group<2>, b, 256, smem, s, g) : launch_pdl(k_group<1>, b, 256, smem, s, g);
+}
+
+cudaError_t launch_pass(const kd_mlp* n, Pass& p, cudaStream_t s) {
+    bool checks = false;
+    for (int i = 0; i < p.n && n->prec == KD_MLP_BF16; ++i) checks = checks || needs_checks(p.g[i], p.nprod[i]);
+    for (int i = 0; i < p.n; ++i) {
+        const cudaError_t e = launch_group(n, p.g[i], p.nprod[i], checks, s);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // KD_ERR_TIMEOUT (and the flag cleared) when a tensor-core GEMM's bounded wait gave up
@@ -782,10 +869,12 @@ struct Batch {
 // a[L]) and, with targets, also writes the loss' gradient to dbuf0 and the squared errors
 int forward(kd_mlp* n, const Batch& in, cudaStream_t s) {
     const long nout = (long)in.rows * n->w[n->L];
+    Pass pass{};
     for (int l = 0; l < n->L; ++l) {
         const int fi = n->w[l], fo = n->w[l + 1];
         const bool last = l == n->L - 1;
-        Group g{};
+        pass.nprod[pass.n] = 1;
+        Group& g = pass.g[pass.n++];
         Product& q = g.prod[0];
         q.A = l == 0 ? operand(in.x, fi, true, in.idx, in.nsrc) : operand(n->a[l], fi, true);
         q.B = operand(n->param + n->woff[l], fi, true);
@@ -805,8 +894,8 @@ int forward(kd_mlp* n, const Batch& in, cudaStream_t s) {
             q.scale = 2.0f / (float)nout;
         }
         tile(n, &q, 1);
-        MLP_CUDA(launch_group(n, g, 1, s));
     }
+    MLP_CUDA(launch_pass(n, pass, s));
     return KD_OK;
 }
 
@@ -847,6 +936,7 @@ int backward(kd_mlp* n, const Batch& in, GradParts* gp, float* loss2, cudaStream
     float* at = n->part;
     float* dcur = n->dbuf0;   // dZ_l
     float* dnext = n->dbuf1;
+    Pass pass{};
     for (int l = L - 1; l >= 0; --l) {
         const int fi = n->w[l], fo = n->w[l + 1], parts = gp->parts[l];
         float* dst = n->grad + n->woff[l];
@@ -855,7 +945,7 @@ int backward(kd_mlp* n, const Batch& in, GradParts* gp, float* loss2, cudaStream
             at += gp->stride[l] * parts;
         }
         gp->src[l] = dst;
-        Group g{};
+        Group& g = pass.g[pass.n];
         int np = 0;
         if (l > 0) {  // dZ_{l-1}[b][i] = (sum_o dZ[b][o] W_l[o][i]) GELU'(Z_{l-1}[b][i])
             Product& q = g.prod[np++];
@@ -885,11 +975,12 @@ int backward(kd_mlp* n, const Batch& in, GradParts* gp, float* loss2, cudaStream
             const long nout = (long)in.rows * fo;
             g.loss = LossSum{n->lossbuf + 1, nout, 1.0f / (float)nout, n->lossbuf, loss2};
         }
-        MLP_CUDA(launch_group(n, g, np, s));
+        pass.nprod[pass.n++] = np;
         float* tmp = dcur;
         dcur = dnext;
         dnext = tmp;
     }
+    MLP_CUDA(launch_pass(n, pass, s));
     return KD_OK;
 }
 

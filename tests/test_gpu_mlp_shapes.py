@@ -85,3 +85,42 @@ def test_gathered_rows_equal_plain_rows(kd, prec, batch):
         net.close()
     assert np.array_equal(got[0], got[1])
     assert float(loss[0]) == float(loss[1])
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+@pytest.mark.parametrize("widths,batch", [
+    ([264, 130, 36], 32), ([264, 130, 36], 200), ([128, 256, 8], 256), ([131, 67, 3], 129), ([20, 36, 4], 17)])
+def test_wide_gathered_rows_equal_plain_rows(kd, prec, widths, batch):
+    """Inputs wide enough for the loaders' vector loads: whole tiles, tiles cut off by the batch
+    or the width, and rows whose stride forbids 16-byte loads, gathered (an index out of range
+    included) and plain, bit for bit; the plain step's loss against the FP64 oracle."""
+    import torch
+    rng = np.random.default_rng(batch)
+    x = rng.standard_normal((300, widths[0])).astype(np.float32)
+    t = rng.standard_normal((300, widths[-1])).astype(np.float32)
+    idx = rng.integers(0, 300, batch).astype(np.int32)
+    idx[:2] = (300, -1)
+    ok = (idx >= 0) & (idx < 300)
+    sel = np.clip(idx, 0, 299)
+    xb = np.where(ok[:, None], x[sel], 0).astype(np.float32)
+    tb = np.where(ok[:, None], t[sel], 0).astype(np.float32)
+    p = mlp.init_params(widths, 4)
+    xd, td, idev, xbd, tbd = (torch.from_numpy(a).cuda() for a in (x, t, idx, xb, tb))
+    loss = torch.zeros(2, device="cuda")
+    got = []
+    for gather in (True, False):
+        net = kd.MLP(widths)
+        net.set_precision(kd.KD_MLP_BF16 if prec == "bf16" else kd.KD_MLP_FP32)
+        net.set_params(p)
+        if gather:
+            net.train_step_gather(xd.data_ptr(), td.data_ptr(), 300, idev.data_ptr(), batch, 1e-3,
+                                  loss_dev=loss[0:].data_ptr())
+        else:
+            net.train_step(xbd.data_ptr(), tbd.data_ptr(), batch, 1e-3, loss_dev=loss[1:].data_ptr())
+        torch.cuda.synchronize()
+        got.append(net.get_params())
+        net.close()
+    assert np.array_equal(got[0], got[1])
+    assert float(loss[0]) == float(loss[1])
+    want, _ = mlp.loss_and_grad(p.astype(np.float64), widths, xb.astype(np.float64), tb.astype(np.float64))
+    assert abs(float(loss[1]) - want) <= TOL[prec][0] * max(1.0, want)
