@@ -36,7 +36,6 @@ struct kd_mlp {
     float* dbuf1 = nullptr;
     float* lossbuf = nullptr;        // the loss, then [cap * w[L]] squared errors
     float* part = nullptr;           // partial gradients of layers whose batch is split
-    size_t part_cap = 0;             // its floats
     int prec = 0;                    // KD_MLP_FP32 or KD_MLP_BF16 (tensor-core GEMMs)
     int* status = nullptr;           // set when a tensor-core GEMM's bounded wait gave up
 };
@@ -833,6 +832,34 @@ int maxw(const kd_mlp* n) {
     return m;
 }
 
+// Parts of the batch the weight gradient of an fo x fi layer is summed in: enough for about
+// two CTAs on every SM when its tiles alone leave most of them idle, at least 128 (BF16: one
+// slab) or 256 rows each, at most eight.
+int grad_parts(int precision, int fo, int fi, int rows) {
+    const bool bf = precision == KD_MLP_BF16;
+    const int bm = bf ? 128 : 32, least = bf ? 128 : 256;
+    const int bn = bf ? tcg::BN : 32;
+    const long tiles = (long)((fo + bm - 1) / bm) * ((fi + bn - 1) / bn);
+    const long fill = (304 + tiles - 1) / tiles, depth = rows / least;
+    const long p = fill < depth ? fill : depth;
+    return (int)(p < 1 ? 1 : p > 8 ? 8 : p);
+}
+
+// Floats of the partial gradients of a batch, whichever the precision (more rows never take
+// fewer parts)
+size_t part_floats(const kd_mlp* n, int rows) {
+    size_t most = 0;
+    for (int prec : {KD_MLP_FP32, KD_MLP_BF16}) {
+        size_t need = 0;
+        for (int l = 0; l < n->L; ++l) {
+            const int parts = grad_parts(prec, n->w[l + 1], n->w[l], rows);
+            if (parts > 1) need += ((size_t)n->w[l + 1] * n->w[l] + n->w[l + 1]) * parts;
+        }
+        most = need > most ? need : most;
+    }
+    return most;
+}
+
 int ensure_cap(kd_mlp* n, int batch) {
     if (batch <= n->cap) return KD_OK;
     for (float* p : n->z) cudaFree(p);
@@ -840,9 +867,10 @@ int ensure_cap(kd_mlp* n, int batch) {
     cudaFree(n->dbuf0);
     cudaFree(n->dbuf1);
     cudaFree(n->lossbuf);
+    cudaFree(n->part);
     // nothing is left to use or free again if one of the allocations below fails
     n->cap = 0;
-    n->dbuf0 = n->dbuf1 = n->lossbuf = nullptr;
+    n->dbuf0 = n->dbuf1 = n->lossbuf = n->part = nullptr;
     n->z.assign(n->L, nullptr);
     n->a.assign(n->L + 1, nullptr);
     for (int l = 0; l < n->L; ++l) {
@@ -852,6 +880,8 @@ int ensure_cap(kd_mlp* n, int batch) {
     MLP_CUDA(cudaMalloc(&n->dbuf0, sizeof(float) * (size_t)batch * maxw(n)));
     MLP_CUDA(cudaMalloc(&n->dbuf1, sizeof(float) * (size_t)batch * maxw(n)));
     MLP_CUDA(cudaMalloc(&n->lossbuf, sizeof(float) * ((size_t)batch * n->w[n->L] + 1)));
+    const size_t part = part_floats(n, batch);
+    if (part > 0) MLP_CUDA(cudaMalloc(&n->part, part * sizeof(float)));
     n->cap = batch;
     return KD_OK;
 }
@@ -899,40 +929,18 @@ int forward(kd_mlp* n, const Batch& in, cudaStream_t s) {
     return KD_OK;
 }
 
-// Parts of the batch the weight gradient of an fo x fi layer is summed in: enough for about
-// two CTAs on every SM when its tiles alone leave most of them idle, at least 128 (BF16: one
-// slab) or 256 rows each, at most eight.
-int grad_parts(const kd_mlp* n, int fo, int fi, int rows) {
-    const bool bf = n->prec == KD_MLP_BF16;
-    const int bm = bf ? 128 : 32, least = bf ? 128 : 256;
-    const int bn = bf ? tcg::BN : 32;
-    const long tiles = (long)((fo + bm - 1) / bm) * ((fi + bn - 1) / bn);
-    const long fill = (304 + tiles - 1) / tiles, depth = rows / least;
-    const long p = fill < depth ? fill : depth;
-    return (int)(p < 1 ? 1 : p > 8 ? 8 : p);
-}
-
 // Gradients after forward() with targets: layer l's partial sums where `gp` says, the mean
 // squared error in lossbuf[0] (and *loss2).
 int backward(kd_mlp* n, const Batch& in, GradParts* gp, float* loss2, cudaStream_t s) {
     const int L = n->L;
-    size_t need = 0;
     gp->L = L;
     for (int l = 0; l < L; ++l) {
         const size_t cnt = (size_t)n->w[l + 1] * n->w[l] + n->w[l + 1];
         gp->off[l] = (long)n->woff[l];
-        gp->parts[l] = grad_parts(n, n->w[l + 1], n->w[l], in.rows);
+        gp->parts[l] = grad_parts(n->prec, n->w[l + 1], n->w[l], in.rows);
         gp->stride[l] = (long)cnt;
-        if (gp->parts[l] > 1) need += cnt * gp->parts[l];
     }
     gp->off[L] = (long)n->nparam;
-    if (need > n->part_cap) {
-        cudaFree(n->part);
-        n->part = nullptr;
-        n->part_cap = 0;
-        MLP_CUDA(cudaMalloc(&n->part, need * sizeof(float)));
-        n->part_cap = need;
-    }
     float* at = n->part;
     float* dcur = n->dbuf0;   // dZ_l
     float* dnext = n->dbuf1;

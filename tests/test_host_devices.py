@@ -221,3 +221,21 @@ def test_no_sweep_kernel_is_first_launched_in_a_capture(fake):
     fake.kd_batch_destroy(b)
     for s in (*sims, big):
         fake.kd_destroy(s)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_training_allocates_nothing_at_a_batch_size_already_seen(fake, precision):
+    """A step at no more rows than an earlier call's makes no allocation (a stream capture, or a
+    device without memory left, allows none), whatever the precision was then."""
+    rc, h = _net(fake, [5, 256, 256, 4])
+    assert rc == 0
+    x = np.zeros(1 << 16, np.float32)
+    p = C.c_void_p(x.ctypes.data)
+    assert fake.kd_mlp_forward(h, p, 1024, p, KD_DEVICE, None) == 0
+    assert fake.kd_mlp_set_precision(h, precision) == 0
+    fake.fake_fail_malloc(0)
+    for batch in (1024, 700, 300, 8):
+        assert _train(fake, h, batch) == 0, batch
+    fake.fake_fail_malloc(-1)
+    fake.kd_mlp_destroy(h)
+    assert fake.fake_bad_frees() == 0
