@@ -308,8 +308,8 @@ int kd_bench_sweep(kd_sim* sim, int32_t kind, int32_t reps);
  * Variant 0 is the default.  kd_autotune times every variant of both sweeps on this
  * simulation's grid (reps back-to-back launches each, graph-replayed, reading the state
  * and writing only scratch: the state is unchanged) with the step's pointwise ops for
- * time step dt, keeps variant 0 unless another is faster by more than 2 %, and applies
- * the choice to this simulation.  The choice is remembered for the process per device,
+ * time step dt, keeps variant 0 unless another is faster by more than 2 %, by itself and
+ * over whole steps, and applies the choice to this simulation.  The choice is remembered for the process per device,
  * grid and field kind, so later simulations of that shape only look it up (flags =
  * KD_TUNE_FORCE times again).  variant_x / variant_y (may be NULL) receive the choice,
  * times_ms (may be NULL, 2 * KD_SWEEP_VARIANTS floats: x then y) the measured ms per

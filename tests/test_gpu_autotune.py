@@ -164,3 +164,30 @@ def test_tuning_is_rejected_during_stream_capture(kd):
         assert e1.value.code == kd.KD_ERR_ARG and e2.value.code == kd.KD_ERR_ARG
         assert sim.sweep_variants == (0, 0)
         assert sim.autotune(wl.dt, reps=2, force=True)["variants"] is not None
+
+
+@pytest.mark.parametrize("nx,ny", [(1024, 128), (512, 256), (256, 256)])
+def test_tuned_runs_are_not_slower_than_the_default(kd, nx, ny):
+    """The fastest sweep by itself need not make the fastest run (it can keep the next one from
+    starting under its tail): what the tuner picks has to hold over whole runs.  Best of ten runs
+    each; they repeat to well below the 3 % allowed."""
+    import time
+
+    import torch
+    wl = W.small(nx, ny, W.GAUSS, units=W.ATOMIC, a0=0.2).with_(precision=1)
+    best = {}
+    for tuned in (False, True):
+        with kd.Sim.from_workload(wl) as sim:
+            sim.init_packet(wl.packet)
+            if tuned:
+                sim.autotune(wl.dt, force=True)
+            sim.step(wl.dt, 400)
+            ts = []
+            for _ in range(10):
+                torch.cuda.synchronize()
+                t = time.perf_counter()
+                sim.step(wl.dt, 400)
+                torch.cuda.synchronize()
+                ts.append(time.perf_counter() - t)
+            best[tuned] = min(ts)
+    assert best[True] <= 1.03 * best[False]
