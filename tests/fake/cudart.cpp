@@ -22,6 +22,7 @@ std::set<void*> live;
 int bad_frees = 0, fail_after = -1, capturing_error = 0, refuse_attr = 0;
 long launches = 0;
 bool capturing = false;
+int instantiated = 0;
 int first_in_capture = 0;                           // kernels first launched inside a capture
 std::set<std::pair<int, const void*>> seen;
 struct Config {
@@ -58,6 +59,7 @@ void fake_capture_query_error(int on) { capturing_error = on; }
 void fake_refuse_attribute(int on) { refuse_attr = on; }
 int fake_set_device(int d) { return cudaSetDevice(d); }
 int fake_last_error() { return last; }
+int fake_instantiated() { return instantiated; }
 int fake_first_in_capture() { return first_in_capture; }
 
 cudaError_t cudaGetDeviceCount(int* n) { *n = kDevices; return cudaSuccess; }
@@ -105,7 +107,7 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* c) {
 }
 cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { capturing = true; return cudaSuccess; }
 cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { capturing = false; *g = (cudaGraph_t)malloc(1); return cudaSuccess; }
-cudaError_t cudaGraphInstantiate(cudaGraphExec_t* x, cudaGraph_t, unsigned long long) { *x = (cudaGraphExec_t)malloc(1); return cudaSuccess; }
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t* x, cudaGraph_t, unsigned long long) { ++instantiated; *x = (cudaGraphExec_t)malloc(1); return cudaSuccess; }
 cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaGraphDestroy(cudaGraph_t g) { free(g); return cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t x) { free(x); return cudaSuccess; }

@@ -239,3 +239,37 @@ def test_training_allocates_nothing_at_a_batch_size_already_seen(fake, precision
     fake.fake_fail_malloc(-1)
     fake.kd_mlp_destroy(h)
     assert fake.fake_bad_frees() == 0
+
+
+def test_runs_of_one_shape_capture_their_steps_once(fake):
+    """Another time, packet or state is no reason to capture the step loop again; other windows,
+    another basis, interval or time step are.  kd_step and kd_batch_step."""
+    from paper_2307_01571_gb300 import kd, workloads as W
+    rc, h, wl = _sim(fake, 64, 128, 1)
+    assert rc == 0
+    b = C.c_void_p()
+    assert fake.kd_batch_create((C.c_void_p * 1)(h), 1, None, C.byref(b)) == 0
+    p = wl.packet
+    buf = (kd.kd_obs * 8)()
+
+    def run(packet, t, batch, dt=wl.dt, every=4):
+        assert fake.kd_init_packet(h, C.byref(kd._fill(kd.kd_packet, packet))) == 0
+        assert fake.kd_set_time(h, C.c_double(t)) == 0
+        before = fake.fake_instantiated()
+        args = (C.c_int64(12), C.c_int64(every), buf, C.c_int64(12 // every), None)
+        rc = fake.kd_batch_step(b, (C.c_double * 1)(dt), *args) if batch else fake.kd_step(h, C.c_double(dt), *args)
+        assert rc == 0
+        return fake.fake_instantiated() - before
+
+    moved = W.Packet(p.p0x, p.p0y, 0.1 * wl.grid.x_max, 0.0, p.sigma_p, -p.spin, p.basis)
+    other_basis = W.Packet(p.p0x, p.p0y, p.r0x, p.r0y, p.sigma_p, p.spin, 1 - p.basis)
+    other_window = W.Packet(0.5 * p.p0x, p.p0y, p.r0x, p.r0y, p.sigma_p, p.spin, p.basis)
+    for batch in (False, True):
+        assert run(p, 0.0, batch) > 0
+        for start, t in ((p, 3.0 * wl.dt), (moved, 0.0), (moved, wl.dt), (p, 0.0)):
+            assert run(start, t, batch) == 0
+        for start, kw in ((other_basis, {}), (other_window, {}), (p, {}), (p, dict(dt=0.5 * wl.dt)), (p, dict(every=6))):
+            assert run(start, 0.0, batch, **kw) > 0
+            assert run(start, wl.dt, batch, **kw) == 0
+    fake.kd_batch_destroy(b)
+    fake.kd_destroy(h)
