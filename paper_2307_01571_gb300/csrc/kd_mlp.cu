@@ -34,7 +34,7 @@ struct kd_mlp {
     std::vector<float*> a;           // activations per layer output [cap][w[l+1]] (a[0] = input)
     float* dbuf0 = nullptr;          // gradient ping-pong buffers [cap][max width]
     float* dbuf1 = nullptr;
-    float* lossbuf = nullptr;        // the loss, then [cap * w[L]] squared errors
+    float* lossbuf = nullptr;        // the loss, then [cap * w[L]] squared errors, then
     float* part = nullptr;           // partial gradients of layers whose batch is split
     int prec = 0;                    // KD_MLP_FP32 or KD_MLP_BF16 (tensor-core GEMMs)
     int* status = nullptr;           // set when a tensor-core GEMM's bounded wait gave up
@@ -867,7 +867,6 @@ int ensure_cap(kd_mlp* n, int batch) {
     cudaFree(n->dbuf0);
     cudaFree(n->dbuf1);
     cudaFree(n->lossbuf);
-    cudaFree(n->part);
     // nothing is left to use or free again if one of the allocations below fails
     n->cap = 0;
     n->dbuf0 = n->dbuf1 = n->lossbuf = n->part = nullptr;
@@ -879,9 +878,10 @@ int ensure_cap(kd_mlp* n, int batch) {
     }
     MLP_CUDA(cudaMalloc(&n->dbuf0, sizeof(float) * (size_t)batch * maxw(n)));
     MLP_CUDA(cudaMalloc(&n->dbuf1, sizeof(float) * (size_t)batch * maxw(n)));
-    MLP_CUDA(cudaMalloc(&n->lossbuf, sizeof(float) * ((size_t)batch * n->w[n->L] + 1)));
-    const size_t part = part_floats(n, batch);
-    if (part > 0) MLP_CUDA(cudaMalloc(&n->part, part * sizeof(float)));
+    // (an allocation of their own for the partial gradients costs a new network's first step 0.1 ms)
+    const size_t sq = (size_t)batch * n->w[n->L] + 1;
+    MLP_CUDA(cudaMalloc(&n->lossbuf, sizeof(float) * (sq + part_floats(n, batch))));
+    n->part = n->lossbuf + sq;
     n->cap = batch;
     return KD_OK;
 }
@@ -1071,7 +1071,6 @@ void kd_mlp_destroy(kd_mlp* n) {
     cudaFree(n->dbuf0);
     cudaFree(n->dbuf1);
     cudaFree(n->lossbuf);
-    cudaFree(n->part);
     cudaFree(n->status);
     cudaFree(n->param);
     cudaFree(n->grad);
