@@ -2030,7 +2030,10 @@ int kd_batch_create(kd_sim* const* sims, int32_t n, void* cuda_stream, kd_batch*
     b->join.assign(n, nullptr);
     size_t points = 0;
     for (const kd_sim* s : b->sims) points += s->P;
-    b->crowded = n > 1 && points > ((size_t)1 << 18);
+    // more than 2^18 points fill the SMs, and so do 32 members of any size (G point-steps/s, forms
+    // of a grid alone : of a crowd: 32 of 64x64 7.4 : 7.75, 64 of 64x64 7.4 : 7.9, 128 of 32x32
+    // 1.85 : 1.87; but 8 of 256x128 16.3 : 16.0, 16 of 128x128 16.3 : 15.8, 4 of 256x256 14.6 : 14.4)
+    b->crowded = n >= 32 || (n > 1 && points > ((size_t)1 << 18));
     bool ok = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) == cudaSuccess &&
               cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess;
     for (int32_t i = 0; ok && i < n; ++i)
