@@ -827,9 +827,10 @@ template <typename T, int LOGN, int AXIS, int SHAPE, int V> struct Sweep {
             if constexpr (sizeof(T) == 4 && Cf::LOGE == 2) {
                 // the expressions below with every fusion written out: the radix-4 forms
                 // differ in components per thread and stand in for one another (a crowded
-                // batch swaps them, a persistent batch runs wide rows for all of them)
-                e[2 * q] = mk<C>(__fadd_rn(u.x, fmaf(c1, u.x, fmaf(sy, l.x, -sax * l.y))), __fadd_rn(u.y, fmaf(c1, u.y, fmaf(sy, l.y, sax * l.x))));
-                e[2 * q + 1] = mk<C>(__fadd_rn(l.x, fmaf(c1, l.x, fmaf(-sy, u.x, -sax * u.y))), __fadd_rn(l.y, fmaf(c1, l.y, fmaf(-sy, u.y, sax * u.x))));
+                // batch swaps them, a persistent batch runs wide rows for all of them).  The c1
+                // product first: last, 200 steps of 128x128 took 1319 us instead of 1309
+                e[2 * q] = mk<C>(__fadd_rn(u.x, fmaf(sy, l.x, fmaf(-sax, l.y, c1 * u.x))), __fadd_rn(u.y, fmaf(sy, l.y, fmaf(sax, l.x, c1 * u.y))));
+                e[2 * q + 1] = mk<C>(__fadd_rn(l.x, fmaf(-sy, u.x, fmaf(-sax, u.y, c1 * l.x))), __fadd_rn(l.y, fmaf(-sy, u.y, fmaf(sax, u.x, c1 * l.y))));
                 continue;
             }
             const C q1 = mk<C>(sy, sax);
