@@ -142,8 +142,9 @@ __host__ __device__ constexpr int sweep_nc(int axis, int v);
 //   wide, tall wide: what members of a batch that fills the SMs run in the place of small and of
 //     the long columns' forms: both pairs per thread, rows in CTAs of 256 threads, columns in
 //     tiles of 256 threads (two columns at 512 points, where four would take 512).
-// Radix-4 forms, and tall with its stand-in, round alike: their pointwise steps have every
-// fusion written out, so that components per thread do not change a bit.
+// All radix-4 rows round alike, and so do small and wide columns, and tall wide ones with tall
+// and, from 1024 points, variant 3: their pointwise steps have every fusion written out, so that
+// components per thread do not change a bit.
 constexpr int kFormSmall = 4, kFormLarge = 5, kFormWide = 6, kFormTall = 7, kFormTallWide = 8, kNumSweepForms = 9;
 __host__ __device__ constexpr SweepVariant sweep_form(int axis, int form) {
     if (form < kNumSweepVariants) return sweep_variant(axis, form);
@@ -157,7 +158,7 @@ __host__ __device__ constexpr SweepVariant sweep_form(int axis, int form) {
 // (axes end at 4096 points)
 __host__ __device__ constexpr bool sweep_form_holds(int axis, int form, int logn) {
     return form <= 1               ? (axis == AXIS_X ? logn >= 7 : logn >= 6 && logn <= 9)
-           : form == kFormSmall      ? logn <= (axis == AXIS_X ? 11 : 10)
+           : form == kFormSmall    ? logn <= (axis == AXIS_X ? 11 : 10)
            : form == kFormWide     ? logn <= (axis == AXIS_X ? 11 : 9)
            : form == kFormTall     ? axis == AXIS_Y && (logn == 10 || logn == 11)
            : form == kFormTallWide ? axis == AXIS_Y && logn >= 10
@@ -178,9 +179,10 @@ __host__ __device__ constexpr bool sweep_form_holds(int axis, int form, int logn
 //     few rows for it (a sweep 11.1 : 16.7);
 //   x 2048 points at 2^17: variant 0 (13.1 with small rows, 11.9);
 //   y small up to 2^16 points (2^15 at 512, tall for few columns of 1024 and more), radix-4
-//     tiles of both pairs (wide) at 2^17 up to 256 points; one pair per CTA for few long columns (128x512 12.1 : 10.3, 256x512 15.3 : 12.3,
-//     128x1024 20.9 : 15.2, 64x2048 23.5 : 16.3, 256x1024 24.1 : 17.3 with small rows); large
-//     beyond (1024x1024 56.5 : 55.0, 2048x1024 125.5 : 118.2, 4096x2048 589 : 562).
+//     tiles of both pairs (wide) at 2^17 up to 256 points; one pair per CTA (variant 3) for few
+//     long columns (128x512 12.1 : 10.3, 256x512 15.3 : 12.3, 128x1024 20.9 : 15.2, 64x2048
+//     23.5 : 16.3, 256x1024 24.1 : 17.3 with small rows); large beyond (1024x1024 56.5 : 55.0,
+//     2048x1024 125.5 : 118.2, 4096x2048 589 : 562).
 // crowded: other simulations run beside this one and fill the SMs (a batch).  The narrow tiles
 // that spread one small grid over the SMs then only cost: the field, the twiddles and the index
 // work of each pair of components, and memory transactions.  The wide forms take their place,
