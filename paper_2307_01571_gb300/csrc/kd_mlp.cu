@@ -34,8 +34,9 @@ struct kd_mlp {
     std::vector<float*> a;           // activations per layer output [cap][w[l+1]] (a[0] = input)
     float* dbuf0 = nullptr;          // gradient ping-pong buffers [cap][max width]
     float* dbuf1 = nullptr;
-    float* lossbuf = nullptr;        // the loss, then [cap * w[L]] squared errors, then
+    float* lossbuf = nullptr;        // the loss, then [cap * w[L]] squared errors
     float* part = nullptr;           // partial gradients of layers whose batch is split
+    size_t part_cap = 0;             // its floats
     int prec = 0;                    // KD_MLP_FP32 or KD_MLP_BF16 (tensor-core GEMMs)
     int* status = nullptr;           // set when a tensor-core GEMM's bounded wait gave up
 };
@@ -845,19 +846,22 @@ int grad_parts(int precision, int fo, int fi, int rows) {
     return (int)(p < 1 ? 1 : p > 8 ? 8 : p);
 }
 
-// Floats of the partial gradients of a batch, whichever the precision (more rows never take
-// fewer parts)
-size_t part_floats(const kd_mlp* n, int rows) {
-    size_t most = 0;
-    for (int prec : {KD_MLP_FP32, KD_MLP_BF16}) {
-        size_t need = 0;
-        for (int l = 0; l < n->L; ++l) {
-            const int parts = grad_parts(prec, n->w[l + 1], n->w[l], rows);
-            if (parts > 1) need += ((size_t)n->w[l + 1] * n->w[l] + n->w[l + 1]) * parts;
-        }
-        most = need > most ? need : most;
+// Room for the partial gradients of any batch up to `rows` (more rows never take fewer parts) at
+// a precision.  Made with the batch buffers and at a change of precision, so that a step at a
+// batch size already seen allocates nothing (it may be inside a stream capture).
+int ensure_part(kd_mlp* n, int precision, int rows) {
+    size_t need = 0;
+    for (int l = 0; l < n->L; ++l) {
+        const int parts = grad_parts(precision, n->w[l + 1], n->w[l], rows);
+        if (parts > 1) need += ((size_t)n->w[l + 1] * n->w[l] + n->w[l + 1]) * parts;
     }
-    return most;
+    if (need <= n->part_cap) return KD_OK;
+    cudaFree(n->part);
+    n->part = nullptr;
+    n->part_cap = 0;
+    MLP_CUDA(cudaMalloc(&n->part, need * sizeof(float)));
+    n->part_cap = need;
+    return KD_OK;
 }
 
 int ensure_cap(kd_mlp* n, int batch) {
@@ -869,7 +873,7 @@ int ensure_cap(kd_mlp* n, int batch) {
     cudaFree(n->lossbuf);
     // nothing is left to use or free again if one of the allocations below fails
     n->cap = 0;
-    n->dbuf0 = n->dbuf1 = n->lossbuf = n->part = nullptr;
+    n->dbuf0 = n->dbuf1 = n->lossbuf = nullptr;
     n->z.assign(n->L, nullptr);
     n->a.assign(n->L + 1, nullptr);
     for (int l = 0; l < n->L; ++l) {
@@ -878,10 +882,9 @@ int ensure_cap(kd_mlp* n, int batch) {
     }
     MLP_CUDA(cudaMalloc(&n->dbuf0, sizeof(float) * (size_t)batch * maxw(n)));
     MLP_CUDA(cudaMalloc(&n->dbuf1, sizeof(float) * (size_t)batch * maxw(n)));
-    // (an allocation of their own for the partial gradients costs a new network's first step 0.1 ms)
-    const size_t sq = (size_t)batch * n->w[n->L] + 1;
-    MLP_CUDA(cudaMalloc(&n->lossbuf, sizeof(float) * (sq + part_floats(n, batch))));
-    n->part = n->lossbuf + sq;
+    MLP_CUDA(cudaMalloc(&n->lossbuf, sizeof(float) * ((size_t)batch * n->w[n->L] + 1)));
+    const int rc = ensure_part(n, n->prec, batch);
+    if (rc) return rc;
     n->cap = batch;
     return KD_OK;
 }
@@ -1071,6 +1074,7 @@ void kd_mlp_destroy(kd_mlp* n) {
     cudaFree(n->dbuf0);
     cudaFree(n->dbuf1);
     cudaFree(n->lossbuf);
+    cudaFree(n->part);
     cudaFree(n->status);
     cudaFree(n->param);
     cudaFree(n->grad);
@@ -1112,6 +1116,11 @@ int kd_mlp_set_precision(kd_mlp* n, int32_t precision) {
     if (precision != n->prec) {
         MLP_CUDA(cudaSetDevice(n->device));
         MLP_CUDA(allow_smem(precision));
+        const int rc = n->cap > 0 ? ensure_part(n, precision, n->cap) : KD_OK;
+        if (rc) {   // the buffer for the present precision may be gone: made again with the others
+            n->cap = 0;
+            return rc;
+        }
     }
     n->prec = precision;
     return KD_OK;

@@ -237,6 +237,12 @@ def test_training_allocates_nothing_at_a_batch_size_already_seen(fake, precision
     for batch in (1024, 700, 300, 8):
         assert _train(fake, h, batch) == 0, batch
     fake.fake_fail_malloc(-1)
+    # a change of precision that finds no memory leaves a network that still trains
+    fake.fake_fail_malloc(0)
+    fake.kd_mlp_set_precision(h, 1 - precision)
+    fake.fake_fail_malloc(-1)
+    for batch in (8, 1024):
+        assert _train(fake, h, batch) == 0
     fake.kd_mlp_destroy(h)
     assert fake.fake_bad_frees() == 0
 
