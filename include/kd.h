@@ -276,8 +276,8 @@ int kd_mlp_train_step(kd_mlp* net, const float* x, const float* targets, int32_t
                       float lr, float* loss_dev, void* cuda_stream);
 /* The same training step on a minibatch selected on the device: rows idx[0 .. batch) of
  * x_all [n_all][widths[0]] and targets_all [n_all][widths[nlayers]] (device pointers;
- * idx device int32, indices outside [0, n_all) select rows of zeros) are gathered by the
- * library's own kernel into its staging buffers. */
+ * idx device int32, indices outside [0, n_all) select rows of zeros), gathered where the
+ * products load them: the arrays stay unchanged until the step has run. */
 int kd_mlp_train_step_gather(kd_mlp* net, const float* x_all, const float* targets_all,
                              int64_t n_all, const int32_t* idx, int32_t batch, float lr,
                              float* loss_dev, void* cuda_stream);
@@ -316,14 +316,16 @@ int kd_bench_sweep(kd_sim* sim, int32_t kind, int32_t reps);
  * launch (the recorded ones when the choice was looked up; -1 for FP64).  FP64
  * simulations have one variant (0).  What variants 0 and 1 launch follows the grid's size
  * (small grids run radix-4 stages in small tiles, long rows both pairs per thread, large
- * grids radix-16 column stages); 2 and 3 are fixed shapes.  Synchronises the simulation's stream: KD_ERR_ARG
- * while that stream is being captured (kd_set_sweep_variants likewise, when it changes the
- * variants).  Variants 0 and 1 differ at most in threads per CTA and give
- * bitwise identical results; the radix-4 schedule (2) and the components-per-CTA change
- * (3) round differently in the last bits (every variant meets the same accuracy).  A
- * simulation's results are reproducible for fixed variants.  kd_set_sweep_variants selects variants directly
- * (KD_ERR_ARG out of range), kd_get_sweep_variants reads them back.  The variants are
- * not part of a kd_get_state checkpoint. */
+ * grids radix-16 column stages) and, in a batch whose members fill the SMs, that (wide tiles
+ * of the same arithmetic, bit for bit); 2 and 3 are fixed shapes.  Synchronises the
+ * simulation's stream: KD_ERR_ARG while that stream is being captured
+ * (kd_set_sweep_variants likewise, when it changes the variants).  Variants 0 and 1 differ at
+ * most in threads per CTA and give bitwise identical results; the radix-4 schedule (2) and
+ * the components-per-CTA change (3) round differently in the last bits (every variant meets
+ * the same accuracy).  A simulation's results are reproducible for fixed variants.
+ * kd_set_sweep_variants selects variants directly (KD_ERR_ARG out of range),
+ * kd_get_sweep_variants reads them back.  The variants are not part of a kd_get_state
+ * checkpoint. */
 #define KD_SWEEP_VARIANTS 4
 #define KD_TUNE_FORCE 1
 int kd_autotune(kd_sim* sim, double dt, int32_t reps, int32_t flags, int32_t* variant_x,

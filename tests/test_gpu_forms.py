@@ -124,7 +124,7 @@ def test_runs_from_new_states_and_times_replay_the_same_steps(kd, prec):
 
 
 @pytest.mark.parametrize("nx,ny", [(4, 1024), (32, 1024), (16, 2048), (32, 2048), (64, 2048), (16, 4096),
-                                   (2048, 32), (1024, 64), (1024, 128), (1024, 256)])
+                                   (2048, 32), (1024, 64), (1024, 128), (1024, 256), (256, 4096)])
 def test_more_default_forms_match_oracle(kd, nx, ny):
     """Tall columns on both sides of their line, and 1024-point rows in each of their forms."""
     test_default_form_matches_oracle(kd, nx, ny)
